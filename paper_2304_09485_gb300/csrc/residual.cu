@@ -19,6 +19,7 @@
 //               summation order is fixed (deterministic results).
 // Arrays are component-major with the cell or face index fastest, so
 // consecutive threads touch consecutive addresses.
+#include <algorithm>
 #include <cmath>
 #include "hgks_internal.h"
 
@@ -59,9 +60,9 @@ __device__ __forceinline__ void rot_out(const double *T, const double *in, doubl
   for (int d = 0; d < 3; d++) out[1 + d] = T[d] * in[1] + T[3 + d] * in[2] + T[6 + d] * in[3];
 }
 
-// Euler eigen-system along x of a face-frame state: scalars from which the
-// rows of R^{-1} (left) and columns of R (right) are formed.
-struct Eig { double u, v, w, a, H, q2, b1, b2, ia; };
+// Euler eigen-system along x of a face-frame state: scalars of which R (right_apply)
+// and R^{-1} (k_recon's projection) are made.
+struct Eig { double u, v, w, a, H, q2, ia; };
 __device__ __forceinline__ Eig eig_of(const double *Q, double gamma) {
   Eig e;
   double ir = 1.0 / Q[0];
@@ -72,19 +73,7 @@ __device__ __forceinline__ Eig eig_of(const double *Q, double gamma) {
   e.ia = rsqrt(a2);
   e.a = a2 * e.ia;
   e.H = (Q[4] + p) * ir;
-  e.b1 = (gamma - 1.0) * e.ia * e.ia;
-  e.b2 = 0.5 * e.b1 * e.q2;
   return e;
-}
-// row c of R^{-1}
-__device__ __forceinline__ void left_row(const Eig &e, int c, double *l) {
-  switch (c) {
-    case 0: l[0] = 0.5 * (e.b2 + e.u * e.ia); l[1] = -0.5 * (e.b1 * e.u + e.ia); l[2] = -0.5 * e.b1 * e.v; l[3] = -0.5 * e.b1 * e.w; l[4] = 0.5 * e.b1; break;
-    case 1: l[0] = 1.0 - e.b2; l[1] = e.b1 * e.u; l[2] = e.b1 * e.v; l[3] = e.b1 * e.w; l[4] = -e.b1; break;
-    case 2: l[0] = -e.v; l[1] = 0.0; l[2] = 1.0; l[3] = 0.0; l[4] = 0.0; break;
-    case 3: l[0] = -e.w; l[1] = 0.0; l[2] = 0.0; l[3] = 1.0; l[4] = 0.0; break;
-    default: l[0] = 0.5 * (e.b2 - e.u * e.ia); l[1] = -0.5 * (e.b1 * e.u - e.ia); l[2] = -0.5 * e.b1 * e.v; l[3] = -0.5 * e.b1 * e.w; l[4] = 0.5 * e.b1;
-  }
 }
 // out = R q (characteristic -> conservative, face frame)
 __device__ __forceinline__ void right_apply(const Eig &e, const double *q, double *out) {
@@ -197,10 +186,29 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 // ------------------------------------------------------------------------
 // 2. reconstruction at the Gauss points of one face, one side
 // ------------------------------------------------------------------------
+// Bound by the FP64 pipe (2 DFMA per SM and clock); all choices below save FP64 work.
+// The thread first projects its cell's coefficients (9 of P0, 3 of every P_m) and average
+// into characteristic variables, each vector once, and keeps them in its own column of
+// shared memory; the loop over the five variables then works from there. R^{-1} q of a
+// conservative vector q = (q0, m, q4) about the projection state (u, sound speed a):
+//   P = (gamma - 1) / (2 a^2) (|u|^2/2 q0 - u . m + q4),   D = (n . m - u_n q0) / (2 a),
+//   (P - D, q0 - 2 P, t1 . m - u_t1 q0, t2 . m - u_t2 q0, P + D): 20 operations against 25
+// for five dense rows. The nonlinear weights take one division: with d_k = beta_k + eps,
+// D = prod d_k, R_k = D / d_k (prefix and suffix products) and sum of the linear weights 1,
+//   kap_0 = (D + tz R_0) / den,  kap_m = gm tz (R_m - R_0) / den,
+//   den = D + tz (g0 R_0 + gm sum R_m).
+// Keeping the projection in shared memory (110 doubles a thread on tetrahedra, 170 on
+// hexahedra) instead of projecting per variable: 28.5 -> 24.8 ms for 9.4M (cell, face) pairs
+// (2,359,296 tetrahedra), 1.24 -> 1.05 ms for 35,937 hexahedra; no spills (604 bytes before).
+// Blocks: any shape up to 256 threads fits on tetrahedra; on hexahedra two blocks of 64
+// fit an SM (85 KB each), one of 128, none of 256.
+constexpr int kReconMax = 256, kReconHex = 64;
+template <class S> constexpr int recon_rows() { return 5 * (10 + 3 * ShapeOf<S>::NSUB); }
 template <bool BATCH, class S>
-__global__ void __launch_bounds__(256) k_recon(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
-                                               const double *__restrict__ coef, double *__restrict__ wface) {
-  constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB;
+__global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
+                                                     const double *__restrict__ coef, double *__restrict__ wface) {
+  constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB, NV = 9 + 3 * NSUB;
+  extern __shared__ double proj[];                      // [5][NV + 1][blockDim.x]: column of this thread
   const int N = m.N, F = m.F;
   const int NL = BATCH ? m.NL : N;
   // block b covers local face (b mod NF) of cell range b / NF: the blocks of a
@@ -211,18 +219,57 @@ __global__ void __launch_bounds__(256) k_recon(DevMesh m, hgks_params Pv, const 
   const hgks_params &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
   const int cf = m.cface[(size_t)slot * N + i];
   const int f = cf >> 1, side = cf & 1;
+  const int bd = blockDim.x;
+  double *my = proj + threadIdx.x;
   double T[9];
 #pragma unroll
   for (int k = 0; k < 9; k++) T[k] = m.fT[(size_t)k * F + f];
-  const int L = m.fl[f], R = m.fr[f];
-  double Qi[5], Qs[5], Qsl[5];
+  {
+    const int L = m.fl[f], R = m.fr[f];
+    double Qi[5], Qs[5], Qsl[5];
 #pragma unroll
-  for (int c = 0; c < 5; c++) {
-    Qi[c] = Q[(size_t)c * N + i];
-    Qs[c] = R >= 0 ? 0.5 * (Q[(size_t)c * N + L] + Q[(size_t)c * N + R]) : Qi[c];
+    for (int c = 0; c < 5; c++) {
+      Qi[c] = Q[(size_t)c * N + i];
+      Qs[c] = R >= 0 ? 0.5 * (Q[(size_t)c * N + L] + Q[(size_t)c * N + R]) : Qi[c];
+    }
+    if (P.characteristic) {
+      rot_in(T, Qs, Qsl);
+      const Eig e = eig_of(Qsl, P.gamma);
+      const double hb = 0.5 * (P.gamma - 1.0) * e.ia * e.ia, hi = 0.5 * e.ia;
+      double pm[3], dm[3];                              // P = p0 q0 + pm . m + hb q4, D = d0 q0 + dm . m
+      const double p0 = 0.5 * hb * e.q2, d0 = -hi * e.u;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        pm[k] = -hb * (T[k] * e.u + T[3 + k] * e.v + T[6 + k] * e.w);
+        dm[k] = hi * T[k];
+      }
+      auto project = [&](const double *q, double *o) {  // o: row stride (NV + 1) bd between the variables
+        const size_t rs = (size_t)(NV + 1) * bd;
+        const double Pq = fma(p0, q[0], fma(pm[0], q[1], fma(pm[1], q[2], fma(pm[2], q[3], hb * q[4]))));
+        const double Dq = fma(d0, q[0], fma(dm[0], q[1], fma(dm[1], q[2], dm[2] * q[3])));
+        o[0] = Pq - Dq;
+        o[rs] = fma(-2.0, Pq, q[0]);
+        o[2 * rs] = fma(-e.v, q[0], fma(T[3], q[1], fma(T[4], q[2], T[5] * q[3])));
+        o[3 * rs] = fma(-e.w, q[0], fma(T[6], q[1], fma(T[7], q[2], T[8] * q[3])));
+        o[4 * rs] = Pq + Dq;
+      };
+#pragma unroll
+      for (int d = 0; d < NV; d++) {
+        double q[5];
+#pragma unroll
+        for (int k = 0; k < 5; k++) q[k] = coef[(size_t)(d * 5 + k) * N + i];
+        project(q, my + d * bd);
+      }
+      project(Qi, my + NV * bd);
+    } else {                                            // conservative variables: the coefficients themselves
+#pragma unroll 1
+      for (int d = 0; d < NV; d++)
+#pragma unroll
+        for (int k = 0; k < 5; k++) my[(size_t)(k * (NV + 1) + d) * bd] = coef[(size_t)(d * 5 + k) * N + i];
+#pragma unroll
+      for (int k = 0; k < 5; k++) my[(size_t)(k * (NV + 1) + NV) * bd] = Qi[k];
+    }
   }
-  rot_in(T, Qs, Qsl);
-  const Eig e = eig_of(Qsl, P.gamma);
   const double ih = 1.0 / m.h[i];
   double m2[6], xg[3 * NG];
 #pragma unroll
@@ -230,141 +277,67 @@ __global__ void __launch_bounds__(256) k_recon(DevMesh m, hgks_params Pv, const 
 #pragma unroll
   for (int k = 0; k < 3 * NG; k++) xg[k] = m.xg[(size_t)(slot * 3 * NG + k) * N + i];
   // weights of the sub-stencils (compact: one per face)
-  unsigned valid = P.scheme == HGKS_WENO ? m.subvalid[i] : (1u << NF) - 1u;
+  const unsigned valid = P.scheme == HGKS_WENO ? m.subvalid[i] : (1u << NF) - 1u;
   const int M = __popc(valid);
   const double gm = P.lin_weight, g0 = M ? 1.0 - gm * M : 1.0;
-  const double ig0 = 1.0 / g0, iM = M ? 1.0 / M : 0.0;
-  double Th[9];                                         // face frame rows / h: scaled derivatives
+  const double iM = M ? 1.0 / M : 0.0;
 #pragma unroll
-  for (int k = 0; k < 9; k++) Th[k] = ih * T[k];
+  for (int k = 0; k < 9; k++) T[k] *= ih;               // face frame rows / h: scaled derivatives
   double *out = wface + (size_t)side * NG * kFaceState * F + f;
+#pragma unroll 1
   for (int c = 0; c < 5; c++) {
-    double mr[5];
-    if (P.characteristic) {
-      double l[5];
-      left_row(e, c, l);
-      mr[0] = l[0]; mr[4] = l[4];
+    const double *pc = my + (size_t)c * (NV + 1) * bd;
+    double ac[9];
 #pragma unroll
-      for (int j = 0; j < 3; j++) mr[1 + j] = l[1] * T[j] + l[2] * T[3 + j] + l[3] * T[6 + j];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 5; k++) mr[k] = k == c ? 1.0 : 0.0;
-    }
-    double q0 = 0.0;
-#pragma unroll
-    for (int k = 0; k < 5; k++) q0 = fma(mr[k], Qi[k], q0);
-    // Sub-stencil coefficients in characteristic variables: tetrahedra (4 sub-
-    // stencils) keep all of them in registers; with 8 the arrays would go to local
-    // memory, so hexahedra form them where they are used (twice) from the
-    // coefficients, which the thread has just read (L1).
-    constexpr bool kHold = NSUB <= 4;
-    double ac[9], bc[kHold ? 3 * NSUB : 1];
-#pragma unroll
-    for (int d = 0; d < 9; d++) {
-      double s = 0.0;
-#pragma unroll
-      for (int k = 0; k < 5; k++) s = fma(mr[k], coef[(size_t)(d * 5 + k) * N + i], s);
-      ac[d] = s;
-    }
-    if constexpr (kHold) {
-#pragma unroll
-      for (int d = 0; d < 3 * NSUB; d++) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < 5; k++) s = fma(mr[k], coef[(size_t)(kCoefA + d * 5 + k) * N + i], s);
-        bc[d] = s;
-      }
-    }
-    auto sub_coef = [&](int mm, double *b3) {
-      if constexpr (kHold) {
-#pragma unroll
-        for (int j = 0; j < 3; j++) b3[j] = bc[3 * mm + j];
-      } else {
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-          double s = 0.0;
-#pragma unroll
-          for (int k = 0; k < 5; k++) s = fma(mr[k], coef[(size_t)(kCoefA + (3 * mm + j) * 5 + k) * N + i], s);
-          b3[j] = s;
-        }
-      }
-    };
-    // smoothness indicators in the scaled frame: beta_0 = avg |grad P0|^2 + sum of squared second derivatives
-    const double H00 = 2.0 * ac[3], H11 = 2.0 * ac[4], H22 = 2.0 * ac[5], H01 = ac[6], H02 = ac[7], H12 = ac[8];
-    // avg |grad P0|^2 = |a|^2 + tr(M2 H^2) (M2: second moments, H symmetric)
-    const double s00 = H00 * H00, s11 = H11 * H11, s22 = H22 * H22, s01 = H01 * H01, s02 = H02 * H02, s12 = H12 * H12;
-    const double S00 = s00 + s01 + s02, S11 = s01 + s11 + s12, S22 = s02 + s12 + s22;
-    const double S01 = fma(H00, H01, fma(H01, H11, H02 * H12));
-    const double S02 = fma(H00, H02, fma(H01, H12, H02 * H22));
-    const double S12 = fma(H01, H02, fma(H11, H12, H12 * H22));
-    const double trMH2 = fma(m2[0], S00, fma(m2[1], S11, m2[2] * S22)) +
-                         2.0 * fma(m2[3], S01, fma(m2[4], S02, m2[5] * S12));
-    const double beta0 = fma(ac[0], ac[0], fma(ac[1], ac[1], ac[2] * ac[2])) + trMH2 +
-                         ((s00 + s11 + s22) + (s01 + s02 + s12));
-    double kap0, kap[NSUB];
+    for (int d = 0; d < 9; d++) ac[d] = pc[d * bd];
+    const double q0 = pc[NV * bd];
+    // combined polynomial: Q = kap0 P0 + sum kap_m P_m (kap0 + sum kap_m = 1)
+    double kap0 = 1.0, lin[3];
     if (P.weights == HGKS_LINEAR || M == 0) {
-      kap0 = 1.0;
 #pragma unroll
-      for (int mm = 0; mm < NSUB; mm++) kap[mm] = 0.0;
+      for (int j = 0; j < 3; j++) lin[j] = ac[j];
     } else {
-      double beta[NSUB], tz = 0.0;
+      // smoothness indicators in the scaled frame: beta_0 = avg |grad P0|^2 + sum of squared second derivatives
+      const double H00 = 2.0 * ac[3], H11 = 2.0 * ac[4], H22 = 2.0 * ac[5], H01 = ac[6], H02 = ac[7], H12 = ac[8];
+      // avg |grad P0|^2 = |a|^2 + tr(M2 H^2) (M2: second moments, H symmetric)
+      const double s00 = H00 * H00, s11 = H11 * H11, s22 = H22 * H22;
+      const double S01 = fma(H00, H01, fma(H01, H11, H02 * H12));
+      const double S02 = fma(H00, H02, fma(H01, H12, H02 * H22));
+      const double S12 = fma(H01, H02, fma(H11, H12, H12 * H22));
+      const double s01 = H01 * H01, s02 = H02 * H02, s12 = H12 * H12, so = s01 + s02 + s12, sd = s00 + s11 + s22;
+      const double trd = fma(m2[0], s00 + (s01 + s02), fma(m2[1], s11 + (s01 + s12), m2[2] * (s22 + (s02 + s12))));
+      const double tro = fma(m2[3], S01, fma(m2[4], S02, m2[5] * S12));
+      const double beta0 = fma(ac[0], ac[0], fma(ac[1], ac[1], fma(ac[2], ac[2], fma(2.0, tro, trd) + (sd + so))));
+      double dm[NSUB], tz = 0.0;
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {
-        double b3[3];
-        sub_coef(mm, b3);
-        beta[mm] = b3[0] * b3[0] + b3[1] * b3[1] + b3[2] * b3[2];
-        if (valid >> mm & 1) tz += fabs(beta0 - beta[mm]);
+        const double b0 = pc[(9 + 3 * mm) * bd], b1 = pc[(10 + 3 * mm) * bd], b2 = pc[(11 + 3 * mm) * bd];
+        const double beta = fma(b0, b0, fma(b1, b1, b2 * b2));
+        if (valid >> mm & 1) tz += fabs(beta0 - beta);
+        dm[mm] = (valid >> mm & 1) ? beta + P.weno_eps : 1.0;
       }
       tz *= iM;
-      // 1 / (beta + eps) of all stencils from one division (prefix products
-      // pre[k] = d0 dm[0] ... dm[k-1], then back through them)
-      const double d0 = beta0 + P.weno_eps;
-      double dm[NSUB], pre[NSUB + 1];
+      double R[NSUB], pre = beta0 + P.weno_eps, R0 = 1.0, sum = 0.0;
 #pragma unroll
-      for (int mm = 0; mm < NSUB; mm++) dm[mm] = (valid >> mm & 1) ? beta[mm] + P.weno_eps : 1.0;
-      pre[0] = d0;
-#pragma unroll
-      for (int mm = 0; mm < NSUB; mm++) pre[mm + 1] = pre[mm] * dm[mm];
-      double inv = 1.0 / pre[NSUB], r[NSUB];
-#pragma unroll
-      for (int mm = NSUB - 1; mm >= 0; mm--) {
-        r[mm] = inv * pre[mm];
-        inv *= dm[mm];
+      for (int mm = 0; mm < NSUB; mm++) {               // R[mm] = d0 dm[0] ... dm[mm - 1]
+        R[mm] = pre;
+        pre *= dm[mm];
       }
-      const double r0 = inv;
-      double w0 = g0 * fma(tz, r0, 1.0), w[NSUB], sum = w0;
 #pragma unroll
-      for (int mm = 0; mm < NSUB; mm++) {
-        w[mm] = (valid >> mm & 1) ? gm * fma(tz, r[mm], 1.0) : 0.0;
-        sum += w[mm];
+      for (int mm = NSUB - 1; mm >= 0; mm--) {          // times dm[mm + 1] ... dm[NSUB - 1]
+        R[mm] *= R0;
+        R0 *= dm[mm];
+        if (valid >> mm & 1) sum += R[mm];
       }
-      double is = 1.0 / sum;
-      double wb0 = w0 * is;
-      kap0 = wb0 * ig0;
-#pragma unroll
-      for (int mm = 0; mm < NSUB; mm++) kap[mm] = (valid >> mm & 1) ? w[mm] * is - wb0 * gm * ig0 : 0.0;
-    }
-    // combined polynomial: Q = kap0 P0 + sum kap_m P_m (kap0 + sum kap_m = 1)
-    double lin[3];
-    if constexpr (kHold) {
-#pragma unroll
-      for (int j = 0; j < 3; j++) {
-        double s = kap0 * ac[j];
-#pragma unroll
-        for (int mm = 0; mm < NSUB; mm++) s = fma(kap[mm], bc[3 * mm + j], s);
-        lin[j] = s;
-      }
-    } else {
+      const double inv = 1.0 / fma(tz, fma(g0, R0, gm * sum), pre), h = gm * tz * inv;
+      kap0 = inv * fma(tz, R0, pre);
 #pragma unroll
       for (int j = 0; j < 3; j++) lin[j] = kap0 * ac[j];
-      if (kap0 != 1.0 || P.weights != HGKS_LINEAR) {
 #pragma unroll
-        for (int mm = 0; mm < NSUB; mm++) {
-          double b3[3];
-          sub_coef(mm, b3);
+      for (int mm = 0; mm < NSUB; mm++) {
+        const double k = (valid >> mm & 1) ? h * (R[mm] - R0) : 0.0;
 #pragma unroll
-          for (int j = 0; j < 3; j++) lin[j] = fma(kap[mm], b3[j], lin[j]);
-        }
+        for (int j = 0; j < 3; j++) lin[j] = fma(k, pc[(9 + 3 * mm + j) * bd], lin[j]);
       }
     }
     double qd[6];
@@ -386,7 +359,7 @@ __global__ void __launch_bounds__(256) k_recon(DevMesh m, hgks_params Pv, const 
       double *o = out + (size_t)g * kFaceState * F;
       o[(size_t)c * F] = val;
 #pragma unroll
-      for (int k = 0; k < 3; k++) o[(size_t)(5 + 5 * k + c) * F] = Th[3 * k] * gx + Th[3 * k + 1] * gy + Th[3 * k + 2] * gz;
+      for (int k = 0; k < 3; k++) o[(size_t)(5 + 5 * k + c) * F] = T[3 * k] * gx + T[3 * k + 1] * gy + T[3 * k + 2] * gz;
     }
   }
 }
@@ -958,7 +931,10 @@ void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &p, const 
   else k_coef_hweno<BATCH, S><<<gc, kBlock, 0, st>>>(m, Q, G, s.coef);
   HGKS_PROF_END(K_COEF, st);
   HGKS_PROF_BEGIN(K_RECON, st);
-  k_recon<BATCH, S><<<S::NF * grid_for(NL, s.blk_recon), s.blk_recon, 0, st>>>(m, p, Q, s.coef, s.wface);
+  const int br = std::min(s.blk_recon, S::NF == 4 ? kReconMax : kReconHex);
+  const size_t shm = sizeof(double) * recon_rows<S>() * br;
+  cudaFuncSetAttribute(k_recon<BATCH, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  k_recon<BATCH, S><<<S::NF * grid_for(NL, br), br, shm, st>>>(m, p, Q, s.coef, s.wface);
   HGKS_PROF_END(K_RECON, st);
   HGKS_PROF_BEGIN(K_FLUX, st);
   const unsigned gf = S::NG * grid_for(FL, s.blk_flux);
