@@ -5,7 +5,7 @@
 //    neighbours sit close in memory and a warp's gathers hit few cache lines;
 //  * faces are matched by sorted vertex lists, then tagged boundary faces,
 //    then periodic pairs (translation of the face centroid by a given shift);
-//    faces are numbered by (left cell, local face) with left = lower cell;
+//    faces are numbered by (left cell, local face) with left = lower cell, boundary faces last;
 //  * stencils: non-compact big stencil = face neighbours and their neighbours
 //    (more rings only while fewer than 12 cells); sub-stencils (Sec. 3.1):
 //    tetrahedron, sub-stencil m = three face neighbours plus the neighbours of
@@ -369,7 +369,12 @@ hgks_status build_host_mesh(const double *xyz, int64_t nv, const int64_t *cells,
       if (!found) { err = "unmatched face without a boundary tag"; return HGKS_ERR_MESH; }
     }
   }
-  std::sort(faces.begin(), faces.end(), [](const Face &a, const Face &b) { return a.L != b.L ? a.L < b.L : a.Ls < b.Ls; });
+  // interior faces first, boundary faces behind them grouped by tag (their flux takes
+  // another path than an interior face's), each group by (left cell, local face)
+  std::sort(faces.begin(), faces.end(), [](const Face &a, const Face &b) {
+    const int ta = a.R < 0 ? a.tag : 0, tb = b.R < 0 ? b.tag : 0;
+    return ta != tb ? ta < tb : a.L != b.L ? a.L < b.L : a.Ls < b.Ls;
+  });
   const int F = (int)faces.size();
   hm.F = F;
   hm.fl.resize(F); hm.fr.resize(F); hm.ftag.resize(F); hm.fT.resize(9 * (size_t)F); hm.fS.resize(F); hm.fdist.resize(F);
