@@ -160,8 +160,12 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     HGKS_CUDA(cudaMemset(s.wface, 0, sizeof(double) * 2 * NG * kFaceState * F));
   }
   s.vstride = (int64_t)((5 * N + 63) / 64 * 64);
-  if (implicit && !s.off) {
-    if ((st = dalloc(m, &s.off, 25 * NF * N))) return st;
+  // the off-diagonal part of A: operands of its products, or an arena's stored blocks
+  const bool arena = m.d.ptab != nullptr;
+  const size_t rows = arena ? 25 * NF : 6 + 5 * NF;
+  double *&blocks = arena ? s.off : s.jv64;
+  if (implicit && !blocks) {
+    if ((st = dalloc(m, &blocks, rows * N))) return st;
     if ((st = dalloc(m, &s.dval, N))) return st;
     if ((st = dalloc(m, &s.dinv, N))) return st;
     if ((st = dalloc(m, &s.R, 5 * N))) return st;
@@ -172,7 +176,11 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     if ((st = dalloc(m, &s.t2, 5 * N))) return st;
     if ((st = dalloc(m, &s.hs, 65 * 64 + 256))) return st;
     if ((st = dalloc(m, &s.gram, 65 * 65 + 2 * 65 + 64))) return st;
-    HGKS_CUDA(cudaMemset(s.off, 0, sizeof(double) * 25 * NF * N));
+    HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
+  }
+  if (implicit && !mixed && !arena && !s.z[0]) {
+    for (double *&z : s.z)
+      if ((st = dalloc(m, &z, 6 * N))) return st;
   }
   if (implicit && mixed && !s.jv32) {
     if ((st = dalloc(m, &s.jv32, (6 + 4 * NF) * N))) return st;
@@ -431,7 +439,7 @@ hgks_status hgks_assemble(hgks_mesh mesh, const hgks_params *p, const double *Q,
 hgks_status hgks_apply_jacobian(hgks_mesh mesh, const double *x, double *y, void *cuda_stream) {
   if (!mesh || !x || !y) return fail(HGKS_ERR_ARG, "NULL argument");
   Mesh &m = mesh->m;
-  if (!m.s.off) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
+  if (!m.s.jv64) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
   HGKS_ON_DEVICE(m.device);
   launch_apply_A(m.d, m.s, x, y, (cudaStream_t)cuda_stream);
   return last_launch();
@@ -481,7 +489,7 @@ hgks_status hgks_precondition(hgks_mesh mesh, int32_t sweeps, const double *b, d
   if (b == x) return fail(HGKS_ERR_ARG, "b and x must not alias");
   if (sweeps < 0) return fail(HGKS_ERR_ARG, "negative sweeps");
   Mesh &m = mesh->m;
-  if (!m.s.off) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
+  if (!m.s.jv64) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
   HGKS_ON_DEVICE(m.device);
   launch_precondition(m.d, m.s, sweeps, b, x, (cudaStream_t)cuda_stream);
   return last_launch();

@@ -115,7 +115,9 @@ struct Scratch {
   double *fpt = nullptr;         // [NG][5][F] global-frame point values * area * Gauss weight
   // implicit
   double *dinv = nullptr, *dval = nullptr;  // [N] the diagonal block is (|Omega|/dt + sum lambda S/2) I
-  double *off = nullptr;         // [NF*25][N]: block of local face p of the row cell (0 on a boundary)
+  double *off = nullptr;         // batches: [NF*25][N] block of local face p of the row cell (0 on a boundary)
+  double *jv64 = nullptr;        // one mesh: [6 + 5 NF][N] the off-diagonal blocks as products (offdiag.cuh)
+  double *z[2] = {nullptr, nullptr};   // [6][N] Krylov vectors in the form of z_of (offdiag.cuh)
   float *jv32 = nullptr;         // [6 + 4 NF][N] mixed precision: the off-diagonal blocks as products,
                                  // rows 0-5 per cell (u, v, w, H, (gamma-1)|u|^2/2, gamma-1),
                                  // rows 6 + 4p + k per (cell, local face p): n S/2 (k < 3), lambda S/2
@@ -130,7 +132,7 @@ struct Scratch {
   double *red = nullptr;         // reduction partials
   unsigned int *red_count = nullptr;
   double *hs = nullptr;          // small device scalars: H, beta, y, norms
-  double *gram = nullptr;        // [65*65 + 2*65] Gram matrix of the Krylov basis and the MGS pass sums
+  double *gram = nullptr;        // [65*65 + 2*65] inner products of the Krylov basis and the MGS pass sums
   int *flags = nullptr;          // [8] device flags (nonphysical count, breakdown)
   double *hostbuf = nullptr;     // [40][N] device state of the *_host entry points
   double *Qp = nullptr, *Rp = nullptr;   // [5][N] perturbed state and its residual (matrix-free products)
@@ -199,6 +201,12 @@ hgks_status gmres_solve(const DevMesh &m, Scratch &s, const hgks_params &p, cons
 // needs s.R = L(Q) and s.dt, and ||Q|| in s.hs[kHsNormQ]
 void launch_apply_fd(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *G,
                      const double *x, const double *b, double *y, cudaStream_t st);
+// FP64 GMRES with the assembled A (gmres64.cu); Hj: column j of H (leading dimension mk)
+void launch_scale_z(const DevMesh &m, const Scratch &s, const double *w, const double *h, double *v, double *zv,
+                    cudaStream_t st);
+void launch_neumann_z(const DevMesh &m, const Scratch &s, int sweeps, const double *v, double *w, int j, int mk, double *Hj,
+                      cudaStream_t st);
+void launch_mgs_blocks(const Scratch &s, int64_t n, double *w, int j, int mk, double *Hj, bool have_first, cudaStream_t st);
 void launch_norm(const DevMesh &m, Scratch &s, const double *x, double *out_dev, cudaStream_t st);
 // force[3] on the boundary faces tagged `tag`, from the face fluxes of the last residual
 void launch_wall_force(const DevMesh &m, const Scratch &s, int tag, double *force_dev, cudaStream_t st);

@@ -6,9 +6,10 @@
 //    The Euler-Jacobian part of A_ii is J(Q_i) applied to sum_p n_p S_p, the
 //    sum of a closed cell's outward area vectors, which is zero: A_ii is a
 //    multiple of the identity and is stored as one number per cell. The
-//    off-diagonal blocks form the per-cell "structure array" of Sec. 4.3,
-//    stored component-major off[(p*25 + k)][N] (p = local face of the row cell)
-//    so that the thread of cell i reads consecutive addresses with its warp.
+//    off-diagonal blocks (the per-cell "structure array" of Sec. 4.3) are kept as
+//    the operands of their products (offdiag.cuh), component-major so that the
+//    thread of cell i reads consecutive addresses with its warp; batches with FP64
+//    vectors store them, off[(p*25 + k)][N] (p = local face of the row cell).
 //  * Jacobi preconditioner of Eq. (precond), k_max sweeps. The first sweep reads
 //    D^{-1} b of the neighbours on the fly (no separate x0 pass).
 //  * Restarted GMRES with modified Gram-Schmidt (Algorithm 1). Every inner
@@ -50,23 +51,25 @@ __device__ __forceinline__ void euler_jacobian(const double *Q, const double *n,
   J[24] = gamma * un;
 }
 
-// jv32 (may be null): FP32 operands of the product form of the off-diagonal
-// blocks (mixed precision), with dval32, dinv32
+// off, off_out: the blocks themselves (may be null); jv64, jv32 (may be null): the operands
+// of their product form, FP32 (mixed precision) with dval32, dinv32. Bound by what it
+// writes: 26 doubles a cell (jv64, tetrahedra) instead of the 100 of the blocks.
 template <bool BATCH, int NF>
 __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
                                                          const double *__restrict__ dt, double *__restrict__ dval,
                                                          double *__restrict__ dinv, double *__restrict__ off,
                                                          double *__restrict__ diag_out, double *__restrict__ off_out,
                                                          float *__restrict__ dval32, float *__restrict__ dinv32,
-                                                         float *__restrict__ jv32) {
+                                                         float *__restrict__ jv32, double *__restrict__ jv64) {
   const int N = m.N, F = m.F;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   if (BATCH && m.cmesh[i] < 0) {                          // padding cell of a batch: identity row
     dval[i] = 1.0;
     dinv[i] = 1.0;
+    if (off)
 #pragma unroll 4
-    for (int k = 0; k < 25 * NF; k++) off[(size_t)k * N + i] = 0.0;
+      for (int k = 0; k < 25 * NF; k++) off[(size_t)k * N + i] = 0.0;
     if (jv32) {
       dval32[i] = 1.0f;
       dinv32[i] = 1.0f;
@@ -80,12 +83,15 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
   double Qi[5];
 #pragma unroll
   for (int c = 0; c < 5; c++) Qi[c] = Q[(size_t)c * N + i];
-  if (jv32) {                                           // this cell's primitives, for the rows of its neighbours
+  if (jv32 || jv64) {                                   // this cell's primitives, for the rows of its neighbours
     const double ir = 1.0 / Qi[0], g1 = P.gamma - 1.0;
     const double u = Qi[1] * ir, v = Qi[2] * ir, w = Qi[3] * ir, phi = 0.5 * g1 * (u * u + v * v + w * w);
     const double pk[6] = {u, v, w, P.gamma * Qi[4] * ir - phi, phi, g1};
 #pragma unroll
-    for (int k = 0; k < 6; k++) jv32[(size_t)k * N + i] = (float)pk[k];
+    for (int k = 0; k < 6; k++) {
+      if (jv32) jv32[(size_t)k * N + i] = (float)pk[k];
+      if (jv64) jv64[(size_t)k * N + i] = pk[k];
+    }
   }
   double d = m.vol[i] / dt[i];
 #pragma unroll 1
@@ -113,13 +119,22 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
 #pragma unroll
       for (int k = 0; k < 4; k++)
         jv32[(size_t)(6 + 4 * p + k) * N + i] = j >= 0 ? (float)(0.5 * S * (k < 3 ? n[k] : lam)) : 0.0f;
-    double J[25];
-    if (j >= 0) euler_jacobian(Qj, n, P.gamma, J);
+    if (jv64) {
+      const double hS = j >= 0 ? 0.5 * S : 0.0, iq = 1.0 / Qj[0];
+      const double un = iq * (Qj[1] * n[0] + Qj[2] * n[1] + Qj[3] * n[2]);
+      const double rec[5] = {hS * n[0], hS * n[1], hS * n[2], hS * lam, hS * (un - lam)};
 #pragma unroll
-    for (int k = 0; k < 25; k++) {
-      const double o = j >= 0 ? 0.5 * (J[k] - (k % 6 == 0 ? lam : 0.0)) * S : 0.0;
-      off[(size_t)(p * 25 + k) * N + i] = o;
-      if (off_out) off_out[(size_t)(p * 25 + k) * N + i] = o;
+      for (int k = 0; k < 5; k++) jv64[(size_t)(6 + 5 * p + k) * N + i] = rec[k];
+    }
+    if (off || off_out) {
+      double J[25];
+      if (j >= 0) euler_jacobian(Qj, n, P.gamma, J);
+#pragma unroll
+      for (int k = 0; k < 25; k++) {
+        const double o = j >= 0 ? 0.5 * (J[k] - (k % 6 == 0 ? lam : 0.0)) * S : 0.0;
+        if (off) off[(size_t)(p * 25 + k) * N + i] = o;
+        if (off_out) off_out[(size_t)(p * 25 + k) * N + i] = o;
+      }
     }
   }
   dval[i] = d;
@@ -180,14 +195,12 @@ __device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, 
 //   kNeumann: y = b + D^{-1} sum_p A_ip x_p
 //   kE, kNegE: y = +- D^{-1} sum_p A_ip x_p
 // and optionally the inner product (y, dotv) reduced into *dot_out.
-// TM: type of the stored blocks, TV: type of b and x (and of the accumulation),
-// TO: type of y.
+// TM: type of the operands of the blocks, TV: type of b and x (and of the
+// accumulation), TO: type of y. The Krylov products of FP64 vectors are in gmres64.cu.
 enum { kSpmv = 0, kJacobi = 1, kNeumann = 2, kE = 3, kNegE = 4 };
 
-// TM = float: the off-diagonal blocks come as products from jv (mixed precision);
-// TM = double: stored 5x5 blocks in off.
 template <typename TM, typename TV, typename TO, int Mode, bool FirstSweep, int NF>
-__global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const TM *__restrict__ off, const TM *__restrict__ dval,
+__global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const TM *__restrict__ jv, const TM *__restrict__ dval,
                                                       const TM *__restrict__ dinv, const TV *__restrict__ b,
                                                       const TV *__restrict__ x, TO *__restrict__ y,
                                                       const TO *__restrict__ dotv, TO *partials, unsigned int *count,
@@ -208,18 +221,7 @@ __global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const TM *__res
       const TV sj = FirstSweep ? (TV)dinv[j] : TV(1);
 #pragma unroll
       for (int c = 0; c < 5; c++) xj[c] = FirstSweep ? sj * b[(size_t)c * N + j] : x[(size_t)c * N + j];
-      if constexpr (std::is_same<TM, float>::value) {
-        offdiag_product<TV>(reinterpret_cast<const float *>(off), N, i, p, j, xj, acc);
-      } else {
-        const TM *O = off + (size_t)p * 25 * N + i;
-#pragma unroll
-        for (int r = 0; r < 5; r++)
-#pragma unroll
-          for (int c = 0; c < 5; c++) {
-            if (r == 0 && c == 4) continue;     // row 0 of J(Q)n is (0, n, 0): this entry is zero
-            acc[r] = fma((TV)O[(size_t)(5 * r + c) * N], xj[c], acc[r]);
-          }
-      }
+      offdiag_product<TV>(jv, N, i, p, j, xj, acc);
     }
     TV out[5];
     if (Mode == kJacobi) {
@@ -253,13 +255,13 @@ __global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const TM *__res
 
 // k_apply for the mesh's cell kind (4 or 6 off-diagonal blocks per row)
 template <typename TM, typename TV, typename TO, int Mode, bool FirstSweep>
-void apply_launch(unsigned grid, cudaStream_t st, const DevMesh &m, const TM *off, const TM *dval, const TM *dinv,
+void apply_launch(unsigned grid, cudaStream_t st, const DevMesh &m, const TM *jv, const TM *dval, const TM *dinv,
                   const TV *b, const TV *x, TO *y, const TO *dotv, TO *partials, unsigned int *count, double *dot_out) {
   if (m.hex)
-    k_apply<TM, TV, TO, Mode, FirstSweep, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, off, dval, dinv, b, x, y, dotv,
+    k_apply<TM, TV, TO, Mode, FirstSweep, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, jv, dval, dinv, b, x, y, dotv,
                                                                                       partials, count, dot_out);
   else
-    k_apply<TM, TV, TO, Mode, FirstSweep, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, off, dval, dinv, b, x, y, dotv,
+    k_apply<TM, TV, TO, Mode, FirstSweep, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, jv, dval, dinv, b, x, y, dotv,
                                                                                       partials, count, dot_out);
 }
 
@@ -450,129 +452,6 @@ __global__ void __launch_bounds__(kBlock) k_mupdate(int64_t n, T *__restrict__ w
   grid_sum(s, partials, count, norm_out, 1);
 }
 
-// ---- modified Gram-Schmidt two basis vectors per pass (FP64 vectors) ----
-// For a pair (v_c, v_{c+1}) Algorithm 1 takes h_c = (w_c, v_c) and
-//   h_{c+1} = (w_c - h_c v_c, v_{c+1}) = (w_c, v_{c+1}) - h_c g_c,  g_c = (v_c, v_{c+1}),
-// so one pass over w, v_c and v_{c+1} gives both coefficients. The same pass first
-// subtracts the previous pair (v_a, v_b) with its known coefficients, in MGS
-// order. The last pass of step j (vc == nullptr) subtracts the last vectors and
-// takes ||w|| and (w, v_j): then g_j = (v_j, w / ||w||) = (v_j, v_{j+1}) for the
-// steps that follow. Per pair 48 bytes and 4 FMAs per element (24 bytes per basis
-// vector against 32 for one vector per pass) keep the pass bound by HBM.
-//   update: w -= ha va; if vb: w -= hb vb
-//   vc:     *hc_out = (w, vc); if vd: *hd_out = (w, vd) - (w, vc) * *g_io
-//   !vc:    *hc_out = ||w||; *g_io = (w, vlast) / ||w|| (0 if ||w|| == 0), vlast = vb ? vb : va
-template <typename T, int NB, int ND>
-__global__ void __launch_bounds__(kBlock) k_mgs2(int64_t n, T *__restrict__ w, const T *__restrict__ va,
-                                                 const T *__restrict__ vb, const double *__restrict__ ha,
-                                                 const double *__restrict__ hb, const T *__restrict__ vc,
-                                                 const T *__restrict__ vd, T *partials, unsigned int *count,
-                                                 double *hc_out, double *hd_out, double *g_io) {
-  // NB: vectors subtracted (1: va, 2: va and vb); ND: vectors dotted (0: the last
-  // pass, 1: vc, 2: vc and vd)
-  typedef typename Vec16<T>::type TV;
-  constexpr int L = Vec16<T>::n;
-  constexpr bool fin = ND == 0;
-  const T na = (T)(-*ha), nb = NB == 2 ? (T)(-*hb) : T(0);
-  // the vectors of the two sums: (w, x0) and (w, x1); the last pass: x0 = w, x1 = vlast
-  const T *x1 = fin ? (NB == 2 ? vb : va) : vd;
-  T s0 = T(0), s1 = T(0);
-  const int64_t nv = n / L, stride = (int64_t)gridDim.x * blockDim.x;
-  const TV *VA = reinterpret_cast<const TV *>(va), *VB = reinterpret_cast<const TV *>(vb);
-  const TV *VC = reinterpret_cast<const TV *>(vc), *X1 = reinterpret_cast<const TV *>(x1);
-  TV *WV = reinterpret_cast<TV *>(w);
-#pragma unroll 2
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nv; k += stride) {
-    // every load of the step first (w is written only after them)
-    TV wk = WV[k];
-    const TV ak = VA[k];
-    TV bk, ck, xk;
-    if constexpr (NB == 2) bk = VB[k];
-    if constexpr (!fin) ck = VC[k];
-    if constexpr (fin || ND == 2) xk = X1[k];
-    T *wa = reinterpret_cast<T *>(&wk);
-    const T *aa = reinterpret_cast<const T *>(&ak);
-#pragma unroll
-    for (int l = 0; l < L; l++) wa[l] = fma(na, aa[l], wa[l]);
-    if constexpr (NB == 2) {
-      const T *ba = reinterpret_cast<const T *>(&bk);
-#pragma unroll
-      for (int l = 0; l < L; l++) wa[l] = fma(nb, ba[l], wa[l]);
-    }
-    if constexpr (fin) {
-#pragma unroll
-      for (int l = 0; l < L; l++) s0 = fma(wa[l], wa[l], s0);
-    } else {
-      const T *ca = reinterpret_cast<const T *>(&ck);
-#pragma unroll
-      for (int l = 0; l < L; l++) s0 = fma(wa[l], ca[l], s0);
-    }
-    if constexpr (fin || ND == 2) {
-      const T *xa = reinterpret_cast<const T *>(&xk);
-#pragma unroll
-      for (int l = 0; l < L; l++) s1 = fma(wa[l], xa[l], s1);
-    }
-    WV[k] = wk;
-  }
-  for (int64_t k = nv * L + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += stride) {
-    T wk = fma(na, va[k], w[k]);
-    if constexpr (NB == 2) wk = fma(nb, vb[k], wk);
-    w[k] = wk;
-    s0 = fma(wk, fin ? wk : vc[k], s0);
-    if constexpr (fin || ND == 2) s1 = fma(wk, x1[k], s1);
-  }
-  // deterministic reduction of both sums (as grid_sum)
-  __shared__ bool last;
-  const T b0 = block_sum(s0);
-  const T b1 = block_sum(s1);
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = b0;
-    partials[gridDim.x + blockIdx.x] = b1;
-    __threadfence();
-    const unsigned int prev = atomicAdd(count, 1u);
-    last = (prev == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  T t0 = T(0), t1 = T(0);
-  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-    t0 += ((volatile T *)partials)[b];
-    t1 += ((volatile T *)partials)[gridDim.x + b];
-  }
-  t0 = block_sum(t0);
-  t1 = block_sum(t1);
-  if (threadIdx.x == 0) {
-    if (fin) {
-      const double nrm = sqrt((double)t0);
-      *hc_out = nrm;
-      *g_io = nrm > 0.0 ? (double)t1 / nrm : 0.0;
-    } else {
-      *hc_out = (double)t0;
-      if (ND == 2) *hd_out = (double)t1 - (double)t0 * *g_io;
-    }
-    *count = 0u;
-  }
-}
-
-// one pass of the pair MGS with the instance for the number of vectors
-template <typename T>
-void launch_mgs2(cudaStream_t st, int64_t n, T *w, const T *va, const T *vb, const double *ha, const double *hb,
-                 const T *vc, const T *vd, T *partials, unsigned int *count, double *hc_out, double *hd_out,
-                 double *g_io) {
-  const int nb = vb ? 2 : 1, nd = vc ? (vd ? 2 : 1) : 0;
-#define HGKS_MGS2(NB, ND)                                                                                        \
-  k_mgs2<T, NB, ND><<<kRedBlocks, kBlock, 0, st>>>(n, w, va, vb, ha, hb, vc, vd, partials, count, hc_out, hd_out, \
-                                                   g_io)
-  if (nb == 1 && nd == 0) HGKS_MGS2(1, 0);
-  else if (nb == 1 && nd == 1) HGKS_MGS2(1, 1);
-  else if (nb == 1) HGKS_MGS2(1, 2);
-  else if (nd == 0) HGKS_MGS2(2, 0);
-  else if (nd == 1) HGKS_MGS2(2, 1);
-  else HGKS_MGS2(2, 2);
-#undef HGKS_MGS2
-}
-
 // v = w / h (v = 0 after a breakdown h == 0), 16 bytes per thread and step
 template <typename T>
 __global__ void k_scale(int64_t n, const T *__restrict__ w, const double *__restrict__ h, T *__restrict__ v) {
@@ -680,10 +559,10 @@ unsigned vec_grid(int64_t n) {
 // Buffers of one precision for the Krylov part of a step.
 template <typename T>
 struct KBuf {
-  const T *off, *dval, *dinv;
+  const T *jv, *dval, *dinv;
   T *V, *w, *t, *t2, *red;
 };
-KBuf<double> kbuf64(Scratch &s) { return {s.off, s.dval, s.dinv, s.V, s.w, s.t, s.t2, s.red}; }
+KBuf<double> kbuf64(Scratch &s) { return {s.jv64, s.dval, s.dinv, s.V, s.w, s.t, s.t2, s.red}; }
 KBuf<float> kbuf32(Scratch &s) { return {s.jv32, s.dval32, s.dinv32, s.V32, s.w32, s.t32, s.t232, s.red32}; }
 
 template <typename T> T *partials(Scratch &s);
@@ -732,10 +611,10 @@ void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, 
     const T *dv = (q == sweeps) ? dotv : nullptr;
     HGKS_PROF_BEGIN(K_JACOBI, st);
     if (q == 1)
-      apply_launch<T, T, T, kJacobi, true>(cg, st, m, k.off, k.dval, k.dinv, b, nullptr, dst, dv, k.red,
+      apply_launch<T, T, T, kJacobi, true>(cg, st, m, k.jv, k.dval, k.dinv, b, nullptr, dst, dv, k.red,
                                                                   s.red_count, dot_out);
     else
-      apply_launch<T, T, T, kJacobi, false>(cg, st, m, k.off, k.dval, k.dinv, b, prev, dst, dv, k.red,
+      apply_launch<T, T, T, kJacobi, false>(cg, st, m, k.jv, k.dval, k.dinv, b, prev, dst, dv, k.red,
                                                                    s.red_count, dot_out);
     HGKS_PROF_END(K_JACOBI, st);
     prev = dst;
@@ -749,27 +628,26 @@ void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, 
 // E^k v with the sign in its first product): k + 1
 // products with O instead of the product with A followed by k sweeps: the same
 // vector up to rounding, without the diagonal terms of A and the scaling of the
-// neighbours' values by D^{-1}. The last launch also reduces (w, dotv) into *dot_out.
-template <typename T>
-void neumann_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, const T *v, T *w, const T *dotv,
-               double *dot_out, cudaStream_t st) {
+// neighbours' values by D^{-1}. (FP32 vectors; FP64: launch_neumann_z.)
+void neumann32(const DevMesh &m, Scratch &s, const KBuf<float> &k, int sweeps, const float *v, float *w,
+               cudaStream_t st) {
   const unsigned cg = grid_for(m.N, kCellBlock);
-  const T *z = v;
+  const float *z = v, *none = nullptr;
   for (int q = 0; q < sweeps; q++) {
-    T *dst = (q % 2 == 0) ? k.t : k.t2;
+    float *dst = (q % 2 == 0) ? k.t : k.t2;
     HGKS_PROF_BEGIN(K_JACOBI, st);
     if (q == 0 && sweeps % 2 == 1)
-      apply_launch<T, T, T, kNegE, false>(cg, st, m, k.off, k.dval, k.dinv, nullptr, z, dst, nullptr,
-                                                                 k.red, s.red_count, nullptr);
+      apply_launch<float, float, float, kNegE, false>(cg, st, m, k.jv, k.dval, k.dinv, none, z, dst, none, k.red,
+                                                      s.red_count, nullptr);
     else
-      apply_launch<T, T, T, kE, false>(cg, st, m, k.off, k.dval, k.dinv, nullptr, z, dst, nullptr,
-                                                              k.red, s.red_count, nullptr);
+      apply_launch<float, float, float, kE, false>(cg, st, m, k.jv, k.dval, k.dinv, none, z, dst, none, k.red,
+                                                   s.red_count, nullptr);
     HGKS_PROF_END(K_JACOBI, st);
     z = dst;
   }
   HGKS_PROF_BEGIN(K_SPMV, st);
-  apply_launch<T, T, T, kNeumann, false>(cg, st, m, k.off, k.dval, k.dinv, v, z, w, dotv, k.red,
-                                                                s.red_count, dot_out);
+  apply_launch<float, float, float, kNeumann, false>(cg, st, m, k.jv, k.dval, k.dinv, v, z, w, none, k.red,
+                                                     s.red_count, nullptr);
   HGKS_PROF_END(K_SPMV, st);
 }
 
@@ -785,7 +663,8 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
   // The one-pass MGS does 3 FMAs per element and basis vector against 2 for the
   // step-by-step form, and reads about half the bytes: with FP32 vectors it is
   // bound by HBM and wins; with FP64 vectors both forms sit at GB300's FP64 rate
-  // (one FP64 FMA per 8 bytes read already exceeds it), so FP64 keeps the steps.
+  // (one FP64 FMA per 8 bytes read already exceeds it), so FP64 goes by blocks
+  // (gmres64.cu), 2 FMAs and 20 bytes.
   constexpr bool one_pass = std::is_same<T, float>::value;
   const unsigned vg = vec_grid(n), cg = grid_for(m.N, kCellBlock);
   for (int it = 0; it < p.restarts; it++) {
@@ -799,7 +678,7 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
       HGKS_PROF_END(K_SPMV, st);
     } else {
       HGKS_PROF_BEGIN(K_SPMV, st);
-      apply_launch<T, double, T, kSpmv, false>(cg, st, m, k.off, k.dval, k.dinv, rhs, dx, k.t, nullptr,
+      apply_launch<T, double, T, kSpmv, false>(cg, st, m, k.jv, k.dval, k.dinv, rhs, dx, k.t, nullptr,
                                                                       nullptr, nullptr, nullptr);
       HGKS_PROF_END(K_SPMV, st);
     }
@@ -808,20 +687,27 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
     k_axpy_dot<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, nullptr, nullptr, k.w, 1, k.red, s.red_count, beta);
     HGKS_PROF_END(K_DOT, st);
     if (it == 0) cudaMemcpyAsync(lres, beta, sizeof(double), cudaMemcpyDeviceToDevice, st);
-    HGKS_PROF_BEGIN(K_SCALE, st);
-    k_scale<T><<<vg, kBlock, 0, st>>>(n, k.w, beta, k.V);
-    HGKS_PROF_END(K_SCALE, st);
+    // v = w / h; FP64 with the assembled A: with the form that the products read
+    auto scale = [&](const double *h, T *v) {
+      if constexpr (!one_pass)
+        if (!fd) return launch_scale_z(m, s, k.w, h, v, s.z[0], st);
+      HGKS_PROF_BEGIN(K_SCALE, st);
+      k_scale<T><<<vg, kBlock, 0, st>>>(n, k.w, h, v);
+      HGKS_PROF_END(K_SCALE, st);
+    };
+    scale(beta, k.V);
     for (int j = 0; j < mk; j++) {
-      // w = P^{-1} A v_j (FP64: with h_0j = (w, v_0) from the last launch)
-      const T *dv = one_pass ? nullptr : k.V;
-      double *dout = one_pass ? nullptr : H + j;
+      // w = P^{-1} A v_j (FP64: with the first block's coefficients from the last product)
+      const T *vj = k.V + (size_t)j * vs;
       if (fd) {
-        fd_apply<T, T>(m, s, p, Q, G, k.V + (size_t)j * vs, nullptr, k.t, st);
-        precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, dv, dout, st);
+        fd_apply<T, T>(m, s, p, Q, G, vj, nullptr, k.t, st);
+        precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, nullptr, nullptr, st);
+      } else if constexpr (one_pass) {
+        neumann32(m, s, k, p.jacobi_sweeps, vj, k.w, st);
       } else {
-        neumann_t<T>(m, s, k, p.jacobi_sweeps, k.V + (size_t)j * vs, k.w, dv, dout, st);
+        launch_neumann_z(m, s, p.jacobi_sweeps, vj, k.w, j, mk, H + j, st);
       }
-      if (one_pass) {
+      if constexpr (one_pass) {
         // modified Gram-Schmidt: the coefficients h_ij from one pass over the basis,
         // then w -= sum h_ij v_i in MGS order and h_{j+1,j} = ||w||
         for (int k0 = 0; k0 <= j; k0 += kMdot) {
@@ -837,30 +723,9 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
         k_mupdate<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, k.V, vs, j, mk, H, k.red, s.red_count, H + (j + 1) * mk + j);
         HGKS_PROF_END(K_DOT, st);
       } else {
-        // modified Gram-Schmidt two vectors per pass (h_0j came with the product):
-        // subtract the pending vectors (ua, ub), take the inner products with the
-        // next two (c, c + 1); the last pass takes ||w|| and g_j = (v_j, v_{j+1})
-        // into gram[j]
-        auto vec = [&](int q) { return k.V + (size_t)q * vs; };
-        int ua = 0, ub = -1, c = 1;
-        for (;;) {
-          const bool fin = c > j;
-          const int d = (!fin && c + 1 <= j) ? c + 1 : -1;
-          HGKS_PROF_BEGIN(K_DOT, st);
-          launch_mgs2<T>(st, n, k.w, vec(ua), ub >= 0 ? vec(ub) : nullptr, H + ua * mk + j,
-                         ub >= 0 ? H + ub * mk + j : nullptr, fin ? nullptr : vec(c), d >= 0 ? vec(d) : nullptr, k.red,
-                         s.red_count, fin ? H + (j + 1) * mk + j : H + c * mk + j, d >= 0 ? H + d * mk + j : nullptr,
-                         fin ? gram + j : (d >= 0 ? gram + c : nullptr));
-          HGKS_PROF_END(K_DOT, st);
-          if (fin) break;
-          ua = c;
-          ub = d;
-          c += d >= 0 ? 2 : 1;
-        }
+        launch_mgs_blocks(s, n, k.w, j, mk, H + j, !fd, st);
       }
-      HGKS_PROF_BEGIN(K_SCALE, st);
-      k_scale<T><<<vg, kBlock, 0, st>>>(n, k.w, H + (j + 1) * mk + j, k.V + (size_t)(j + 1) * vs);
-      HGKS_PROF_END(K_SCALE, st);
+      scale(H + (j + 1) * mk + j, k.V + (size_t)(j + 1) * vs);
     }
     HGKS_PROF_BEGIN(K_GIVENS, st);
     k_givens<<<1, 32, 0, st>>>(mk, H, beta, y, lres + 1);
@@ -881,24 +746,26 @@ void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &p, const d
   float *dv32 = mixed ? s.dval32 : nullptr, *di32 = mixed ? s.dinv32 : nullptr, *jv = mixed ? s.jv32 : nullptr;
   HGKS_PROF_BEGIN(K_ASSEMBLE, st);
   batch = batch || m.ptab;
+  // batches with FP64 vectors read the stored blocks, one mesh the operands
+  double *off = batch && !mixed ? s.off : nullptr, *j64 = batch ? nullptr : s.jv64;
   if (batch && m.hex)
-    k_assemble<true, HexShape::NF><<<grid_for(m.NL, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, s.off,
-                                                                                       diag_out, off_out, dv32, di32, jv);
+    k_assemble<true, HexShape::NF><<<grid_for(m.NL, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, off,
+                                                                                       diag_out, off_out, dv32, di32, jv, j64);
   else if (batch)
-    k_assemble<true, TetShape::NF><<<grid_for(m.NL, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, s.off,
-                                                                                       diag_out, off_out, dv32, di32, jv);
+    k_assemble<true, TetShape::NF><<<grid_for(m.NL, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, off,
+                                                                                       diag_out, off_out, dv32, di32, jv, j64);
   else if (m.hex)
-    k_assemble<false, HexShape::NF><<<grid_for(m.N, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, s.off,
-                                                                                       diag_out, off_out, dv32, di32, jv);
+    k_assemble<false, HexShape::NF><<<grid_for(m.N, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, off,
+                                                                                       diag_out, off_out, dv32, di32, jv, j64);
   else
-    k_assemble<false, TetShape::NF><<<grid_for(m.N, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, s.off,
-                                                                                       diag_out, off_out, dv32, di32, jv);
+    k_assemble<false, TetShape::NF><<<grid_for(m.N, kCellBlock), kCellBlock, 0, st>>>(m, p, Q, dt, s.dval, s.dinv, off,
+                                                                                       diag_out, off_out, dv32, di32, jv, j64);
   HGKS_PROF_END(K_ASSEMBLE, st);
 }
 
 void launch_apply_A(const DevMesh &m, const Scratch &s, const double *x, double *y, cudaStream_t st) {
   HGKS_PROF_BEGIN(K_SPMV, st);
-  apply_launch<double, double, double, kSpmv, false>(grid_for(m.N, kCellBlock), st, m, s.off, s.dval, s.dinv,
+  apply_launch<double, double, double, kSpmv, false>(grid_for(m.N, kCellBlock), st, m, s.jv64, s.dval, s.dinv,
                                                      (const double *)nullptr, x, y, (const double *)nullptr,
                                                      (double *)nullptr, nullptr, nullptr);
   HGKS_PROF_END(K_SPMV, st);
