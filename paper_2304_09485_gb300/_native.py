@@ -18,7 +18,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libhgks.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["residual.cu", "implicit.cu", "gmres64.cu", "batch.cu", "batch_capi.cu", "server.cu", "capi.cu", "noalloc.cu", "peak.cu", "mesh_setup.cpp"]
-HEADERS = ["hgks_internal.h", "givens.cuh", "offdiag.cuh", "reduce.cuh", "batch_impl.h"]
+HEADERS = ["hgks_internal.h", "givens.cuh", "offdiag.cuh", "reduce.cuh", "fp64.cuh", "fp64_tables.h", "batch_impl.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

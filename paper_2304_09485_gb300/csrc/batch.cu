@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kB) k_bdensity(int N, BatchDev bd, const doubl
 }
 
 // Q += dQ and G = G_new for the meshes still iterating
-__global__ void __launch_bounds__(kB) k_bupdate(int N, BatchDev bd, const hgks_params *__restrict__ ptab,
+__global__ void __launch_bounds__(kB) k_bupdate(int N, BatchDev bd, const KParams *__restrict__ ptab,
                                                 double *__restrict__ Q, const double *__restrict__ dQ,
                                                 double *__restrict__ G, const double *__restrict__ Gnew, int ng) {
   const int i = blockIdx.x * kB + threadIdx.x;

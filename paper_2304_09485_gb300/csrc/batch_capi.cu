@@ -291,7 +291,7 @@ hgks_status batch_new(int device, int64_t cell_cap, int64_t face_cap, int nslot,
     cudaMemsetAsync(d.H0, 0, sizeof(double) * 9 * rw.HCOLS * N, st);
     cudaMemsetAsync(d.Hm, 0, sizeof(double) * rw.NF * 21 * N, st);
   }
-  cudaMemsetAsync(B->ptab, 0, sizeof(hgks_params) * nslot, st);
+  cudaMemsetAsync(B->ptab, 0, sizeof(KParams) * nslot, st);
   cudaMemsetAsync(B->cmesh, 0xff, sizeof(short) * N, st);
   cudaMemsetAsync(B->fmesh, 0xff, sizeof(short) * F, st);
   cudaMemsetAsync(B->bmesh, 0xff, sizeof(short) * nb, st);
@@ -375,7 +375,8 @@ hgks_status batch_place(Batch &B, const MeshSource &src, const hgks_params &p, i
   launch_fill_short(B.fmesh + f0, fk, (short)k, st);
   launch_fill_short(B.bmesh + b0, cpad / kBatchBlock, (short)k, st);
   const int bst = (int)b0, bcn = (int)(cpad / kBatchBlock), nc = (int)nk;
-  if ((s = upload(B.ptab + k, &S.p, 1, st)) || (s = upload(B.bstart + k, &bst, 1, st)) ||
+  const KParams kp = kernel_params(S.p);
+  if ((s = upload(B.ptab + k, &kp, 1, st)) || (s = upload(B.bstart + k, &bst, 1, st)) ||
       (s = upload(B.bcount + k, &bcn, 1, st)) || (s = upload(B.ncell + k, &nc, 1, st)))
     return s;
   BCUDA(cudaMemsetAsync(B.bs.hs + (size_t)k * B.bs.hsz, 0, sizeof(double) * B.bs.hsz, st));

@@ -50,7 +50,7 @@ struct Batch {
   std::vector<Slot> slots;
   RangeAlloc cells, faces;               // cells in units of kBatchBlock
   double *Q = nullptr, *G = nullptr;     // [5][N], [15][N] (compact scheme)
-  hgks_params *ptab = nullptr;           // [nslot]
+  KParams *ptab = nullptr;               // [nslot]
   short *cmesh = nullptr, *fmesh = nullptr, *bmesh = nullptr;
   int *bstart = nullptr, *bcount = nullptr, *ncell = nullptr;
   int *active_base = nullptr;            // [nslot + 1], entry 0 = slot -1

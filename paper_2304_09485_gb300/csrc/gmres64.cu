@@ -9,6 +9,7 @@
 // ||w|| in the last pass of step j, whose subtracted vectors they are.
 #include <algorithm>
 #include "hgks_internal.h"
+#include "fp64.cuh"
 #include "offdiag.cuh"
 #include "reduce.cuh"
 
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(kCell) k_scale_z(int N, const double *__restri
                                                    double *__restrict__ zv) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  const double hv = *h, ih = hv != 0.0 ? 1.0 / hv : 0.0;
+  const double hv = *h, ih = hv != 0.0 ? rcp(hv) : 0.0;
   double y[5], z[6];
 #pragma unroll
   for (int c = 0; c < 5; c++) {

@@ -37,6 +37,28 @@ template <class S> struct ShapeOf {
   static constexpr int HCOLS = S::NF + 3 * (1 + S::NF);            // data columns of the compact fit
 };
 
+// Parameters as the kernels take them: with what depends on them alone (an FP64 division in
+// every thread costs nine FP64 instructions).
+struct KParams : hgks_params {
+  double g1, ig1, K2, K4;        // gamma - 1, 1 / (gamma - 1); K + 2 and K + 4 of K internal degrees of freedom
+  double flux_dt_ratio;          // flux_cfl / cfl
+  double prandtl;                // 1 / Pr - 1
+  int32_t fix_prandtl, pad;      // Pr != 1
+};
+inline KParams kernel_params(const hgks_params &p) {
+  KParams k;
+  static_cast<hgks_params &>(k) = p;
+  k.g1 = p.gamma - 1.0;
+  k.ig1 = 1.0 / k.g1;
+  k.K2 = (3.0 - p.gamma) * k.ig1;
+  k.K4 = (p.gamma + 1.0) * k.ig1;
+  k.flux_dt_ratio = p.flux_cfl / p.cfl;
+  k.prandtl = 1.0 / p.Pr - 1.0;
+  k.fix_prandtl = p.Pr != 1.0;
+  k.pad = 0;
+  return k;
+}
+
 struct DevMesh {
   int N = 0, F = 0;
   int hex = 0;                   // 0: tetrahedra (TetShape), 1: hexahedra (HexShape)
@@ -66,7 +88,7 @@ struct DevMesh {
   double *fdist = nullptr;       // [F] |x_L - x_R| (or twice the wall distance on a boundary)
   // batches of meshes (hgks_batch_*): per-mesh parameters and the mesh of every
   // cell (-1 for the padding cells that align each mesh to a 256-cell block) and face
-  const hgks_params *ptab = nullptr;
+  const KParams *ptab = nullptr;
   const short *cmesh = nullptr, *fmesh = nullptr;
   const int *mact = nullptr;             // [meshes] 1 while the mesh iterates; its cells are skipped otherwise
   int NL = 0, FL = 0;                    // batches: cells [0, NL) and faces [0, FL) hold every mesh in use

@@ -21,6 +21,7 @@
 #include <cmath>
 #include <type_traits>
 #include "hgks_internal.h"
+#include "fp64.cuh"
 #include "givens.cuh"
 #include "offdiag.cuh"
 
@@ -55,7 +56,7 @@ __device__ __forceinline__ void euler_jacobian(const double *Q, const double *n,
 // of their product form, FP32 (mixed precision) with dval32, dinv32. Bound by what it
 // writes: 26 doubles a cell (jv64, tetrahedra) instead of the 100 of the blocks.
 template <bool BATCH, int NF>
-__global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
+__global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                          const double *__restrict__ dt, double *__restrict__ dval,
                                                          double *__restrict__ dinv, double *__restrict__ off,
                                                          double *__restrict__ diag_out, double *__restrict__ off_out,
@@ -79,12 +80,12 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
     return;
   }
   if (BATCH && !m.mact[m.cmesh[i]]) return;             // a mesh of a batch that has stopped
-  const hgks_params &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
+  const KParams &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
   double Qi[5];
 #pragma unroll
   for (int c = 0; c < 5; c++) Qi[c] = Q[(size_t)c * N + i];
   if (jv32 || jv64) {                                   // this cell's primitives, for the rows of its neighbours
-    const double ir = 1.0 / Qi[0], g1 = P.gamma - 1.0;
+    const double ir = rcp(Qi[0]), g1 = P.g1;
     const double u = Qi[1] * ir, v = Qi[2] * ir, w = Qi[3] * ir, phi = 0.5 * g1 * (u * u + v * v + w * w);
     const double pk[6] = {u, v, w, P.gamma * Qi[4] * ir - phi, phi, g1};
 #pragma unroll
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
       if (jv64) jv64[(size_t)k * N + i] = pk[k];
     }
   }
-  double d = m.vol[i] / dt[i];
+  double d = m.vol[i] * rcp(dt[i]);
 #pragma unroll 1
   for (int p = 0; p < NF; p++) {
     const int cf = m.cface[(size_t)p * N + i], f = cf >> 1, side = cf & 1;
@@ -109,18 +110,18 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
       Qj[c] = j >= 0 ? Q[(size_t)c * N + j] : Qi[c];
       Qf[c] = 0.5 * (Qi[c] + Qj[c]);
     }
-    const double ir = 1.0 / Qf[0];
+    const double ir = rcp(Qf[0]);
     const double u = Qf[1] * ir, v = Qf[2] * ir, w = Qf[3] * ir;
-    const double pr = (P.gamma - 1.0) * (Qf[4] - 0.5 * Qf[0] * (u * u + v * v + w * w));
-    double lam = fabs(u * n[0] + v * n[1] + w * n[2]) + sqrt(P.gamma * pr * ir);
-    if (P.viscous) lam += 2.0 * P.mu / (Qf[0] * m.fdist[f]);
+    const double pr = P.g1 * (Qf[4] - 0.5 * Qf[0] * (u * u + v * v + w * w));
+    double lam = fabs(u * n[0] + v * n[1] + w * n[2]) + sqrt64(P.gamma * pr * ir);
+    if (P.viscous) lam += 2.0 * P.mu * ir * rcp(m.fdist[f]);
     d += 0.5 * lam * S;
     if (jv32)
 #pragma unroll
       for (int k = 0; k < 4; k++)
         jv32[(size_t)(6 + 4 * p + k) * N + i] = j >= 0 ? (float)(0.5 * S * (k < 3 ? n[k] : lam)) : 0.0f;
     if (jv64) {
-      const double hS = j >= 0 ? 0.5 * S : 0.0, iq = 1.0 / Qj[0];
+      const double hS = j >= 0 ? 0.5 * S : 0.0, iq = rcp(Qj[0]);
       const double un = iq * (Qj[1] * n[0] + Qj[2] * n[1] + Qj[3] * n[2]);
       const double rec[5] = {hS * n[0], hS * n[1], hS * n[2], hS * lam, hS * (un - lam)};
 #pragma unroll
@@ -137,11 +138,12 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, hgks_params 
       }
     }
   }
+  const double id = rcp(d);
   dval[i] = d;
-  dinv[i] = 1.0 / d;
+  dinv[i] = id;
   if (jv32) {
     dval32[i] = (float)d;
-    dinv32[i] = (float)(1.0 / d);
+    dinv32[i] = (float)id;
   }
   if (diag_out)
 #pragma unroll
@@ -738,9 +740,10 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
 
 }  // namespace
 
-void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *dt,
+void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &hp, const double *Q, const double *dt,
                      double *diag_out, double *off_out, cudaStream_t st, bool batch) {
   HGKS_RANGE("hgks assemble");
+  const KParams p = kernel_params(hp);
   // mixed precision: the FP32 operands of the product form come out of the same pass
   const bool mixed = p.precision == HGKS_MIXED && s.jv32;
   float *dv32 = mixed ? s.dval32 : nullptr, *di32 = mixed ? s.dinv32 : nullptr, *jv = mixed ? s.jv32 : nullptr;

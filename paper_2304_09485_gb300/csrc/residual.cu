@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <cmath>
 #include "hgks_internal.h"
+#include "fp64.cuh"
 
 namespace hgks {
 
@@ -34,13 +35,16 @@ constexpr int kBlock = 128;
 // primitive state of a Maxwellian: lam = rho / (2 p), il = 1 / (2 lam) = p / rho, ir = 1 / rho
 struct Prim { double rho, U, V, W, lam, il, ir; };
 
-__device__ __forceinline__ Prim to_prim(const double *Q, double gamma) {
-  // rho p from the conservative variables without a division; one reciprocal
-  // r = 1 / (rho^2 p) then gives both 1/rho = rho p r and lam = rho / (2p) = rho^3 r / 2
+// rho p of a conservative state, without a division
+__device__ __forceinline__ double rho_p(const double *Q, double g1) {
+  return g1 * fma(Q[4], Q[0], -0.5 * fma(Q[1], Q[1], fma(Q[2], Q[2], Q[3] * Q[3])));
+}
+// from Q and rp = rho p: one reciprocal r = 1 / (rho^2 p) gives both 1/rho = rho p r and
+// lam = rho / (2p) = rho^3 r / 2
+__device__ __forceinline__ Prim to_prim(const double *Q, double rp) {
   Prim p;
   p.rho = Q[0];
-  const double rp = (gamma - 1.0) * (Q[4] * Q[0] - 0.5 * (Q[1] * Q[1] + Q[2] * Q[2] + Q[3] * Q[3]));   // rho p
-  const double r = 1.0 / (Q[0] * rp);
+  const double r = rcp(Q[0] * rp);
   p.ir = rp * r;
   p.U = Q[1] * p.ir; p.V = Q[2] * p.ir; p.W = Q[3] * p.ir;
   p.il = rp * p.ir * p.ir;
@@ -63,14 +67,14 @@ __device__ __forceinline__ void rot_out(const double *T, const double *in, doubl
 // Euler eigen-system along x of a face-frame state: scalars of which R (right_apply)
 // and R^{-1} (k_recon's projection) are made.
 struct Eig { double u, v, w, a, H, q2, ia; };
-__device__ __forceinline__ Eig eig_of(const double *Q, double gamma) {
+__device__ __forceinline__ Eig eig_of(const double *Q, double gamma, double g1) {
   Eig e;
-  double ir = 1.0 / Q[0];
+  double ir = rcp(Q[0]);
   e.u = Q[1] * ir; e.v = Q[2] * ir; e.w = Q[3] * ir;
   e.q2 = e.u * e.u + e.v * e.v + e.w * e.w;
-  double p = (gamma - 1.0) * (Q[4] - 0.5 * Q[0] * e.q2);
+  double p = g1 * (Q[4] - 0.5 * Q[0] * e.q2);
   const double a2 = gamma * p * ir;
-  e.ia = rsqrt(a2);
+  e.ia = rsqrt64(a2);
   e.a = a2 * e.ia;
   e.H = (Q[4] + p) * ir;
   return e;
@@ -198,14 +202,14 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 //   kap_0 = (D + tz R_0) / den,  kap_m = gm tz (R_m - R_0) / den,
 //   den = D + tz (g0 R_0 + gm sum R_m).
 // Keeping the projection in shared memory (110 doubles a thread on tetrahedra, 170 on
-// hexahedra) instead of projecting per variable: 28.5 -> 24.8 ms for 9.4M (cell, face) pairs
-// (2,359,296 tetrahedra), 1.24 -> 1.05 ms for 35,937 hexahedra; no spills (604 bytes before).
+// hexahedra) instead of projecting per variable: 28.5 -> 24.4 ms for 9.4M (cell, face) pairs
+// (2,359,296 tetrahedra), 1.24 -> 1.01 ms for 35,937 hexahedra; no spills (604 bytes before).
 // Blocks: any shape up to 256 threads fits on tetrahedra; on hexahedra two blocks of 64
 // fit an SM (85 KB each), one of 128, none of 256.
 constexpr int kReconMax = 256, kReconHex = 64;
 template <class S> constexpr int recon_rows() { return 5 * (10 + 3 * ShapeOf<S>::NSUB); }
 template <bool BATCH, class S>
-__global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
+__global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                      const double *__restrict__ coef, double *__restrict__ wface) {
   constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB, NV = 9 + 3 * NSUB;
   extern __shared__ double proj[];                      // [5][NV + 1][blockDim.x]: column of this thread
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
   const int slot = blockIdx.x % NF, i = (blockIdx.x / NF) * blockDim.x + threadIdx.x;
   if (i >= NL) return;
   if (BATCH && !live(m, i)) return;                     // padding cell, or a mesh that has stopped
-  const hgks_params &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
+  const KParams &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
   const int cf = m.cface[(size_t)slot * N + i];
   const int f = cf >> 1, side = cf & 1;
   const int bd = blockDim.x;
@@ -234,8 +238,8 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
     }
     if (P.characteristic) {
       rot_in(T, Qs, Qsl);
-      const Eig e = eig_of(Qsl, P.gamma);
-      const double hb = 0.5 * (P.gamma - 1.0) * e.ia * e.ia, hi = 0.5 * e.ia;
+      const Eig e = eig_of(Qsl, P.gamma, P.g1);
+      const double hb = 0.5 * P.g1 * e.ia * e.ia, hi = 0.5 * e.ia;
       double pm[3], dm[3];                              // P = p0 q0 + pm . m + hb q4, D = d0 q0 + dm . m
       const double p0 = 0.5 * hb * e.q2, d0 = -hi * e.u;
 #pragma unroll
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
       for (int k = 0; k < 5; k++) my[(size_t)(k * (NV + 1) + NV) * bd] = Qi[k];
     }
   }
-  const double ih = 1.0 / m.h[i];
+  const double ih = rcp(m.h[i]);
   double m2[6], xg[3 * NG];
 #pragma unroll
   for (int k = 0; k < 6; k++) m2[k] = m.m2[(size_t)k * N + i];
@@ -280,7 +284,7 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
   const unsigned valid = P.scheme == HGKS_WENO ? m.subvalid[i] : (1u << NF) - 1u;
   const int M = __popc(valid);
   const double gm = P.lin_weight, g0 = M ? 1.0 - gm * M : 1.0;
-  const double iM = M ? 1.0 / M : 0.0;
+  const double iM = M ? rcp((double)M) : 0.0;
 #pragma unroll
   for (int k = 0; k < 9; k++) T[k] *= ih;               // face frame rows / h: scaled derivatives
   double *out = wface + (size_t)side * NG * kFaceState * F + f;
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
         R0 *= dm[mm];
         if (valid >> mm & 1) sum += R[mm];
       }
-      const double inv = 1.0 / fma(tz, fma(g0, R0, gm * sum), pre), h = gm * tz * inv;
+      const double inv = rcp(fma(tz, fma(g0, R0, gm * sum), pre)), h = gm * tz * inv;
       kap0 = inv * fma(tz, R0, pre);
 #pragma unroll
       for (int j = 0; j < 3; j++) lin[j] = kap0 * ac[j];
@@ -370,8 +374,8 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, hgks_params Pv, 
 // Moments of the normalised Maxwellian of variance il = T = p / rho about (U, V, W),
 // in u over the half range (sgn = +1: u > 0, sgn = -1: u < 0) or the full one:
 //   M_n = <u^n>, M_{n+1} = U M_n + n T M_{n-1} (+ T del for n = 0),
-// del = sgn g(u = 0) the density at the end of the half range (0 for the full range).
-struct Mom { double m0, m1, m2, m3, m4, del; };
+// del = sgn g(u = 0) the density at the end of the half range (0 for the full range); hd = del / 2.
+struct Mom { double m0, m1, m2, m3, m4, hd; };
 __device__ __forceinline__ void mom_up(const Prim &p, Mom &m) {
   m.m2 = fma(p.U, m.m1, p.il * m.m0);
   m.m3 = fma(p.U, m.m2, 2.0 * p.il * m.m1);
@@ -379,17 +383,20 @@ __device__ __forceinline__ void mom_up(const Prim &p, Mom &m) {
 }
 __device__ __forceinline__ Mom mom_full(const Prim &p) {
   Mom m;
-  m.m0 = 1.0; m.m1 = p.U; m.del = 0.0;
+  m.m0 = 1.0; m.m1 = p.U; m.hd = 0.0;
   mom_up(p, m);
   return m;
 }
 // <u^0>, T del and <u^1> = U <u^0> + T del over sgn u > 0
 __device__ __forceinline__ void half01(double U, double lam, double sgn, double &m0, double &td, double &m1) {
-  // erfc(x) = erfcx(|x|) exp(-x^2) for x >= 0 and 2 - erfcx(|x|) exp(-x^2) below,
-  // with the exponential that T del needs as well
-  const double rs = rsqrt(lam), x = -sgn * (lam * rs) * U, e = exp(-lam * U * U);
-  const double t = erfcx(fabs(x)) * e;
-  m0 = 0.5 * (x >= 0.0 ? t : 2.0 - t);
+  const double rs = rsqrt64(lam), y = lam * rs * U, x = sgn > 0.0 ? -y : y, e = exp64(-y * y);
+  if (((unsigned)__double2hiint(x) & 0x7fffffffu) < kErfcRange) {
+    m0 = half_erfc64(x);
+  } else {
+    // erfc(x) = erfcx(|x|) exp(-x^2) for x >= 0 and 2 - erfcx(|x|) exp(-x^2) below
+    const double t = erfcx(fabs(x)) * e;
+    m0 = 0.5 * (x >= 0.0 ? t : 2.0 - t);
+  }
   td = sgn * 0.28209479177387814347 * e * rs;          // 1 / (2 sqrt(pi))
   m1 = fma(U, m0, td);
 }
@@ -397,7 +404,7 @@ __device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
   Mom m;
   double td;
   half01(p.U, p.lam, sgn, m.m0, td, m.m1);
-  m.del = 2.0 * p.lam * td;
+  m.hd = p.lam * td;
   mom_up(p, m);
   return m;
 }
@@ -422,14 +429,14 @@ __device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
 //   psi_4 = psi'_4 + V psi'_2 + W psi'_3 + (V^2 + W^2)/2 psi'_0.
 struct Dir { double r, u, v, w, p; };    // drho, rho dU, rho dV, rho dW, dp along one axis of the face frame
 
-// out += L x (x in the tangential frame of p)
+// out += L x (x in the tangential frame of p, x[4] twice the component)
 __device__ __forceinline__ void acc_from_frame(const Prim &p, const double *x, double *out) {
-  const double h = 0.5 * fma(p.V, p.V, p.W * p.W);
+  const double q = fma(p.V, p.V, p.W * p.W);
   out[0] += x[0];
   out[1] += x[1];
-  out[2] += fma(p.V, x[0], x[2]);
-  out[3] += fma(p.W, x[0], x[3]);
-  out[4] += fma(p.V, x[2], fma(p.W, x[3], fma(h, x[0], x[4])));
+  out[2] = fma(p.V, x[0], out[2] + x[2]);
+  out[3] = fma(p.W, x[0], out[3] + x[3]);
+  out[4] = fma(p.V, x[2], fma(p.W, x[3], fma(0.5, fma(q, x[0], x[4]), out[4])));
 }
 
 // What the flux and the point values of one Maxwellian share: its convective and source
@@ -460,7 +467,7 @@ __device__ __forceinline__ Slopes slopes_of(const Prim &p, double g1, const Dir 
 // F += c rho <u psi> + e sum_d <u u_d d_d psi> + f <u d_t psi>
 __device__ __forceinline__ void acc_flux(const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
                                          double c, double e, double f, double *F) {
-  const double T = p.il, ef = e - f, hd = 0.5 * m.del;
+  const double T = p.il, ef = e - f, hd = m.hd;
   // the derivatives that come with one power of u: e conv + f d_t, and c rho in the density slot
   const double br = fma(c, p.rho, fma(ef, k.cr, -f * k.qr)), bu = fma(ef, k.cu, -f * k.qu);
   const double bv = fma(ef, k.cv, -f * k.qv), bw = fma(ef, k.cw, -f * k.qw), bs = fma(ef, k.cs, -f * k.qs);
@@ -479,32 +486,32 @@ __device__ __forceinline__ void acc_flux(const Prim &p, const Mom &m, const Dir 
   x[2] = fma(e, fma(d[0].v, m.m2, fma(T, Y1, k.s1 * m.m1)), bv * m.m1);
   x[3] = fma(e, fma(d[0].w, m.m2, fma(T, Z1, k.s2 * m.m1)), bw * m.m1);
   const double t4 = fma(K2, fma(T, E2, k.s0 * m.m2), E4);
-  x[4] = 0.5 * fma(e, fma(k.y, fma(K4 * T, m.m1, m.m3), t4), fma(K2, fma(T, B1, bs * m.m1), B3));
+  x[4] = fma(e, fma(k.y, fma(K4 * T, m.m1, m.m3), t4), fma(K2, fma(T, B1, bs * m.m1), B3));
   acc_from_frame(p, x, F);
 }
 
 // the moments sum_d <u_d d_d psi'> without the part of conv (u d_0, v' d_1, w' d_2)
 __device__ __forceinline__ void own_moments(const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
                                             double *z) {
-  const double T = p.il, hd = 0.5 * m.del, h0 = -p.lam * p.U * m.del;
+  const double T = p.il, hd = m.hd, del = 2.0 * hd, h0 = -p.lam * p.U * del;
   const double E1 = fma(d[0].r, m.m1, fma(d[0].u, m.m0, k.s0 * hd));
   const double E2 = fma(d[0].r, m.m2, fma(2.0 * d[0].u, m.m1, k.s0 * m.m0));
   const double E3 = fma(d[0].r, m.m3, 3.0 * fma(d[0].u, m.m2, k.s0 * m.m1));
-  const double Y0 = fma(d[1].r, m.m0, fma(d[1].u, m.del, k.s1 * h0));
-  const double Z0 = fma(d[2].r, m.m0, fma(d[2].u, m.del, k.s2 * h0));
+  const double Y0 = fma(d[1].r, m.m0, fma(d[1].u, del, k.s1 * h0));
+  const double Z0 = fma(d[2].r, m.m0, fma(d[2].u, del, k.s2 * h0));
   z[0] = fma(k.y, m.m0, E1);
   z[1] = fma(k.y, m.m1, E2);
   z[2] = fma(d[0].v, m.m1, fma(T, Y0, k.s1 * m.m0));
   z[3] = fma(d[0].w, m.m1, fma(T, Z0, k.s2 * m.m0));
-  z[4] = 0.5 * fma(k.y, fma(K4 * T, m.m0, m.m2), fma(K2, fma(T, E1, k.s0 * m.m1), E3));
+  z[4] = fma(k.y, fma(K4 * T, m.m0, m.m2), fma(K2, fma(T, E1, k.s0 * m.m1), E3));   // twice the component
 }
 // W += c rho <psi> + e sum_d <u_d d_d psi> + f <d_t psi>, z from own_moments
 __device__ __forceinline__ void acc_state(const Prim &p, const Mom &m, const Slopes &k, const double *z, double K2, double c,
                                           double e, double f, double *W) {
-  const double T = p.il, ef = e - f, hd = 0.5 * m.del, h0 = -p.lam * p.U * m.del;
+  const double T = p.il, ef = e - f, hd = m.hd, del = 2.0 * hd, h0 = -p.lam * p.U * del;
   const double br = fma(c, p.rho, fma(ef, k.cr, -f * k.qr)), bu = fma(ef, k.cu, -f * k.qu);
   const double bv = fma(ef, k.cv, -f * k.qv), bw = fma(ef, k.cw, -f * k.qw), bs = fma(ef, k.cs, -f * k.qs);
-  const double B0 = fma(br, m.m0, fma(bu, m.del, bs * h0));
+  const double B0 = fma(br, m.m0, fma(bu, del, bs * h0));
   const double B1 = fma(br, m.m1, fma(bu, m.m0, bs * hd));
   const double B2 = fma(br, m.m2, fma(2.0 * bu, m.m1, bs * m.m0));
   double x[5];
@@ -512,15 +519,14 @@ __device__ __forceinline__ void acc_state(const Prim &p, const Mom &m, const Slo
   x[1] = fma(e, z[1], B1);
   x[2] = fma(e, z[2], bv * m.m0);
   x[3] = fma(e, z[3], bw * m.m0);
-  x[4] = fma(e, z[4], 0.5 * fma(K2, fma(T, B0, bs * m.m0), B2));
+  x[4] = fma(e, z[4], fma(K2, fma(T, B0, bs * m.m0), B2));
   acc_from_frame(p, x, W);
 }
 
 // State outside a boundary face (face frame, x = outward normal), from the inner one: walls
 // mirror it in (p, U, V, W, T = p/rho), an isothermal wall's image with the density of zero
 // mass exchange; far field = free stream. M1: <u>_{u>0} of the inner state.
-__device__ void image_state(const hgks_params &P, int tag, const double *T, const Prim &l, double M1, bool held, double *Wr) {
-  const double g = P.gamma;
+__device__ void image_state(const KParams &P, int tag, const double *T, const Prim &l, double M1, bool held, double *Wr) {
   if (tag == HGKS_BC_FARFIELD) {
     double u[3];
 #pragma unroll
@@ -528,7 +534,7 @@ __device__ void image_state(const hgks_params &P, int tag, const double *T, cons
     Wr[0] = P.rho_inf;
 #pragma unroll
     for (int r = 0; r < 3; r++) Wr[1 + r] = P.rho_inf * u[r];
-    Wr[4] = P.p_inf / (g - 1.0) + 0.5 * P.rho_inf * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    Wr[4] = P.p_inf * P.ig1 + 0.5 * P.rho_inf * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     return;
   }
   const double u[3] = {l.U, l.V, l.W};
@@ -546,16 +552,16 @@ __device__ void image_state(const hgks_params &P, int tag, const double *T, cons
   double rg = l.rho;
   if (T_odd) {
     double m0, td, Mg;
-    half01(l.U, 0.5 / Tg, 1.0, m0, td, Mg);
-    rg = l.rho * M1 / Mg;
+    half01(l.U, 0.5 * rcp(Tg), 1.0, m0, td, Mg);
+    rg = l.rho * M1 * rcp(Mg);
   }
   Wr[0] = rg;
 #pragma unroll
   for (int r = 0; r < 3; r++) Wr[1 + r] = rg * ug[r];
-  Wr[4] = rg * Tg / (g - 1.0) + 0.5 * rg * (ug[0] * ug[0] + ug[1] * ug[1] + ug[2] * ug[2]);
+  Wr[4] = rg * Tg * P.ig1 + 0.5 * rg * (ug[0] * ug[0] + ug[1] * ug[1] + ug[2] * ug[2]);
 }
 // an isothermal image colder than T_w / 2 (a cell hotter than 1.5 T_w) is held at T_w / 2, uniform
-__device__ __forceinline__ bool image_held(const hgks_params &P, int tag, double Tl) {
+__device__ __forceinline__ bool image_held(const KParams &P, int tag, double Tl) {
   return (tag == HGKS_BC_WALL_ISO || tag == HGKS_BC_WALL_LID) && 2.0 * P.wall_T - Tl < 0.5 * P.wall_T;
 }
 // the image's derivatives from the inner ones, in place: quantities even under the mirror
@@ -583,21 +589,15 @@ __device__ __forceinline__ void image_slopes(int tag, const Prim &l, const Prim 
   }
 }
 
-// rho > 0 and p > 0, the latter as rho p > 0 (no division)
-__device__ __forceinline__ bool physical(const double *W, double gamma) {
-  const double rp = (gamma - 1.0) * (W[4] * W[0] - 0.5 * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3]));
-  return W[0] > 0.0 && rp > 0.0;
-}
-
 // Derivatives of side s (a Maxwellian with primitive state p) at one Gauss point, from the
 // reconstruction's derivatives `in` (15 rows of pitch F). In characteristic variables
 // R* q back-projects to conservative derivatives, whose primitive form with respect to the
 // side's own state follows directly: with (du, dv, dw) = u* - (U, V, W) and c* the sound
 // speed of the projection state, dp = (gamma - 1)(dE - u . dm + |u|^2/2 drho) takes five
 // products instead of the fourteen of R* and nine of the change of variables.
-__device__ __forceinline__ void load_dirs(const hgks_params &P, const Eig &e, const double *T, const Prim &p,
+__device__ __forceinline__ void load_dirs(const KParams &P, const Eig &e, const double *T, const Prim &p,
                                           const double *__restrict__ in, size_t F, Dir *d) {
-  const double g1 = P.gamma - 1.0;
+  const double g1 = P.g1;
   if (P.characteristic) {
     const double du = e.u - p.U, dv = e.v - p.V, dw = e.w - p.W;
     const double gu = g1 * du, gv = g1 * dv, gw = g1 * dw, h = 0.5 * fma(gu, du, fma(gv, dv, gw * dw)), a2 = e.a * e.a;
@@ -637,9 +637,10 @@ __device__ __forceinline__ void load_dirs(const hgks_params &P, const Eig &e, co
 // by dt throughout so that the time average needs no division of its own; the derivatives
 // are read where they are used, so one side's fifteen are live at a time. Against slopes
 // solved for each axis and summed with moments up to u^6: 37.5 -> 24.5 ms at 14.2M Gauss
-// points (inviscid, 2,359,296 tetrahedra), 1.22 -> 0.79 ms at 295k (viscous, compact scheme).
+// points (inviscid, 2,359,296 tetrahedra), 1.22 -> 0.74 ms at 295k (viscous, compact scheme);
+// with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms.
 template <bool BATCH, class S, bool COMPACT>
-__global__ void __launch_bounds__(256) k_flux(DevMesh m, hgks_params Pv, const double *__restrict__ Q,
+__global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                   const double *__restrict__ dt, const double *__restrict__ wface,
                                                   double *__restrict__ fflux, double *__restrict__ fpt, int *__restrict__ flags) {
   constexpr int NG = S::NG;
@@ -650,13 +651,13 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, hgks_params Pv, const d
   const int g = blockIdx.x % NG, f = (blockIdx.x / NG) * blockDim.x + threadIdx.x;
   if (f >= FL) return;
   if (BATCH && !m.mact[m.fmesh[f]]) return;             // a mesh of a batch that has stopped
-  const hgks_params &P = BATCH ? m.ptab[m.fmesh[f]] : Pv;
+  const KParams &P = BATCH ? m.ptab[m.fmesh[f]] : Pv;
   double T[9];
 #pragma unroll
   for (int k = 0; k < 9; k++) T[k] = m.fT[(size_t)k * F + f];
   const int L = m.fl[f], R = m.fr[f];
   const bool inner = R >= 0;
-  const double gam = P.gamma, g1 = gam - 1.0, ig1 = 1.0 / g1, K2 = (3.0 - gam) * ig1, K4 = (gam + 1.0) * ig1;
+  const double g1 = P.g1, K2 = P.K2, K4 = P.K4;
   Prim pl, pr;
   Mom ml, mr;
   Eig e;
@@ -671,52 +672,56 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, hgks_params Pv, const d
       Qs[c] = inner ? 0.5 * (QL[c] + QR[c]) : QL[c];
     }
     rot_in(T, Qs, Qsl);
-    e = eig_of(Qsl, gam);
+    e = eig_of(Qsl, P.gamma, g1);
     auto side = [&](int s, const double *Qc) {
       const double *in = wface + ((size_t)(s * NG + g) * kFaceState) * F + f;
 #pragma unroll
       for (int c = 0; c < 5; c++) q[c] = in[(size_t)c * F];
       if (P.characteristic) right_apply(e, q, W);
       else rot_in(T, q, W);
-      if (!physical(W, gam)) {
+      double rp = rho_p(W, g1);
+      if (!positive(W[0]) || !positive(rp)) {
         rot_in(T, Qc, W);
+        rp = rho_p(W, g1);
         bad |= 1 << s;
       }
+      return rp;
     };
-    side(0, QL);
-    pl = to_prim(W, gam);
+    double rp = side(0, QL);
+    pl = to_prim(W, rp);
     ml = mom_half(pl, 1.0);
     if (inner) {
-      side(1, QR);
+      rp = side(1, QR);
     } else {
       held = image_held(P, m.ftag[f], pl.il);
       image_state(P, m.ftag[f], T, pl, ml.m1, held, W);
+      rp = rho_p(W, g1);
     }
-    pr = to_prim(W, gam);
+    pr = to_prim(W, rp);
     mr = mom_half(pr, -1.0);
   }
   // compatibility condition: Q0 = int_{u>0} psi g_l + int_{u<0} psi g_r
   Prim p0;
   {
     double Q0[5] = {0, 0, 0, 0, 0};
-    const double xl[5] = {pl.rho * ml.m0, pl.rho * ml.m1, 0.0, 0.0, 0.5 * pl.rho * fma(K2 * pl.il, ml.m0, ml.m2)};
-    const double xr[5] = {pr.rho * mr.m0, pr.rho * mr.m1, 0.0, 0.0, 0.5 * pr.rho * fma(K2 * pr.il, mr.m0, mr.m2)};
+    const double xl[5] = {pl.rho * ml.m0, pl.rho * ml.m1, 0.0, 0.0, pl.rho * fma(K2 * pl.il, ml.m0, ml.m2)};
+    const double xr[5] = {pr.rho * mr.m0, pr.rho * mr.m1, 0.0, 0.0, pr.rho * fma(K2 * pr.il, mr.m0, mr.m2)};
     acc_from_frame(pl, xl, Q0);
     acc_from_frame(pr, xr, Q0);
-    p0 = to_prim(Q0, gam);
+    p0 = to_prim(Q0, rho_p(Q0, g1));
   }
   double dtf;
-  if (P.flux_dt > 0.0) dtf = P.flux_dt;
-  else dtf = (inner ? fmin(dt[L], dt[R]) : dt[L]) * (P.flux_cfl / P.cfl);
+  if (positive(P.flux_dt)) dtf = P.flux_dt;
+  else dtf = (inner ? min_positive(dt[L], dt[R]) : dt[L]) * P.flux_dt_ratio;
   // collision time (Sec. 5) over dt, and the time coefficients of Eq. (flux) over dt
   const double prl = pl.rho * pl.il, prr = pr.rho * pr.il, pp0 = p0.rho * p0.il;
-  const double jump = fabs((prl - prr) / (prl + prr));
-  const double tq = P.viscous ? P.mu / (pp0 * dtf) + P.tau_C * jump : P.tau_eps + P.tau_C * jump;   // tau / dt
-  const double eta = exp(-1.0 / tq);
+  const double jump = fabs((prl - prr) * rcp(prl + prr));
+  const double tq = fma(P.tau_C, jump, P.viscous ? P.mu * rcp(pp0 * dtf) : P.tau_eps);   // tau / dt
+  const double eta = exp64(-rcp(tq));
   const double c4 = tq * (1.0 - eta), k4 = tq * c4, tau = tq * dtf;
   const double c1 = 1.0 - c4, c2 = dtf * (2.0 * k4 - tq * (1.0 + eta)), c3 = dtf * (0.5 - tq + k4);
   const double c5 = dtf * (2.0 * k4 - tq * eta);
-  const bool prandtl = P.Pr != 1.0;
+  const bool prandtl = P.fix_prandtl;
   const double ts = P.tstar_end ? dtf : 0.0, es = P.tstar_end ? eta : 1.0;   // exp(-t* / tau)
   double Fl[5] = {0, 0, 0, 0, 0}, Wb[5] = {0, 0, 0, 0, 0}, Pt[5] = {0, 0, 0, 0, 0};
   // derivatives of g_0: the mean of both sides' conservative derivatives, taken with
@@ -774,7 +779,7 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, hgks_params Pv, const d
     const double U = p0.U, V = p0.V, W = p0.W, q2 = U * U + V * V + W * W;
     const double q = Fl[4] - (U * Fl[1] + V * Fl[2] + W * Fl[3]) + 0.5 * q2 * Fl[0] - U * Wb[4] +
                      U * (U * Wb[1] + V * Wb[2] + W * Wb[3]) - 0.5 * U * q2 * Wb[0];
-    Fl[4] += (1.0 / P.Pr - 1.0) * q;
+    Fl[4] += P.prandtl * q;
   }
   // walls are impermeable: their faces carry momentum and energy, no mass
   if (!inner && m.ftag[f] >= HGKS_BC_WALL_ISO && m.ftag[f] <= HGKS_BC_NOSLIP_ADIA) Fl[0] = 0.0;
@@ -851,20 +856,20 @@ __global__ void __launch_bounds__(kBlock) k_gather(DevMesh m, int compact, const
 }
 
 template <bool BATCH, class S>
-__global__ void k_local_dt(DevMesh m, hgks_params Pv, const double *__restrict__ Q, double *__restrict__ dt) {
+__global__ void k_local_dt(DevMesh m, KParams Pv, const double *__restrict__ Q, double *__restrict__ dt) {
   const int N = m.N, F = m.F;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   if (BATCH && m.cmesh[i] < 0) { dt[i] = 1.0; return; }   // padding cell of a batch
   if (BATCH && !m.mact[m.cmesh[i]]) return;
-  const hgks_params &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
+  const KParams &P = BATCH ? m.ptab[m.cmesh[i]] : Pv;
   double q[5];
 #pragma unroll
   for (int c = 0; c < 5; c++) q[c] = Q[(size_t)c * N + i];
-  const double ir = 1.0 / q[0], u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
-  const double p = (P.gamma - 1.0) * (q[4] - 0.5 * q[0] * (u * u + v * v + w * w));
-  const double a = sqrt(P.gamma * p * ir);
-  const double nu = P.viscous ? 2.0 * P.gamma * P.mu / (P.Pr * q[0] * m.h[i]) : 0.0;
+  const double ir = rcp(q[0]), u = q[1] * ir, v = q[2] * ir, w = q[3] * ir;
+  const double p = P.g1 * (q[4] - 0.5 * q[0] * (u * u + v * v + w * w));
+  const double a = sqrt64(P.gamma * p * ir);
+  const double nu = P.viscous ? 2.0 * P.gamma * P.mu * rcp(P.Pr * q[0] * m.h[i]) : 0.0;
   double s = 0.0;
 #pragma unroll
   for (int k = 0; k < S::NF; k++) {
@@ -872,7 +877,7 @@ __global__ void k_local_dt(DevMesh m, hgks_params Pv, const double *__restrict__
     const double un = u * m.fT[f] + v * m.fT[(size_t)F + f] + w * m.fT[(size_t)2 * F + f];
     s += m.fS[f] * (fabs(un) + a + nu);
   }
-  dt[i] = P.cfl * m.vol[i] / s;
+  dt[i] = P.cfl * m.vol[i] * rcp(s);
 }
 
 }  // namespace
@@ -910,7 +915,8 @@ void launch_wall_force(const DevMesh &m, const Scratch &s, int tag, double *forc
   HGKS_PROF_END(K_NORM, st);
 }
 
-void launch_local_dt(const DevMesh &m, const hgks_params &p, const double *Q, double *dt, cudaStream_t st) {
+void launch_local_dt(const DevMesh &m, const hgks_params &hp, const double *Q, double *dt, cudaStream_t st) {
+  const KParams p = kernel_params(hp);
   HGKS_PROF_BEGIN(K_DT, st);
   if (m.ptab && m.hex) k_local_dt<true, HexShape><<<grid_for(m.NL, kBlock), kBlock, 0, st>>>(m, p, Q, dt);
   else if (m.ptab) k_local_dt<true, TetShape><<<grid_for(m.NL, kBlock), kBlock, 0, st>>>(m, p, Q, dt);
@@ -922,8 +928,9 @@ void launch_local_dt(const DevMesh &m, const hgks_params &p, const double *Q, do
 namespace {
 // the four residual kernels of one cell kind
 template <bool BATCH, class S>
-void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *G, double *R,
+void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const double *Q, const double *G, double *R,
                       double *Gnew, cudaStream_t st) {
+  const KParams p = kernel_params(hp);
   const int64_t NL = BATCH ? m.NL : m.N, FL = BATCH ? m.FL : m.F;
   HGKS_PROF_BEGIN(K_COEF, st);
   const unsigned gc = grid_for(5 * NL, kBlock);
