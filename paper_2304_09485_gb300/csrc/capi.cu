@@ -566,17 +566,18 @@ static hgks_status gmres_step_impl(Mesh &m, const hgks_params *p, double *Q, dou
   const int mk = p->krylov_dim;
   HGKS_CUDA(cudaMemcpyAsync(host, res_dev, sizeof(double), cudaMemcpyDeviceToHost, st_));
   HGKS_CUDA(cudaMemcpyAsync(host + 1, s.hs + (mk + 1) * mk + 1 + mk, 2 * sizeof(double), cudaMemcpyDeviceToHost, st_));
-  int nonphys = 0;
-  HGKS_CUDA(cudaMemcpyAsync(&nonphys, s.flags, sizeof(int), cudaMemcpyDeviceToHost, st_));
-  HGKS_CUDA(cudaMemsetAsync(s.flags, 0, sizeof(int), st_));
+  int flags[2] = {0, 0};               // non-physical states, a grid barrier that gave up
+  HGKS_CUDA(cudaMemcpyAsync(flags, s.flags, sizeof(flags), cudaMemcpyDeviceToHost, st_));
+  HGKS_CUDA(cudaMemsetAsync(s.flags, 0, sizeof(flags), st_));
   HGKS_CUDA(cudaStreamSynchronize(st_));
   const double res = host[0] / (double)m.N;
   if (info) {
     info->res_l1 = res;
     info->lin_res[0] = host[1];
     info->lin_res[1] = host[2];
-    info->nonphysical = nonphys;
+    info->nonphysical = flags[0];
   }
+  if (flags[1]) return fail(HGKS_ERR_CUDA, "a grid barrier of the GMRES solve timed out");
   if (!std::isfinite(res)) return fail(HGKS_ERR_NONPHYSICAL, "non-finite residual");
   return HGKS_OK;
 }

@@ -1,5 +1,6 @@
 // FP64 GMRES of one mesh with the assembled A: the Krylov products on vectors in the
-// form of offdiag.cuh and modified Gram-Schmidt by blocks of basis vectors.
+// form of offdiag.cuh, modified Gram-Schmidt by blocks of basis vectors, and, for
+// meshes small enough, all restart cycles in one cooperative launch.
 //
 // Modified Gram-Schmidt by blocks. Algorithm 1 takes h_i = (w_i, v_i), w_{i+1} = w_i - h_i v_i
 // one vector after the other. For the vectors v_c ... of a block with w_c given,
@@ -8,6 +9,7 @@
 // known. Those of a new v_{j+1} = w / ||w|| with the earlier members of its block come with
 // ||w|| in the last pass of step j, whose subtracted vectors they are.
 #include <algorithm>
+#include <cmath>
 #include "hgks_internal.h"
 #include "fp64.cuh"
 #include "offdiag.cuh"
@@ -18,7 +20,7 @@ namespace {
 
 constexpr int kCell = 128;      // threads of the cell kernels
 constexpr int kVec = 256;       // threads of the vector kernels
-constexpr int kRed = 152 * 4;   // blocks of the vector kernels
+constexpr int kRed = 152 * 3;   // blocks of the vector kernels: those resident at 80 registers
 constexpr int kBlk = 4;         // basis vectors of a block (separate launches)
 
 // Reduction over the grid: the last block to arrive adds the blocks' partials in block
@@ -75,7 +77,7 @@ __global__ void __launch_bounds__(kCell) k_scale_z(int N, const double *__restri
     y[c] = w[(size_t)c * N + i] * ih;
     v[(size_t)c * N + i] = y[c];
   }
-  z_of(jv, N, i, y, z);
+  z_of(cell_prim(jv, N, i), y, z);
   z_store(zv, N, i, z);
 }
 
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(kCell) k_zprod(int N, const int *__restrict__ 
   const double d = sign * dinv[i];
 #pragma unroll
   for (int c = 0; c < 5; c++) acc[c] *= d;
-  z_of(jv, N, i, acc, z);
+  z_of(cell_prim(jv, N, i), acc, z);
   z_store(y, N, i, z);
 }
 
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(kCell) k_zlast(int N, const int *__restrict__ 
 // vector, thread and step, every load of the step first. (2 + NB + ND) x 8 bytes and NB + ND
 // FMAs per element: with NB = ND = 4 the FP64 rate (2 DFMA per SM and clock) and HBM are near balance.
 template <int NB, int ND, bool FIN>
-__global__ void __launch_bounds__(kVec) k_mgs_block(int64_t n, double *__restrict__ w, const double *__restrict__ V,
+__global__ void __launch_bounds__(kVec, 3) k_mgs_block(int64_t n, double *__restrict__ w, const double *__restrict__ V,
                                                     int64_t vs, int a, int c, int j, int mk, double *G, double *Hj,
                                                     double *partials, unsigned *count) {
   constexpr int NG = FIN ? (NB < kBlk ? NB : 0) : ND;   // products besides ||w||^2
@@ -223,6 +225,435 @@ void zlast(cudaStream_t st, const DevMesh &m, const Scratch &s, const double *x,
 #undef HGKS_ZL
 }
 
+
+// ---- all restart cycles in one cooperative launch ----
+// A cycle in separate launches is a chain of some 200 dependent ones, 4 to 9 microseconds each on
+// a small mesh: launch gaps, block scheduling, tails of the reductions and of the FP64-bound
+// kernels. Here one block per SM keeps its cells for the whole solve: w stays in registers (or
+// shared memory), the basis is only touched by the thread that wrote it, and blocks meet at a
+// grid barrier (1.1 us) where neighbours' vectors or sums are needed: one per product, one per
+// block of kPB basis vectors, one for the norm (z(w) is written before it, unscaled, so the next
+// product starts right after). Every block adds the blocks' partial sums itself, in the same
+// order, so all of them hold the same H; an extra warp turns its columns into R while the others
+// form the next product.
+// An SM sub-partition takes 64 clocks per FP64 warp instruction, however few lanes are active and
+// also when its predicate is false. So below one warp of cells per sub-partition LPC = 2 or 4
+// lanes share a cell (its faces in the products, its components elsewhere), and the loops over a
+// partial block of basis vectors have exact trip counts.
+// Per step outside the residual, separate launches against this one: 3,072 tetrahedra 1.40 /
+// 0.68 ms, 48,000 2.16 / 1.46, 124,416 (20 vectors) 8.31 / 7.36, 110,592 hexahedra 4.15 / 3.32.
+constexpr int kPT = 384;        // threads with cells, three warps per SM sub-partition (and a warp for the rotations)
+constexpr int kPB = 8;          // basis vectors of a block (one grid barrier each)
+constexpr int kPG = 160;        // blocks at most (the sums read one partial per block)
+constexpr int kPMax = 64;       // Krylov vectors at most
+// Cells at most. Whole steps, one launch against separate ones: 343,332 tetrahedra 23.7 / 25.3 ms,
+// 576,000 39.0 / 39.9; beyond 700,000 w no longer fits shared memory, and with w in global memory
+// 766,656 take 53.3 / 52.3, 2,359,296 159 / 153.
+constexpr int kGridCells = 600000;
+constexpr unsigned kSpin = 1u << 22;   // polls of a barrier (a second or more) before it gives up
+
+struct GridSolve {
+  int N, C;                     // cells, cells per block
+  const int *cnb;
+  const double *jv, *dval, *dinv, *rhs;
+  double *dx, *b, *V, *z0, *z1, *part, *lres;
+  int64_t vs;
+  unsigned *bar;                // arrivals, 0 at launch
+  int *err;                     // set to 1 by a barrier that gave up
+  int mk, restarts, sweeps;
+};
+
+// shared memory of a block
+struct GridShared {
+  double H[(kPMax + 1) * kPMax], G[(kPMax + 1) * kPB], cs[kPMax], sn[kPMax], gv[kPMax + 1], y[kPMax];
+  double sh[kPT / 32][kPB], sum[kPB], nrm, inrm;
+  int used, dead;
+};
+
+// The arrival of every block at step `gen` (1, 2, ...). false: given up, the block returns.
+__device__ __forceinline__ bool grid_barrier(const GridSolve &a, GridShared &S, unsigned &gen) {
+  const unsigned want = ++gen * gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
+    unsigned seen, spin = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
+    } while (seen < want && ++spin < kSpin);
+    if (seen < want) {
+      S.dead = 1;
+      atomicExch(a.err, 1);
+    }
+  }
+  __syncthreads();
+  return S.dead == 0;
+}
+
+// the sums over the grid of the first `ns` of kPB values per thread, in S.sum (all threads);
+// S.nrm and S.inrm: the root of sum `norm` and its reciprocal (0 for 0)
+__device__ __forceinline__ bool grid_total(const GridSolve &a, GridShared &S, unsigned &gen, double *v, int ns, int nwarps,
+                                           int norm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < nwarps) {
+    const double t = warp_sums<kPB>(v);
+    if (lane % (32 / kPB) == 0) S.sh[warp][lane / (32 / kPB)] = t;
+  }
+  __syncthreads();
+  double *part = a.part + (gen & 1) * (kPB * kPG);     // two sets: a slow block may still read the last one
+  if (threadIdx.x < ns) {
+    double s = S.sh[0][threadIdx.x];
+    for (int w = 1; w < nwarps; w++) s += S.sh[w][threadIdx.x];
+    part[threadIdx.x * kPG + blockIdx.x] = s;
+  }
+  if (!grid_barrier(a, S, gen)) return false;
+  if (warp < ns) {
+    double t[5], s;
+#pragma unroll
+    for (int k = 0; k < 5; k++) t[k] = lane + 32 * k < gridDim.x ? __ldcg(part + warp * kPG + lane + 32 * k) : 0.0;
+    s = t[0];
+#pragma unroll
+    for (int k = 1; k < 5; k++)
+      if (32 * k < gridDim.x) s += t[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      S.sum[warp] = s;
+      if (warp == norm) {
+        const double r = sqrt64(s);
+        S.nrm = r;
+        S.inrm = r != 0.0 ? rcp(r) : 0.0;
+      }
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
+// column j of H: the earlier rotations, its own, and the right-hand side (one thread; as givens_lsq)
+__device__ __forceinline__ void givens_column(GridShared &S, int mk, int j) {
+  if (S.used < j) return;                               // a breakdown ended the basis before
+  double h1 = S.H[j];
+  for (int i = 0; i < j; i++) {
+    const double h2 = S.H[(i + 1) * mk + j];
+    S.H[i * mk + j] = S.cs[i] * h1 + S.sn[i] * h2;
+    h1 = S.cs[i] * h2 - S.sn[i] * h1;
+  }
+  const double b = S.H[(j + 1) * mk + j], r = rsqrt64(h1 * h1 + b * b), c = h1 * r, s = b * r;
+  S.cs[j] = c;
+  S.sn[j] = s;
+  S.H[j * mk + j] = c * h1 + s * b;
+  const double g1 = S.gv[j];
+  S.gv[j] = c * g1;
+  S.gv[j + 1] = -s * g1;
+  S.used = b == 0.0 ? -(j + 1) : j + 1;                 // negative: the basis ends here
+}
+
+// f(n) with the count as a constant, for n in 1..kPB: a predicated FP64 instruction costs as much as
+// an executed one, so the loops over a partial block have exact trip counts
+template <int n> struct Count { static constexpr int value = n; };
+template <class F>
+__device__ __forceinline__ void with_count(int n, F f) {
+  switch (n) {
+    case 1: f(Count<1>{}); break;
+    case 2: f(Count<2>{}); break;
+    case 3: f(Count<3>{}); break;
+    case 4: f(Count<4>{}); break;
+    case 5: f(Count<5>{}); break;
+    case 6: f(Count<6>{}); break;
+    case 7: f(Count<7>{}); break;
+    case 8: f(Count<8>{}); break;
+    default: break;
+  }
+}
+
+// the sums over a cell's LPC lanes of acc[5], each lane keeping its components l, l + LPC, ...
+template <int LPC>
+__device__ __forceinline__ void lane_components(const double *acc, double *own) {
+  const int l = threadIdx.x % LPC;
+  auto swap = [&](bool up, double lo, double hi, int o) {   // up lanes keep hi, the others lo
+    return (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+  };
+  if constexpr (LPC == 1) {
+#pragma unroll
+    for (int c = 0; c < 5; c++) own[c] = acc[c];
+  } else if constexpr (LPC == 2) {
+    own[0] = swap(l, acc[0], acc[1], 1);
+    own[1] = swap(l, acc[2], acc[3], 1);
+    own[2] = swap(l, acc[4], 0.0, 1);
+  } else {
+    const double t0 = swap(l >> 1, acc[0], acc[2], 2), t1 = swap(l >> 1, acc[1], acc[3], 2), t2 = swap(l >> 1, acc[4], 0.0, 2);
+    own[0] = swap(l & 1, t0, t1, 1);
+    own[1] = swap(l & 1, t2, 0.0, 1);
+  }
+}
+
+// ONE: a thread has one cell at most (and LPC lanes share it), with what it reads of it in
+// registers; otherwise its cells' w live in shared memory and it goes through them in turn.
+template <int NF, int LPC, bool ONE>
+__global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
+  constexpr int CP = (5 + LPC - 1) / LPC;               // components per lane: l, l + LPC, ...
+  constexpr int LF = (NF + LPC - 1) / LPC;              // faces per lane, alike
+  static_assert(ONE || LPC == 1, "several cells per thread: whole cells");
+  extern __shared__ __align__(16) unsigned char smem[];
+  GridShared &S = *reinterpret_cast<GridShared *>(smem);
+  double *ws = reinterpret_cast<double *>(smem + sizeof(GridShared));   // !ONE: [5][C]
+  const int tid = threadIdx.x, mk = a.mk, l = tid % LPC;
+  const size_t N = a.N;
+  const int c0 = blockIdx.x * a.C, nc = min(a.C, a.N - c0);             // this block's cells (nc <= 0: none)
+  const int nwarps = min(kPT / 32, (a.C * LPC + 31) / 32);
+  const bool rot = tid == kPT;                          // the thread of the rotations
+  // a load after a barrier goes to L2: keep what every phase reads of the cell
+  const int own_cell = tid < kPT && tid / LPC < nc ? c0 + tid / LPC : -1;
+  int own_nb[LF];
+  CellPrim own_prim = {0, 0, 0, 0, 0, 0};
+  double own_w[CP], own_dinv = 0.0;
+#pragma unroll
+  for (int k = 0; k < CP; k++) own_w[k] = 0.0;
+  if (ONE) {
+#pragma unroll
+    for (int q = 0; q < LF; q++)
+      own_nb[q] = own_cell >= 0 && q * LPC + l < NF ? a.cnb[(q * LPC + l) * N + own_cell] : -1;
+    if (own_cell >= 0) {
+      own_prim = cell_prim(a.jv, N, own_cell);
+      own_dinv = a.dinv[own_cell];
+    }
+  }
+  // f(i, w) for every cell i of the thread and its components of w (ONE: also for none, i = -1,
+  // so that all lanes of a warp reach the exchanges inside)
+  auto each = [&](auto f) {
+    if constexpr (ONE) {
+      f(own_cell, own_w);
+    } else {
+      for (int r = tid; r < nc && tid < kPT; r += kPT) {
+        double w[CP];
+#pragma unroll
+        for (int k = 0; k < CP; k++) w[k] = ws[k * a.C + r];
+        f(c0 + r, w);
+#pragma unroll
+        for (int k = 0; k < CP; k++) ws[k * a.C + r] = w[k];
+      }
+    }
+  };
+  // component k of a lane: whether it has one, and its element
+  auto mine = [&](int i, int k) { return (!ONE || i >= 0) && l + LPC * k < 5; };
+  auto at = [&](int i, int k) { return (l + LPC * k) * N + i; };
+  auto dinv = [&](int i) { return ONE ? own_dinv : a.dinv[i]; };
+  // this lane's components of sum_p A_ip x_p
+  auto off = [&](int i, const double *z, double *acc) {
+    double t[5] = {0, 0, 0, 0, 0};
+    int nb[LF];
+#pragma unroll
+    for (int q = 0; q < LF; q++) nb[q] = ONE ? own_nb[q] : a.cnb[q * N + i];
+#pragma unroll
+    for (int q = 0; q < LF; q++)
+      if (nb[q] >= 0) z_product(a.jv, N, i, q * LPC + l, nb[q], z, t);
+    lane_components<LPC>(t, acc);
+  };
+  // z form of a cell's vector from its lanes' components
+  auto put_z = [&](double *z, int i, const double *x) {
+    double y[5], t[6];
+#pragma unroll
+    for (int c = 0; c < 5; c++)
+      y[c] = LPC == 1 ? x[c] : __shfl_sync(0xffffffffu, x[c / LPC], (tid & 31 & ~(LPC - 1)) | (c % LPC));
+    if (ONE && i < 0) return;
+    z_of(ONE ? own_prim : cell_prim(a.jv, N, i), y, t);
+#pragma unroll
+    for (int k = 0; k < 6; k++)
+      if (LPC == 1 || k % LPC == l) z[k * N + i] = t[k];
+  };
+  unsigned gen = 0;
+  if (tid == 0) S.dead = 0;
+  double *zs = a.z0, *zd = a.z1;                        // the vector to multiply, and the other buffer
+  auto flip = [&] { double *t = zs; zs = zd; zd = t; };
+  for (int it = 0; it < a.restarts; it++) {
+    // w = P^{-1} (rhs - A dx), b kept for the sweeps
+    if (it > 0) {
+      each([&](int i, double *) {
+        double x[CP];
+#pragma unroll
+        for (int k = 0; k < CP; k++) x[k] = mine(i, k) ? a.dx[at(i, k)] : 0.0;
+        put_z(zs, i, x);
+      });
+      if (!grid_barrier(a, S, gen)) return;
+    }
+    each([&](int i, double *w) {
+      double acc[CP];
+      if (it > 0) off(i, zs, acc);
+#pragma unroll
+      for (int k = 0; k < CP; k++)
+        if (mine(i, k)) {
+          double b = a.rhs[at(i, k)];
+          if (it > 0) b -= fma(a.dval[i], a.dx[at(i, k)], acc[k]);
+          else a.dx[at(i, k)] = 0.0;
+          a.b[at(i, k)] = b;
+          w[k] = dinv(i) * b;
+        }
+      put_z(zd, i, w);
+    });
+    for (int q = 0; q < a.sweeps; q++) {
+      if (!grid_barrier(a, S, gen)) return;
+      flip();
+      each([&](int i, double *w) {
+        double acc[CP];
+        off(i, zs, acc);
+#pragma unroll
+        for (int k = 0; k < CP; k++)
+          if (mine(i, k)) w[k] = dinv(i) * (a.b[at(i, k)] - acc[k]);
+        put_z(zd, i, w);
+      });
+    }
+    double s[kPB];
+#pragma unroll
+    for (int q = 0; q < kPB; q++) s[q] = 0.0;
+    each([&](int i, double *w) {
+#pragma unroll
+      for (int k = 0; k < CP; k++)
+        if (mine(i, k)) s[0] = fma(w[k], w[k], s[0]);
+    });
+    if (!grid_total(a, S, gen, s, 1, nwarps, 0)) return;
+    flip();                                             // zs = z(w), unscaled
+    const double beta = S.nrm;
+    double ih = S.inrm;
+    if (rot) {
+      S.used = 0;
+      S.gv[0] = beta;
+      if (it == 0 && blockIdx.x == 0) a.lres[0] = beta;
+    }
+    for (int j = 0; j < mk; j++) {
+      // v_j = w / ||w||; w = v_j + E (-E)^sweeps v_j from z(w) and the scale
+      if (rot && j > 0) givens_column(S, mk, j - 1);
+      each([&](int i, double *w) {
+#pragma unroll
+        for (int k = 0; k < CP; k++)
+          if (mine(i, k)) {
+            w[k] *= ih;
+            a.V[(size_t)j * a.vs + at(i, k)] = w[k];
+          }
+      });
+      double sc = ih;
+      for (int q = 0; q < a.sweeps; q++) {
+        if (q == 0 && a.sweeps % 2 == 1) sc = -sc;
+        each([&](int i, double *) {
+          double acc[CP];
+          off(i, zs, acc);
+          const double d = q == 0 ? sc * dinv(i) : dinv(i);
+#pragma unroll
+          for (int k = 0; k < CP; k++) acc[k] *= d;
+          put_z(zd, i, acc);
+        });
+        if (!grid_barrier(a, S, gen)) return;
+        flip();
+      }
+      each([&](int i, double *w) {
+        double acc[CP];
+        off(i, zs, acc);
+        const double d = a.sweeps == 0 ? sc * dinv(i) : dinv(i);
+#pragma unroll
+        for (int k = 0; k < CP; k++)
+          if (mine(i, k)) w[k] = fma(d, acc[k], w[k]);
+      });
+      for (int p = 0;; p += kPB) {                      // p: the block whose coefficients are taken
+        const bool fin = p > j;
+        const int ns = p == 0 ? 0 : min(kPB, j + 1 - (p - kPB)), nd = fin ? 0 : min(kPB, j + 1 - p);
+        const bool gram = fin && ns < kPB;              // v_{j+1} joins the last block
+#pragma unroll
+        for (int q = 0; q < kPB; q++) s[q] = 0.0;
+        with_count(ns, [&](auto count) {                // subtract the previous block
+          constexpr int n = decltype(count)::value;
+          const double *h = S.H + (p - kPB) * mk + j;
+          each([&](int i, double *w) {
+#pragma unroll
+            for (int k = 0; k < CP; k++) {
+              if (!mine(i, k)) continue;
+              const double *v = a.V + (int64_t)(p - kPB) * a.vs + at(i, k);
+              double t[n], x = w[k];
+#pragma unroll
+              for (int q = 0; q < n; q++) t[q] = v[q * a.vs];
+#pragma unroll
+              for (int q = 0; q < n; q++) x = fma(-h[q * mk], t[q], x);
+              w[k] = x;
+              if constexpr (n < kPB)
+                if (gram)
+#pragma unroll
+                  for (int q = 0; q < n; q++) s[q] = fma(x, t[q], s[q]);
+            }
+          });
+        });
+        with_count(nd, [&](auto count) {                // the next one's products
+          constexpr int n = decltype(count)::value;
+          each([&](int i, double *w) {
+#pragma unroll
+            for (int k = 0; k < CP; k++) {
+              if (!mine(i, k)) continue;
+              const double *v = a.V + (int64_t)p * a.vs + at(i, k);
+#pragma unroll
+              for (int q = 0; q < n; q++) s[q] = fma(w[k], v[q * a.vs], s[q]);
+            }
+          });
+        });
+        if (fin)
+          each([&](int i, double *w) {
+#pragma unroll
+            for (int k = 0; k < CP; k++)
+              if (mine(i, k)) s[kPB - 1] = fma(w[k], w[k], s[kPB - 1]);
+            put_z(zd, i, w);
+          });
+        if (!grid_total(a, S, gen, s, fin ? kPB : nd, nwarps, fin ? kPB - 1 : -1)) return;
+        if (fin) {
+          ih = S.inrm;
+          if (tid >= kPT) {                             // the warp that reads column j next
+            if (rot) S.H[(j + 1) * mk + j] = S.nrm;
+            if (gram && tid - kPT < ns) S.G[(j + 1) * kPB + tid - kPT] = S.sum[tid - kPT] * ih;
+          }
+          break;
+        }
+        if (tid < 32) {                                 // h by forward substitution, a lane per coefficient
+          double h = tid < nd ? S.sum[tid] : 0.0;
+          for (int k = 0; k < nd - 1; k++) {
+            const double hk = __shfl_sync(0xffffffffu, h, k);
+            if (tid > k && tid < nd) h = fma(-hk, S.G[(p + tid) * kPB + k], h);
+          }
+          if (tid < nd) S.H[(p + tid) * mk + j] = h;
+        }
+        __syncthreads();
+      }
+      flip();
+    }
+    __syncthreads();
+    if (tid >= kPT) {                                   // the last column, then back substitution by the warp
+      const int lane = tid - kPT;
+      if (lane == 0) givens_column(S, mk, mk - 1);
+      __syncwarp();
+      const int used = beta == 0.0 ? 0 : abs(S.used);
+      double g0 = lane < used ? S.gv[lane] : 0.0, g1 = lane + 32 < used ? S.gv[lane + 32] : 0.0;
+      double y0 = 0.0, y1 = 0.0;
+      for (int k = used - 1; k >= 0; k--) {
+        const double yk = __shfl_sync(0xffffffffu, k < 32 ? g0 : g1, k & 31) * rcp(S.H[k * mk + k]);
+        if (lane < k) g0 = fma(-S.H[lane * mk + k], yk, g0);
+        if (lane + 32 < k) g1 = fma(-S.H[(lane + 32) * mk + k], yk, g1);
+        if (lane == k) y0 = yk;
+        if (lane + 32 == k) y1 = yk;
+      }
+      if (lane < mk) S.y[lane] = y0;
+      if (lane + 32 < mk) S.y[lane + 32] = y1;
+      if (lane == 0 && blockIdx.x == 0) a.lres[1] = beta == 0.0 ? 0.0 : fabs(S.gv[used]);
+    }
+    __syncthreads();
+    // dx += sum_q y_q v_q
+    each([&](int i, double *) {
+#pragma unroll
+      for (int k = 0; k < CP; k++)
+        if (mine(i, k)) {
+          const double *v = a.V + at(i, k);
+          double x = a.dx[at(i, k)];
+#pragma unroll 8
+          for (int q = 0; q < mk; q++) x = fma(S.y[q], v[(size_t)q * a.vs], x);
+          a.dx[at(i, k)] = x;
+        }
+    });
+  }
+}
+
 }  // namespace
 
 void launch_scale_z(const DevMesh &m, const Scratch &s, const double *w, const double *h, double *v, double *zv,
@@ -269,6 +700,46 @@ void launch_mgs_blocks(const Scratch &s, int64_t n, double *w, int j, int mk, do
     else mgs_pass<4>(st, n, w, s.V, s.vstride, a, c, nd, j, mk, s.gram, Hj, s.red, s.red_count);
     HGKS_PROF_END(K_DOT, st);
   }
+}
+
+namespace {
+template <int NF>
+const void *grid_kernel(int lpc, bool one) {
+  if (lpc == 4) return (const void *)k_gmres_grid<NF, 4, true>;
+  if (lpc == 2) return (const void *)k_gmres_grid<NF, 2, true>;
+  return one ? (const void *)k_gmres_grid<NF, 1, true> : (const void *)k_gmres_grid<NF, 1, false>;
+}
+}  // namespace
+
+// All restart cycles in one cooperative launch, for meshes small enough. false: not launched
+// (mesh too large, or no cooperative launches).
+bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double *rhs, double *dx, cudaStream_t st) {
+  int dev = 0, sms = 0, coop = 0;
+  if (m.N > kGridCells || p.restarts < 1 || p.krylov_dim > kPMax || cudaGetDevice(&dev) != cudaSuccess) return false;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (!coop || sms < 1) return false;
+  const int blocks = std::min({sms, kPG, (m.N + 7) / 8}), C = (m.N + blocks - 1) / blocks;
+  const int lpc = C <= 32 ? 4 : C <= 64 ? 2 : 1;        // one warp per SM sub-partition at most
+  const bool one = C <= kPT;
+  const size_t shm = sizeof(GridShared) + (one ? 0 : sizeof(double) * 5 * C);
+  const void *fn = m.hex ? grid_kernel<HexShape::NF>(lpc, one) : grid_kernel<TetShape::NF>(lpc, one);
+  int fit = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, kPT + 32, shm) != cudaSuccess || fit < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaMemsetAsync(s.red_count + 2, 0, sizeof(unsigned), st);
+  GridSolve a{m.N, C, m.cnb, s.jv64, s.dval, s.dinv, rhs, dx, s.t, s.V, s.z[0], s.z[1], s.red,
+              s.hs + (p.krylov_dim + 1) * p.krylov_dim + 1 + p.krylov_dim, s.vstride, s.red_count + 2, s.flags + 1,
+              p.krylov_dim, p.restarts, p.jacobi_sweeps};
+  void *args[] = {&a};
+  HGKS_PROF_BEGIN(K_JACOBI, st);
+  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPT + 32), args, shm, st);
+  HGKS_PROF_END(K_JACOBI, st);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
 }
 
 }  // namespace hgks

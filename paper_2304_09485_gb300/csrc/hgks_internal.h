@@ -155,7 +155,7 @@ struct Scratch {
   unsigned int *red_count = nullptr;
   double *hs = nullptr;          // small device scalars: H, beta, y, norms
   double *gram = nullptr;        // [65*65 + 2*65] inner products of the Krylov basis and the MGS pass sums
-  int *flags = nullptr;          // [8] device flags (nonphysical count, breakdown)
+  int *flags = nullptr;          // [8] device flags (nonphysical count, a grid barrier that gave up)
   double *hostbuf = nullptr;     // [40][N] device state of the *_host entry points
   double *Qp = nullptr, *Rp = nullptr;   // [5][N] perturbed state and its residual (matrix-free products)
   int kdim = 0;
@@ -229,6 +229,7 @@ void launch_scale_z(const DevMesh &m, const Scratch &s, const double *w, const d
 void launch_neumann_z(const DevMesh &m, const Scratch &s, int sweeps, const double *v, double *w, int j, int mk, double *Hj,
                       cudaStream_t st);
 void launch_mgs_blocks(const Scratch &s, int64_t n, double *w, int j, int mk, double *Hj, bool have_first, cudaStream_t st);
+bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double *rhs, double *dx, cudaStream_t st);
 void launch_norm(const DevMesh &m, Scratch &s, const double *x, double *out_dev, cudaStream_t st);
 // force[3] on the boundary faces tagged `tag`, from the face fluxes of the last residual
 void launch_wall_force(const DevMesh &m, const Scratch &s, int tag, double *force_dev, cudaStream_t st);

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, KParams Pv, 
     if (jv64) {
       const double hS = j >= 0 ? 0.5 * S : 0.0, iq = rcp(Qj[0]);
       const double un = iq * (Qj[1] * n[0] + Qj[2] * n[1] + Qj[3] * n[2]);
-      const double rec[5] = {hS * n[0], hS * n[1], hS * n[2], hS * lam, hS * (un - lam)};
+      const double rec[5] = {hS * n[0], hS * n[1], hS * n[2], hS * (un - lam), hS * un};
 #pragma unroll
       for (int k = 0; k < 5; k++) jv64[(size_t)(6 + 5 * p + k) * N + i] = rec[k];
     }
@@ -815,7 +815,7 @@ hgks_status gmres_solve(const DevMesh &m, Scratch &s, const hgks_params &p, cons
     launch_norm(m, s, Q, s.hs + kHsNormQ, st);
   }
   if (p.precision == HGKS_MIXED) gmres_t<float>(m, s, kbuf32(s), p, rhs, dx, st, Q, G);
-  else gmres_t<double>(m, s, kbuf64(s), p, rhs, dx, st, Q, G);
+  else if (p.jv_mode == 1 || !gmres_grid(m, s, p, rhs, dx, st)) gmres_t<double>(m, s, kbuf64(s), p, rhs, dx, st, Q, G);
   if (info) info->krylov_iters = p.restarts * p.krylov_dim;
   return HGKS_OK;
 }

@@ -4,8 +4,8 @@
 
 namespace hgks {
 
-// Rows per (cell, local face) behind the six rows per cell of the operands: n S/2 (3),
-// lambda S/2, and in FP64 also u_j . n S/2 - lambda S/2.
+// Rows per (cell, local face) behind the six rows per cell of the operands: n S/2 (3), then
+// lambda S/2 (FP32) or s = u_j . n S/2 - lambda S/2 and t = u_j . n S/2 (FP64).
 template <typename TJ> struct JvRows;
 template <> struct JvRows<float> { static constexpr int face = 4; };
 template <> struct JvRows<double> { static constexpr int face = 5; };
@@ -19,7 +19,8 @@ __device__ __forceinline__ void offdiag_product(const TJ *__restrict__ jv, int N
   const TV u = jv[j], v = jv[(size_t)N + j], w = jv[2 * (size_t)N + j], H = jv[3 * (size_t)N + j];
   const TV phi = jv[4 * (size_t)N + j], g1 = jv[5 * (size_t)N + j];
   const TJ *f = jv + (size_t)(6 + JvRows<TJ>::face * p) * N + i;
-  const TV nx = f[0], ny = f[N], nz = f[2 * (size_t)N], ls = f[3 * (size_t)N];
+  const TV nx = f[0], ny = f[N], nz = f[2 * (size_t)N];
+  const TV ls = JvRows<TJ>::face == 4 ? f[3 * (size_t)N] : f[(JvRows<TJ>::face - 1) * (size_t)N] - f[3 * (size_t)N];
   const TV un = u * nx + v * ny + w * nz, nm = nx * x[1] + ny * x[2] + nz * x[3], um = u * x[1] + v * x[2] + w * x[3];
   const TV dp = g1 * (x[4] - um) + phi * x[0], t = nm - un * x[0];
   acc[0] += nm - ls * x[0];
@@ -30,19 +31,22 @@ __device__ __forceinline__ void offdiag_product(const TJ *__restrict__ jv, int N
 }
 
 // The same product in FP64 with what depends on the neighbour alone taken out of the sum
-// over faces: a vector x is kept as z = (x0, a, dp, e) per cell,
-//   a = m - u x0,  dp = (gamma - 1)(x4 - u . a) - (gamma - 1)|u|^2/2 x0,  e = x4 + dp - H x0,
-// and with s = u . n S/2 - lambda S/2 (stored) the block takes 17 operations instead of 28
-// (or 24 for a stored 5x5 block, whose 200 bytes per face it replaces with 40):
-//   r0 = n . a + s x0,  rows (r0, u r0 + s a + n dp, H r0 + s e + lambda S/2 dp).
-__device__ __forceinline__ void z_of(const double *__restrict__ jv, size_t N, int i, const double *y, double *z) {
-  const double u = jv[i], v = jv[N + i], w = jv[2 * N + i], H = jv[3 * N + i], phi = jv[4 * N + i], g1 = jv[5 * N + i];
+// over faces: a vector x is kept as z = (x0, a, dp, x4) per cell,
+//   a = m - u x0,  dp = (gamma - 1)(x4 - u . a) - (gamma - 1)|u|^2/2 x0,
+// and with s = u . n S/2 - lambda S/2 and t = u . n S/2 (stored) the block takes 17 operations
+// instead of 28 (or 24 for a stored 5x5 block, whose 200 bytes per face it replaces with 40):
+//   r = n . a,  r0 = r + s x0,  rows (r0, u r0 + s a + n dp, H r + s x4 + t dp).
+struct CellPrim { double u, v, w, H, phi, g1; };
+__device__ __forceinline__ CellPrim cell_prim(const double *__restrict__ jv, size_t N, int i) {
+  return {jv[i], jv[N + i], jv[2 * N + i], jv[3 * N + i], jv[4 * N + i], jv[5 * N + i]};
+}
+__device__ __forceinline__ void z_of(const CellPrim &q, const double *y, double *z) {
   z[0] = y[0];
-  z[1] = fma(-u, y[0], y[1]);
-  z[2] = fma(-v, y[0], y[2]);
-  z[3] = fma(-w, y[0], y[3]);
-  z[4] = fma(g1, fma(-u, z[1], fma(-v, z[2], fma(-w, z[3], y[4]))), -phi * y[0]);
-  z[5] = fma(-H, y[0], y[4] + z[4]);
+  z[1] = fma(-q.u, y[0], y[1]);
+  z[2] = fma(-q.v, y[0], y[2]);
+  z[3] = fma(-q.w, y[0], y[3]);
+  z[4] = fma(q.g1, fma(-q.u, z[1], fma(-q.v, z[2], fma(-q.w, z[3], y[4]))), -q.phi * y[0]);
+  z[5] = y[4];
 }
 __device__ __forceinline__ void z_store(double *zv, size_t N, int i, const double *z) {
 #pragma unroll
@@ -52,14 +56,14 @@ __device__ __forceinline__ void z_store(double *zv, size_t N, int i, const doubl
 __device__ __forceinline__ void z_product(const double *__restrict__ jv, size_t N, int i, int p, int j, const double *zv,
                                           double *acc) {
   const double *f = jv + (6 + 5 * (size_t)p) * N + i;
-  const double nx = f[0], ny = f[N], nz = f[2 * N], ls = f[3 * N], s = f[4 * N];
-  const double x0 = zv[j], a0 = zv[N + j], a1 = zv[2 * N + j], a2 = zv[3 * N + j], dp = zv[4 * N + j], e = zv[5 * N + j];
-  const double r0 = fma(nx, a0, fma(ny, a1, fma(nz, a2, s * x0)));
+  const double nx = f[0], ny = f[N], nz = f[2 * N], s = f[3 * N], t = f[4 * N];
+  const double x0 = zv[j], a0 = zv[N + j], a1 = zv[2 * N + j], a2 = zv[3 * N + j], dp = zv[4 * N + j], x4 = zv[5 * N + j];
+  const double r = fma(nx, a0, fma(ny, a1, nz * a2)), r0 = fma(s, x0, r);
   acc[0] += r0;
   acc[1] = fma(jv[j], r0, fma(s, a0, fma(nx, dp, acc[1])));
   acc[2] = fma(jv[N + j], r0, fma(s, a1, fma(ny, dp, acc[2])));
   acc[3] = fma(jv[2 * N + j], r0, fma(s, a2, fma(nz, dp, acc[3])));
-  acc[4] = fma(jv[3 * N + j], r0, fma(s, e, fma(ls, dp, acc[4])));
+  acc[4] = fma(jv[3 * N + j], r, fma(s, x4, fma(t, dp, acc[4])));
 }
 
 }  // namespace hgks
