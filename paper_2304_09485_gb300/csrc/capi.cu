@@ -176,11 +176,9 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     if ((st = dalloc(m, &s.t2, 5 * N))) return st;
     if ((st = dalloc(m, &s.hs, 65 * 64 + 256))) return st;
     if ((st = dalloc(m, &s.gram, 65 * 65 + 2 * 65 + 64))) return st;
-    HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
-  }
-  if (implicit && !mixed && !arena && !s.z[0]) {
     for (double *&z : s.z)
-      if ((st = dalloc(m, &z, 6 * N))) return st;
+      if (!arena && (st = dalloc(m, &z, 6 * N))) return st;
+    HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
   }
   if (implicit && mixed && !s.jv32) {
     if ((st = dalloc(m, &s.jv32, (6 + 4 * NF) * N))) return st;
@@ -441,7 +439,7 @@ hgks_status hgks_apply_jacobian(hgks_mesh mesh, const double *x, double *y, void
   Mesh &m = mesh->m;
   if (!m.s.jv64) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
   HGKS_ON_DEVICE(m.device);
-  launch_apply_A(m.d, m.s, x, y, (cudaStream_t)cuda_stream);
+  launch_apply_A(m.d, m.s, nullptr, x, y, (cudaStream_t)cuda_stream);
   return last_launch();
 }
 

@@ -81,24 +81,62 @@ __global__ void __launch_bounds__(kCell) k_scale_z(int N, const double *__restri
   z_store(zv, N, i, z);
 }
 
-// y = sign D^{-1} O x, both in z form
-template <int NF>
+// z(x), or z(D^{-1} x) with dinv
+__global__ void __launch_bounds__(kCell) k_z(int N, const double *__restrict__ jv, const double *__restrict__ dinv,
+                                             const double *__restrict__ x, double *__restrict__ zv) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  double y[5], z[6];
+#pragma unroll
+  for (int c = 0; c < 5; c++) y[c] = x[(size_t)c * N + i];
+  if (dinv) {
+    const double d = dinv[i];
+#pragma unroll
+    for (int c = 0; c < 5; c++) y[c] *= d;
+  }
+  z_of(cell_prim(jv, N, i), y, z);
+  z_store(zv, N, i, z);
+}
+
+// One product with the off-diagonal part of A, x in z form:
+//   kE      y = sign D^{-1} O x, in z form
+//   kSweep  y = D^{-1} (b - O x), in z form;   kLast the same, y as it is
+//   kSpmv   y = d x5 + O x, or b - that with b (x5: the vector of x)
+enum { kE, kSweep, kLast, kSpmv };
+template <int NF, int Mode>
 __global__ void __launch_bounds__(kCell) k_zprod(int N, const int *__restrict__ cnb, const double *__restrict__ jv,
-                                                 const double *__restrict__ dinv, double sign, const double *__restrict__ x,
+                                                 const double *__restrict__ dd, double sign, const double *__restrict__ b,
+                                                 const double *__restrict__ x5, const double *__restrict__ x,
                                                  double *__restrict__ y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  double acc[5] = {0, 0, 0, 0, 0}, z[6];
+  double acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll
   for (int p = 0; p < NF; p++) {
     const int j = cnb[(size_t)p * N + i];
     if (j >= 0) z_product(jv, N, i, p, j, x, acc);
   }
-  const double d = sign * dinv[i];
+  const double d = Mode == kE ? sign * dd[i] : dd[i];    // D^{-1}, or D for kSpmv
 #pragma unroll
-  for (int c = 0; c < 5; c++) acc[c] *= d;
-  z_of(cell_prim(jv, N, i), acc, z);
-  z_store(y, N, i, z);
+  for (int c = 0; c < 5; c++) {
+    const size_t k = (size_t)c * N + i;
+    if (Mode == kE) acc[c] *= d;
+    else if (Mode != kSpmv) acc[c] = d * (b[k] - acc[c]);
+    else acc[c] = b ? b[k] - fma(d, x5[k], acc[c]) : fma(d, x5[k], acc[c]);
+    if (Mode == kLast || Mode == kSpmv) y[k] = acc[c];
+  }
+  if (Mode == kE || Mode == kSweep) {
+    double z[6];
+    z_of(cell_prim(jv, N, i), acc, z);
+    z_store(y, N, i, z);
+  }
+}
+template <int Mode>
+void zprod(cudaStream_t st, const DevMesh &m, const Scratch &s, const double *dd, double sign, const double *b,
+           const double *x5, const double *x, double *y) {
+  const unsigned g = grid_for(m.N, kCell);
+  if (m.hex) k_zprod<HexShape::NF, Mode><<<g, kCell, 0, st>>>(m.N, m.cnb, s.jv64, dd, sign, b, x5, x, y);
+  else k_zprod<TetShape::NF, Mode><<<g, kCell, 0, st>>>(m.N, m.cnb, s.jv64, dd, sign, b, x5, x, y);
 }
 
 // w = v + D^{-1} O x (x in z form), then the coefficients of the first ND basis vectors
@@ -663,16 +701,37 @@ void launch_scale_z(const DevMesh &m, const Scratch &s, const double *w, const d
   HGKS_PROF_END(K_SCALE, st);
 }
 
+// y = A x, or b - A x
+void launch_apply_A(const DevMesh &m, const Scratch &s, const double *b, const double *x, double *y, cudaStream_t st) {
+  HGKS_PROF_BEGIN(K_SCALE, st);
+  k_z<<<grid_for(m.N, kCell), kCell, 0, st>>>(m.N, s.jv64, nullptr, x, s.z[0]);
+  HGKS_PROF_END(K_SCALE, st);
+  HGKS_PROF_BEGIN(K_SPMV, st);
+  zprod<kSpmv>(st, m, s, s.dval, 1.0, b, x, s.z[0], y);
+  HGKS_PROF_END(K_SPMV, st);
+}
+
+// x = P^{-1} b (Eq. (precond)), at least one sweep
+void launch_sweeps_z(const DevMesh &m, const Scratch &s, int sweeps, const double *b, double *x, cudaStream_t st) {
+  HGKS_PROF_BEGIN(K_SCALE, st);
+  k_z<<<grid_for(m.N, kCell), kCell, 0, st>>>(m.N, s.jv64, s.dinv, b, s.z[0]);
+  HGKS_PROF_END(K_SCALE, st);
+  for (int q = 1; q <= sweeps; q++) {
+    HGKS_PROF_BEGIN(K_JACOBI, st);
+    if (q < sweeps) zprod<kSweep>(st, m, s, s.dinv, 1.0, b, nullptr, s.z[(q - 1) & 1], s.z[q & 1]);
+    else zprod<kLast>(st, m, s, s.dinv, 1.0, b, nullptr, s.z[(q - 1) & 1], x);
+    HGKS_PROF_END(K_JACOBI, st);
+  }
+}
+
 void launch_neumann_z(const DevMesh &m, const Scratch &s, int sweeps, const double *v, double *w, int j, int mk, double *Hj,
                       cudaStream_t st) {
   // s.z[0] holds z(v); E^sweeps v with the sign in its first product, then w = v + E z
-  const unsigned g = grid_for(m.N, kCell);
   int src = 0;
   for (int q = 0; q < sweeps; q++, src ^= 1) {
     const double sign = q == 0 && sweeps % 2 == 1 ? -1.0 : 1.0;
     HGKS_PROF_BEGIN(K_JACOBI, st);
-    if (m.hex) k_zprod<HexShape::NF><<<g, kCell, 0, st>>>(m.N, m.cnb, s.jv64, s.dinv, sign, s.z[src], s.z[src ^ 1]);
-    else k_zprod<TetShape::NF><<<g, kCell, 0, st>>>(m.N, m.cnb, s.jv64, s.dinv, sign, s.z[src], s.z[src ^ 1]);
+    zprod<kE>(st, m, s, s.dinv, sign, nullptr, nullptr, s.z[src], s.z[src ^ 1]);
     HGKS_PROF_END(K_JACOBI, st);
   }
   const int nd = std::min(kBlk, j + 1);

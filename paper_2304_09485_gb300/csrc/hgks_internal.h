@@ -214,7 +214,6 @@ void launch_residual(const DevMesh &m, Scratch &s, const hgks_params &p, const d
                      double *R, double *Gnew, cudaStream_t st, bool batch = false, bool fresh_dt = true);
 void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *dt,
                      double *diag_out, double *off_out, cudaStream_t st, bool batch = false);
-void launch_apply_A(const DevMesh &m, const Scratch &s, const double *x, double *y, cudaStream_t st);
 void launch_precondition(const DevMesh &m, Scratch &s, int sweeps, const double *b, double *x, cudaStream_t st);
 // Q, G: the step's state, for the matrix-free products of jv_mode 1 (s.R = L(Q), s.dt its time step)
 hgks_status gmres_solve(const DevMesh &m, Scratch &s, const hgks_params &p, const double *rhs, double *dx,
@@ -223,7 +222,10 @@ hgks_status gmres_solve(const DevMesh &m, Scratch &s, const hgks_params &p, cons
 // needs s.R = L(Q) and s.dt, and ||Q|| in s.hs[kHsNormQ]
 void launch_apply_fd(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *G,
                      const double *x, const double *b, double *y, cudaStream_t st);
-// FP64 GMRES with the assembled A (gmres64.cu); Hj: column j of H (leading dimension mk)
+// FP64 products with the assembled A (gmres64.cu): y = A x (b null) or b - A x; x = P^{-1} b with sweeps > 0
+void launch_apply_A(const DevMesh &m, const Scratch &s, const double *b, const double *x, double *y, cudaStream_t st);
+void launch_sweeps_z(const DevMesh &m, const Scratch &s, int sweeps, const double *b, double *x, cudaStream_t st);
+// its GMRES; Hj: column j of H (leading dimension mk)
 void launch_scale_z(const DevMesh &m, const Scratch &s, const double *w, const double *h, double *v, double *zv,
                     cudaStream_t st);
 void launch_neumann_z(const DevMesh &m, const Scratch &s, int sweeps, const double *v, double *w, int j, int mk, double *Hj,

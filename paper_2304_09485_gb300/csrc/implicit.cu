@@ -10,8 +10,8 @@
 //    the operands of their products (offdiag.cuh), component-major so that the
 //    thread of cell i reads consecutive addresses with its warp; batches with FP64
 //    vectors store them, off[(p*25 + k)][N] (p = local face of the row cell).
-//  * Jacobi preconditioner of Eq. (precond), k_max sweeps. The first sweep reads
-//    D^{-1} b of the neighbours on the fly (no separate x0 pass).
+//  * Jacobi preconditioner of Eq. (precond), k_max sweeps (FP32: the first sweep reads
+//    D^{-1} b of the neighbours on the fly).
 //  * Restarted GMRES with modified Gram-Schmidt (Algorithm 1). Every inner
 //    product finishes inside its launch: blocks write partial sums, the last
 //    block to finish adds them in a fixed order (deterministic, no host round
@@ -32,24 +32,23 @@ constexpr int kBlock = 256;
 constexpr int kCellBlock = 128;
 constexpr int kRedBlocks = 152 * 4;   // blocks of the vector reductions: a multiple of the SM count
 
-__device__ __forceinline__ void euler_jacobian(const double *Q, const double *n, double gamma, double *J) {
-  const double ir = 1.0 / Q[0];
-  const double u = Q[1] * ir, v = Q[2] * ir, w = Q[3] * ir, E = Q[4] * ir;
-  const double g1 = gamma - 1.0, phi = 0.5 * g1 * (u * u + v * v + w * w);
-  const double un = u * n[0] + v * n[1] + w * n[2], H = gamma * E - phi;
-  const double vel[3] = {u, v, w};
-  J[0] = 0.0; J[1] = n[0]; J[2] = n[1]; J[3] = n[2]; J[4] = 0.0;
+// (J(Q) - lambda I) S/2 for nS = n S/2 and lS = lambda S/2, Q with primitives (vel, H), phi = (gamma - 1)|u|^2/2,
+// un = u . nS: every entry from products that carry S/2 already
+__device__ __forceinline__ void offdiag_block(const double *vel, double H, double phi, double g1, const double *nS,
+                                              double un, double lS, double *J) {
+  const double gv[3] = {g1 * vel[0], g1 * vel[1], g1 * vel[2]}, s = un - lS;
+  J[0] = -lS; J[1] = nS[0]; J[2] = nS[1]; J[3] = nS[2]; J[4] = 0.0;
 #pragma unroll
   for (int r = 0; r < 3; r++) {
-    J[5 * (r + 1)] = phi * n[r] - vel[r] * un;
+    J[5 * (r + 1)] = fma(phi, nS[r], -vel[r] * un);
 #pragma unroll
-    for (int c = 0; c < 3; c++) J[5 * (r + 1) + 1 + c] = vel[r] * n[c] - g1 * vel[c] * n[r] + (r == c ? un : 0.0);
-    J[5 * (r + 1) + 4] = g1 * n[r];
+    for (int c = 0; c < 3; c++) J[5 * (r + 1) + 1 + c] = fma(vel[r], nS[c], r == c ? fma(-gv[c], nS[r], s) : -gv[c] * nS[r]);
+    J[5 * (r + 1) + 4] = g1 * nS[r];
   }
   J[20] = (phi - H) * un;
 #pragma unroll
-  for (int c = 0; c < 3; c++) J[21 + c] = H * n[c] - g1 * vel[c] * un;
-  J[24] = gamma * un;
+  for (int c = 0; c < 3; c++) J[21 + c] = fma(H, nS[c], -gv[c] * un);
+  J[24] = fma(g1, un, s);
 }
 
 // off, off_out: the blocks themselves (may be null); jv64, jv32 (may be null): the operands
@@ -99,40 +98,45 @@ __global__ void __launch_bounds__(kCellBlock) k_assemble(DevMesh m, KParams Pv, 
   for (int p = 0; p < NF; p++) {
     const int cf = m.cface[(size_t)p * N + i], f = cf >> 1, side = cf & 1;
     const int j = m.cnb[(size_t)p * N + i];
-    const double sg = side ? -1.0 : 1.0;
     double n[3];
 #pragma unroll
-    for (int k = 0; k < 3; k++) n[k] = sg * m.fT[(size_t)k * F + f];
-    const double S = m.fS[f];
-    double Qj[5], Qf[5];
+    for (int k = 0; k < 3; k++) {
+      const double t = m.fT[(size_t)k * F + f];
+      n[k] = side ? -t : t;
+    }
+    const double hS = 0.5 * m.fS[f];
+    double Qj[5], Qf[5];                                // Qf: twice the face state (only ratios are taken)
 #pragma unroll
     for (int c = 0; c < 5; c++) {
       Qj[c] = j >= 0 ? Q[(size_t)c * N + j] : Qi[c];
-      Qf[c] = 0.5 * (Qi[c] + Qj[c]);
+      Qf[c] = Qi[c] + Qj[c];
     }
     const double ir = rcp(Qf[0]);
     const double u = Qf[1] * ir, v = Qf[2] * ir, w = Qf[3] * ir;
     const double pr = P.g1 * (Qf[4] - 0.5 * Qf[0] * (u * u + v * v + w * w));
     double lam = fabs(u * n[0] + v * n[1] + w * n[2]) + sqrt64(P.gamma * pr * ir);
-    if (P.viscous) lam += 2.0 * P.mu * ir * rcp(m.fdist[f]);
-    d += 0.5 * lam * S;
+    if (P.viscous) lam += 4.0 * P.mu * ir * rcp(m.fdist[f]);
+    const double lS = lam * hS;
+    d += lS;
     if (jv32)
 #pragma unroll
       for (int k = 0; k < 4; k++)
-        jv32[(size_t)(6 + 4 * p + k) * N + i] = j >= 0 ? (float)(0.5 * S * (k < 3 ? n[k] : lam)) : 0.0f;
+        jv32[(size_t)(6 + 4 * p + k) * N + i] = j >= 0 ? (float)(k < 3 ? hS * n[k] : lS) : 0.0f;
+    if (!jv64 && !off && !off_out) continue;
+    const double iq = rcp(Qj[0]), vel[3] = {Qj[1] * iq, Qj[2] * iq, Qj[3] * iq}, nS[3] = {hS * n[0], hS * n[1], hS * n[2]};
+    const double un = vel[0] * nS[0] + vel[1] * nS[1] + vel[2] * nS[2];
     if (jv64) {
-      const double hS = j >= 0 ? 0.5 * S : 0.0, iq = rcp(Qj[0]);
-      const double un = iq * (Qj[1] * n[0] + Qj[2] * n[1] + Qj[3] * n[2]);
-      const double rec[5] = {hS * n[0], hS * n[1], hS * n[2], hS * (un - lam), hS * un};
+      const double rec[5] = {nS[0], nS[1], nS[2], un - lS, un};
 #pragma unroll
-      for (int k = 0; k < 5; k++) jv64[(size_t)(6 + 5 * p + k) * N + i] = rec[k];
+      for (int k = 0; k < 5; k++) jv64[(size_t)(6 + 5 * p + k) * N + i] = j >= 0 ? rec[k] : 0.0;
     }
     if (off || off_out) {
       double J[25];
-      if (j >= 0) euler_jacobian(Qj, n, P.gamma, J);
+      const double phi = 0.5 * P.g1 * (vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2]);
+      offdiag_block(vel, P.gamma * Qj[4] * iq - phi, phi, P.g1, nS, un, lS, J);
 #pragma unroll
       for (int k = 0; k < 25; k++) {
-        const double o = j >= 0 ? 0.5 * (J[k] - (k % 6 == 0 ? lam : 0.0)) * S : 0.0;
+        const double o = j >= 0 ? J[k] : 0.0;
         if (off) off[(size_t)(p * 25 + k) * N + i] = o;
         if (off_out) off_out[(size_t)(p * 25 + k) * N + i] = o;
       }
@@ -191,80 +195,63 @@ __device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, 
   }
 }
 
-// One product with the off-diagonal part of A. Modes:
-//   kSpmv   : y = [b -] (d x + sum_p A_ip x_p)
+// One product with the off-diagonal part of A from FP32 operands (mixed precision; FP64
+// vectors: gmres64.cu). Modes:
+//   kSpmv   : y = b - (d x + sum_p A_ip x_p)
 //   kJacobi : y = D^{-1} (b - sum_p A_ip x_p); FirstSweep: x_p = D^{-1} b at the neighbours
 //   kNeumann: y = b + D^{-1} sum_p A_ip x_p
 //   kE, kNegE: y = +- D^{-1} sum_p A_ip x_p
-// and optionally the inner product (y, dotv) reduced into *dot_out.
-// TM: type of the operands of the blocks, TV: type of b and x (and of the
-// accumulation), TO: type of y. The Krylov products of FP64 vectors are in gmres64.cu.
+// TV: type of b and x (and of the accumulation).
 enum { kSpmv = 0, kJacobi = 1, kNeumann = 2, kE = 3, kNegE = 4 };
 
-template <typename TM, typename TV, typename TO, int Mode, bool FirstSweep, int NF>
-__global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const TM *__restrict__ jv, const TM *__restrict__ dval,
-                                                      const TM *__restrict__ dinv, const TV *__restrict__ b,
-                                                      const TV *__restrict__ x, TO *__restrict__ y,
-                                                      const TO *__restrict__ dotv, TO *partials, unsigned int *count,
-                                                      double *dot_out) {
+template <typename TV, int Mode, bool FirstSweep, int NF>
+__global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const float *__restrict__ jv,
+                                                      const float *__restrict__ dval, const float *__restrict__ dinv,
+                                                      const TV *__restrict__ b, const TV *__restrict__ x,
+                                                      float *__restrict__ y) {
   const int N = m.N;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  TO part = TO(0);
-  if (i < N) {
-    TV acc[5];
-    const TV di = Mode == kSpmv ? (TV)dval[i] : TV(0);
+  if (i >= N) return;
+  TV acc[5];
+  const TV di = Mode == kSpmv ? (TV)dval[i] : TV(0);
 #pragma unroll
-    for (int r = 0; r < 5; r++) acc[r] = Mode == kSpmv ? di * x[(size_t)r * N + i] : TV(0);
+  for (int r = 0; r < 5; r++) acc[r] = Mode == kSpmv ? di * x[(size_t)r * N + i] : TV(0);
 #pragma unroll
-    for (int p = 0; p < NF; p++) {
-      const int j = m.cnb[(size_t)p * N + i];
-      if (j < 0) continue;
-      TV xj[5];
-      const TV sj = FirstSweep ? (TV)dinv[j] : TV(1);
+  for (int p = 0; p < NF; p++) {
+    const int j = m.cnb[(size_t)p * N + i];
+    if (j < 0) continue;
+    TV xj[5];
+    const TV sj = FirstSweep ? (TV)dinv[j] : TV(1);
 #pragma unroll
-      for (int c = 0; c < 5; c++) xj[c] = FirstSweep ? sj * b[(size_t)c * N + j] : x[(size_t)c * N + j];
-      offdiag_product<TV>(jv, N, i, p, j, xj, acc);
-    }
-    TV out[5];
-    if (Mode == kJacobi) {
-      const TV dd = (TV)dinv[i];
-#pragma unroll
-      for (int r = 0; r < 5; r++) out[r] = dd * (b[(size_t)r * N + i] - acc[r]);
-    } else if (Mode == kE || Mode == kNegE) {
-      const TV dd = Mode == kE ? (TV)dinv[i] : -(TV)dinv[i];
-#pragma unroll
-      for (int r = 0; r < 5; r++) out[r] = dd * acc[r];
-    } else if (Mode == kNeumann) {
-      const TV dd = (TV)dinv[i];
-#pragma unroll
-      for (int r = 0; r < 5; r++) out[r] = fma(dd, acc[r], b[(size_t)r * N + i]);
-    } else if (b) {
-#pragma unroll
-      for (int r = 0; r < 5; r++) out[r] = b[(size_t)r * N + i] - acc[r];
-    } else {
-#pragma unroll
-      for (int r = 0; r < 5; r++) out[r] = acc[r];
-    }
-#pragma unroll
-    for (int r = 0; r < 5; r++) {
-      const TO o = (TO)out[r];
-      y[(size_t)r * N + i] = o;
-      if (dotv) part = fma(o, dotv[(size_t)r * N + i], part);
-    }
+    for (int c = 0; c < 5; c++) xj[c] = FirstSweep ? sj * b[(size_t)c * N + j] : x[(size_t)c * N + j];
+    offdiag_product<TV>(jv, N, i, p, j, xj, acc);
   }
-  if (dotv) grid_sum(part, partials, count, dot_out, 0);
+#pragma unroll
+  for (int r = 0; r < 5; r++) {
+    const TV dd = Mode == kNegE ? -(TV)dinv[i] : (TV)dinv[i], br = Mode == kE || Mode == kNegE ? TV(0) : b[(size_t)r * N + i];
+    TV o;
+    if (Mode == kJacobi) o = dd * (br - acc[r]);
+    else if (Mode == kE || Mode == kNegE) o = dd * acc[r];
+    else if (Mode == kNeumann) o = fma(dd, acc[r], br);
+    else o = br - acc[r];
+    y[(size_t)r * N + i] = (float)o;
+  }
 }
 
 // k_apply for the mesh's cell kind (4 or 6 off-diagonal blocks per row)
-template <typename TM, typename TV, typename TO, int Mode, bool FirstSweep>
-void apply_launch(unsigned grid, cudaStream_t st, const DevMesh &m, const TM *jv, const TM *dval, const TM *dinv,
-                  const TV *b, const TV *x, TO *y, const TO *dotv, TO *partials, unsigned int *count, double *dot_out) {
+template <typename TV, int Mode, bool FirstSweep>
+void apply_launch(cudaStream_t st, const DevMesh &m, const Scratch &s, const TV *b, const TV *x, float *y) {
+  const unsigned grid = grid_for(m.N, kCellBlock);
   if (m.hex)
-    k_apply<TM, TV, TO, Mode, FirstSweep, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, jv, dval, dinv, b, x, y, dotv,
-                                                                                      partials, count, dot_out);
+    k_apply<TV, Mode, FirstSweep, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x, y);
   else
-    k_apply<TM, TV, TO, Mode, FirstSweep, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, jv, dval, dinv, b, x, y, dotv,
-                                                                                      partials, count, dot_out);
+    k_apply<TV, Mode, FirstSweep, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x, y);
+}
+
+// y = x rounded to float
+__global__ void k_round(int64_t n, const double *__restrict__ x, float *__restrict__ y) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+    y[k] = (float)x[k];
 }
 
 template <typename T>
@@ -561,11 +548,11 @@ unsigned vec_grid(int64_t n) {
 // Buffers of one precision for the Krylov part of a step.
 template <typename T>
 struct KBuf {
-  const T *jv, *dval, *dinv;
+  const T *dinv;
   T *V, *w, *t, *t2, *red;
 };
-KBuf<double> kbuf64(Scratch &s) { return {s.jv64, s.dval, s.dinv, s.V, s.w, s.t, s.t2, s.red}; }
-KBuf<float> kbuf32(Scratch &s) { return {s.jv32, s.dval32, s.dinv32, s.V32, s.w32, s.t32, s.t232, s.red32}; }
+KBuf<double> kbuf64(Scratch &s) { return {s.dinv, s.V, s.w, s.t, s.t2, s.red}; }
+KBuf<float> kbuf32(Scratch &s) { return {s.dinv32, s.V32, s.w32, s.t32, s.t232, s.red32}; }
 
 template <typename T> T *partials(Scratch &s);
 template <> double *partials<double>(Scratch &s) { return s.red; }
@@ -590,36 +577,28 @@ void fd_apply(const DevMesh &m, Scratch &s, const hgks_params &p, const double *
   HGKS_PROF_END(K_SPMV, st);
 }
 
-// x = P^{-1} b (Eq. (precond)); if dotv is given, also (x, dotv) into *dot_out.
+// x = P^{-1} b (Eq. (precond))
 template <typename T>
-void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, const T *b, T *x, const T *dotv,
-                    double *dot_out, cudaStream_t st) {
-  const unsigned cg = grid_for(m.N, kCellBlock);
+void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, const T *b, T *x, cudaStream_t st) {
   if (sweeps == 0) {
     HGKS_PROF_BEGIN(K_DIAG, st);
     k_diag_scale<T><<<grid_for(5 * (int64_t)m.N, kBlock), kBlock, 0, st>>>(m.N, k.dinv, b, x);
     HGKS_PROF_END(K_DIAG, st);
-    if (dotv) {
-      HGKS_PROF_BEGIN(K_DOT, st);
-      k_axpy_dot<T><<<kRedBlocks, kBlock, 0, st>>>(5 * (int64_t)m.N, x, nullptr, nullptr, dotv, 0, k.red, s.red_count, dot_out);
-      HGKS_PROF_END(K_DOT, st);
-    }
     return;
   }
-  // sweep k writes to x when (sweeps - k) is even, else to t2: the last lands in x
-  const T *prev = nullptr;
-  for (int q = 1; q <= sweeps; q++) {
-    T *dst = ((sweeps - q) % 2 == 0) ? x : k.t2;
-    const T *dv = (q == sweeps) ? dotv : nullptr;
-    HGKS_PROF_BEGIN(K_JACOBI, st);
-    if (q == 1)
-      apply_launch<T, T, T, kJacobi, true>(cg, st, m, k.jv, k.dval, k.dinv, b, nullptr, dst, dv, k.red,
-                                                                  s.red_count, dot_out);
-    else
-      apply_launch<T, T, T, kJacobi, false>(cg, st, m, k.jv, k.dval, k.dinv, b, prev, dst, dv, k.red,
-                                                                   s.red_count, dot_out);
-    HGKS_PROF_END(K_JACOBI, st);
-    prev = dst;
+  if constexpr (std::is_same<T, double>::value) {
+    launch_sweeps_z(m, s, sweeps, b, x, st);
+  } else {
+    // sweep k writes to x when (sweeps - k) is even, else to t2: the last lands in x
+    const float *prev = nullptr;
+    for (int q = 1; q <= sweeps; q++) {
+      float *dst = ((sweeps - q) % 2 == 0) ? x : k.t2;
+      HGKS_PROF_BEGIN(K_JACOBI, st);
+      if (q == 1) apply_launch<float, kJacobi, true>(st, m, s, b, prev, dst);
+      else apply_launch<float, kJacobi, false>(st, m, s, b, prev, dst);
+      HGKS_PROF_END(K_JACOBI, st);
+      prev = dst;
+    }
   }
 }
 
@@ -633,23 +612,17 @@ void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, 
 // neighbours' values by D^{-1}. (FP32 vectors; FP64: launch_neumann_z.)
 void neumann32(const DevMesh &m, Scratch &s, const KBuf<float> &k, int sweeps, const float *v, float *w,
                cudaStream_t st) {
-  const unsigned cg = grid_for(m.N, kCellBlock);
   const float *z = v, *none = nullptr;
   for (int q = 0; q < sweeps; q++) {
     float *dst = (q % 2 == 0) ? k.t : k.t2;
     HGKS_PROF_BEGIN(K_JACOBI, st);
-    if (q == 0 && sweeps % 2 == 1)
-      apply_launch<float, float, float, kNegE, false>(cg, st, m, k.jv, k.dval, k.dinv, none, z, dst, none, k.red,
-                                                      s.red_count, nullptr);
-    else
-      apply_launch<float, float, float, kE, false>(cg, st, m, k.jv, k.dval, k.dinv, none, z, dst, none, k.red,
-                                                   s.red_count, nullptr);
+    if (q == 0 && sweeps % 2 == 1) apply_launch<float, kNegE, false>(st, m, s, none, z, dst);
+    else apply_launch<float, kE, false>(st, m, s, none, z, dst);
     HGKS_PROF_END(K_JACOBI, st);
     z = dst;
   }
   HGKS_PROF_BEGIN(K_SPMV, st);
-  apply_launch<float, float, float, kNeumann, false>(cg, st, m, k.jv, k.dval, k.dinv, v, z, w, none, k.red,
-                                                     s.red_count, nullptr);
+  apply_launch<float, kNeumann, false>(st, m, s, v, z, w);
   HGKS_PROF_END(K_SPMV, st);
 }
 
@@ -668,7 +641,7 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
   // (one FP64 FMA per 8 bytes read already exceeds it), so FP64 goes by blocks
   // (gmres64.cu), 2 FMAs and 20 bytes.
   constexpr bool one_pass = std::is_same<T, float>::value;
-  const unsigned vg = vec_grid(n), cg = grid_for(m.N, kCellBlock);
+  const unsigned vg = vec_grid(n);
   for (int it = 0; it < p.restarts; it++) {
     cudaMemsetAsync(H, 0, sizeof(double) * (mk + 1) * mk, st);
     // r0 = rhs - A dx (FP64 vectors, blocks of precision T), v1 = P^{-1} r0 / ||P^{-1} r0||
@@ -678,13 +651,18 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
       HGKS_PROF_BEGIN(K_SPMV, st);
       k_fd_combine<double, T><<<vec_grid(n), kBlock, 0, st>>>(m.N, m.vol, s.dt, dx, s.Rp, s.R, s.hs + kHsNormQ + 3, rhs, k.t);
       HGKS_PROF_END(K_SPMV, st);
-    } else {
+    } else if constexpr (one_pass) {
       HGKS_PROF_BEGIN(K_SPMV, st);
-      apply_launch<T, double, T, kSpmv, false>(cg, st, m, k.jv, k.dval, k.dinv, rhs, dx, k.t, nullptr,
-                                                                      nullptr, nullptr, nullptr);
+      if (it > 0) apply_launch<double, kSpmv, false>(st, m, s, rhs, dx, k.t);
+      else k_round<<<vec_grid(n), kBlock, 0, st>>>(n, rhs, k.t);
       HGKS_PROF_END(K_SPMV, st);
+    } else if (it > 0) {
+      launch_apply_A(m, s, rhs, dx, k.t, st);
     }
-    precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, nullptr, nullptr, st);
+    const T *r0 = k.t;
+    if constexpr (!one_pass)
+      if (!fd && it == 0) r0 = rhs;        // dx = 0
+    precondition_t<T>(m, s, k, p.jacobi_sweeps, r0, k.w, st);
     HGKS_PROF_BEGIN(K_DOT, st);
     k_axpy_dot<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, nullptr, nullptr, k.w, 1, k.red, s.red_count, beta);
     HGKS_PROF_END(K_DOT, st);
@@ -703,7 +681,7 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
       const T *vj = k.V + (size_t)j * vs;
       if (fd) {
         fd_apply<T, T>(m, s, p, Q, G, vj, nullptr, k.t, st);
-        precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, nullptr, nullptr, st);
+        precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, st);
       } else if constexpr (one_pass) {
         neumann32(m, s, k, p.jacobi_sweeps, vj, k.w, st);
       } else {
@@ -766,16 +744,8 @@ void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &hp, const 
   HGKS_PROF_END(K_ASSEMBLE, st);
 }
 
-void launch_apply_A(const DevMesh &m, const Scratch &s, const double *x, double *y, cudaStream_t st) {
-  HGKS_PROF_BEGIN(K_SPMV, st);
-  apply_launch<double, double, double, kSpmv, false>(grid_for(m.N, kCellBlock), st, m, s.jv64, s.dval, s.dinv,
-                                                     (const double *)nullptr, x, y, (const double *)nullptr,
-                                                     (double *)nullptr, nullptr, nullptr);
-  HGKS_PROF_END(K_SPMV, st);
-}
-
 void launch_precondition(const DevMesh &m, Scratch &s, int sweeps, const double *b, double *x, cudaStream_t st) {
-  precondition_t<double>(m, s, kbuf64(s), sweeps, b, x, nullptr, nullptr, st);
+  precondition_t<double>(m, s, kbuf64(s), sweeps, b, x, st);
 }
 
 void launch_norm(const DevMesh &m, Scratch &s, const double *x, double *out_dev, cudaStream_t st) {

@@ -4,23 +4,17 @@
 
 namespace hgks {
 
-// Rows per (cell, local face) behind the six rows per cell of the operands: n S/2 (3), then
-// lambda S/2 (FP32) or s = u_j . n S/2 - lambda S/2 and t = u_j . n S/2 (FP64).
-template <typename TJ> struct JvRows;
-template <> struct JvRows<float> { static constexpr int face = 4; };
-template <> struct JvRows<double> { static constexpr int face = 5; };
-
 // acc += 1/2 (J(Q_j) n - lambda I) S x_j, the off-diagonal block of Eq. (deri-matrix)
 // applied as a product (no stored 5x5 block): J(Q_j)(n S/2) x_j from j's primitives
 // (jv rows 0-5: u, v, w, H, (gamma-1)|u|^2/2, gamma-1) and the record of face p of cell i
-template <typename TV, typename TJ>
-__device__ __forceinline__ void offdiag_product(const TJ *__restrict__ jv, int N, int i, int p, int j, const TV *x,
+// (rows 6 + 4p + k: n S/2, lambda S/2)
+template <typename TV>
+__device__ __forceinline__ void offdiag_product(const float *__restrict__ jv, int N, int i, int p, int j, const TV *x,
                                                 TV *acc) {
   const TV u = jv[j], v = jv[(size_t)N + j], w = jv[2 * (size_t)N + j], H = jv[3 * (size_t)N + j];
   const TV phi = jv[4 * (size_t)N + j], g1 = jv[5 * (size_t)N + j];
-  const TJ *f = jv + (size_t)(6 + JvRows<TJ>::face * p) * N + i;
-  const TV nx = f[0], ny = f[N], nz = f[2 * (size_t)N];
-  const TV ls = JvRows<TJ>::face == 4 ? f[3 * (size_t)N] : f[(JvRows<TJ>::face - 1) * (size_t)N] - f[3 * (size_t)N];
+  const float *f = jv + (size_t)(6 + 4 * p) * N + i;
+  const TV nx = f[0], ny = f[N], nz = f[2 * (size_t)N], ls = f[3 * (size_t)N];
   const TV un = u * nx + v * ny + w * nz, nm = nx * x[1] + ny * x[2] + nz * x[3], um = u * x[1] + v * x[2] + w * x[3];
   const TV dp = g1 * (x[4] - um) + phi * x[0], t = nm - un * x[0];
   acc[0] += nm - ls * x[0];
@@ -31,7 +25,7 @@ __device__ __forceinline__ void offdiag_product(const TJ *__restrict__ jv, int N
 }
 
 // The same product in FP64 with what depends on the neighbour alone taken out of the sum
-// over faces: a vector x is kept as z = (x0, a, dp, x4) per cell,
+// over faces (rows 6 + 5p + k of the FP64 operands: n S/2, s, t): a vector x is kept as z = (x0, a, dp, x4) per cell,
 //   a = m - u x0,  dp = (gamma - 1)(x4 - u . a) - (gamma - 1)|u|^2/2 x0,
 // and with s = u . n S/2 - lambda S/2 and t = u . n S/2 (stored) the block takes 17 operations
 // instead of 28 (or 24 for a stored 5x5 block, whose 200 bytes per face it replaces with 40):
