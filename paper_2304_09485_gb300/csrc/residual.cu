@@ -32,23 +32,20 @@ namespace {
 
 constexpr int kBlock = 128;
 
-// primitive state of a Maxwellian: lam = rho / (2 p), il = 1 / (2 lam) = p / rho, ir = 1 / rho
-struct Prim { double rho, U, V, W, lam, il, ir; };
+// primitive state of a Maxwellian: il = p / rho (its variance), ir = 1 / rho
+struct Prim { double rho, U, V, W, il, ir; };
 
 // rho p of a conservative state, without a division
 __device__ __forceinline__ double rho_p(const double *Q, double g1) {
   return g1 * fma(Q[4], Q[0], -0.5 * fma(Q[1], Q[1], fma(Q[2], Q[2], Q[3] * Q[3])));
 }
-// from Q and rp = rho p: one reciprocal r = 1 / (rho^2 p) gives both 1/rho = rho p r and
-// lam = rho / (2p) = rho^3 r / 2
+// from Q and rp = rho p
 __device__ __forceinline__ Prim to_prim(const double *Q, double rp) {
   Prim p;
   p.rho = Q[0];
-  const double r = rcp(Q[0] * rp);
-  p.ir = rp * r;
+  p.ir = rcp(Q[0]);
   p.U = Q[1] * p.ir; p.V = Q[2] * p.ir; p.W = Q[3] * p.ir;
   p.il = rp * p.ir * p.ir;
-  p.lam = 0.5 * Q[0] * Q[0] * Q[0] * r;
   return p;
 }
 
@@ -202,8 +199,8 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 //   kap_0 = (D + tz R_0) / den,  kap_m = gm tz (R_m - R_0) / den,
 //   den = D + tz (g0 R_0 + gm sum R_m).
 // Keeping the projection in shared memory (110 doubles a thread on tetrahedra, 170 on
-// hexahedra) instead of projecting per variable: 28.5 -> 24.4 ms for 9.4M (cell, face) pairs
-// (2,359,296 tetrahedra), 1.24 -> 1.01 ms for 35,937 hexahedra; no spills (604 bytes before).
+// hexahedra) instead of projecting per variable: 28.5 -> 24.2 ms for 9.4M (cell, face) pairs
+// (2,359,296 tetrahedra), 1.24 -> 1.00 ms for 35,937 hexahedra; no spills (604 bytes before).
 // Blocks: any shape up to 256 threads fits on tetrahedra; on hexahedra two blocks of 64
 // fit an SM (85 KB each), one of 128, none of 256.
 constexpr int kReconMax = 256, kReconHex = 64;
@@ -234,7 +231,7 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
 #pragma unroll
     for (int c = 0; c < 5; c++) {
       Qi[c] = Q[(size_t)c * N + i];
-      Qs[c] = R >= 0 ? 0.5 * (Q[(size_t)c * N + L] + Q[(size_t)c * N + R]) : Qi[c];
+      Qs[c] = R >= 0 ? Q[(size_t)c * N + L] + Q[(size_t)c * N + R] : Qi[c];   // twice Q*: only ratios are taken
     }
     if (P.characteristic) {
       rot_in(T, Qs, Qsl);
@@ -278,6 +275,12 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
   double m2[6], xg[3 * NG];
 #pragma unroll
   for (int k = 0; k < 6; k++) m2[k] = m.m2[(size_t)k * N + i];
+  // beta_0 = |a|^2 + tr(M2 H^2) + sum of squared second derivatives as a quadratic form of
+  // the coefficients (xx, yy, zz, xy, xz, yz), H_xx = 2 a_xx: weights of the squares, and of
+  // the products by m_xy, m_xz, m_yz without (c) and with (f) a factor from a diagonal entry
+  const double w0 = fma(4.0, m2[0], 4.0), w1 = fma(4.0, m2[1], 4.0), w2 = fma(4.0, m2[2], 4.0);
+  const double w3 = m2[0] + m2[1] + 1.0, w4 = m2[0] + m2[2] + 1.0, w5 = m2[1] + m2[2] + 1.0;
+  const double c3 = 2.0 * m2[3], c4 = 2.0 * m2[4], c5 = 2.0 * m2[5], f3 = 2.0 * c3, f4 = 2.0 * c4, f5 = 2.0 * c5;
 #pragma unroll
   for (int k = 0; k < 3 * NG; k++) xg[k] = m.xg[(size_t)(slot * 3 * NG + k) * N + i];
   // weights of the sub-stencils (compact: one per face)
@@ -301,27 +304,26 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
 #pragma unroll
       for (int j = 0; j < 3; j++) lin[j] = ac[j];
     } else {
-      // smoothness indicators in the scaled frame: beta_0 = avg |grad P0|^2 + sum of squared second derivatives
-      const double H00 = 2.0 * ac[3], H11 = 2.0 * ac[4], H22 = 2.0 * ac[5], H01 = ac[6], H02 = ac[7], H12 = ac[8];
-      // avg |grad P0|^2 = |a|^2 + tr(M2 H^2) (M2: second moments, H symmetric)
-      const double s00 = H00 * H00, s11 = H11 * H11, s22 = H22 * H22;
-      const double S01 = fma(H00, H01, fma(H01, H11, H02 * H12));
-      const double S02 = fma(H00, H02, fma(H01, H12, H02 * H22));
-      const double S12 = fma(H01, H02, fma(H11, H12, H12 * H22));
-      const double s01 = H01 * H01, s02 = H02 * H02, s12 = H12 * H12, so = s01 + s02 + s12, sd = s00 + s11 + s22;
-      const double trd = fma(m2[0], s00 + (s01 + s02), fma(m2[1], s11 + (s01 + s12), m2[2] * (s22 + (s02 + s12))));
-      const double tro = fma(m2[3], S01, fma(m2[4], S02, m2[5] * S12));
-      const double beta0 = fma(ac[0], ac[0], fma(ac[1], ac[1], fma(ac[2], ac[2], fma(2.0, tro, trd) + (sd + so))));
+      // smoothness indicators in the scaled frame (beta_0 = avg |grad P0|^2 + sum of squared
+      // second derivatives), each with weno_eps added
+      const double xx = ac[3], yy = ac[4], zz = ac[5], xy = ac[6], xz = ac[7], yz = ac[8];
+      double d0 = fma(ac[0], ac[0], fma(ac[1], ac[1], fma(ac[2], ac[2], P.weno_eps)));
+      d0 = fma(xx, fma(w0, xx, fma(f3, xy, f4 * xz)), d0);
+      d0 = fma(xy, fma(w3, xy, fma(f3, yy, fma(c4, yz, c5 * xz))), d0);
+      d0 = fma(xz, fma(w4, xz, fma(f4, zz, c3 * yz)), d0);
+      d0 = fma(yy, fma(w1, yy, f5 * yz), d0);
+      d0 = fma(yz, fma(w5, yz, f5 * zz), d0);
+      d0 = fma(zz, w2 * zz, d0);
       double dm[NSUB], tz = 0.0;
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {
         const double b0 = pc[(9 + 3 * mm) * bd], b1 = pc[(10 + 3 * mm) * bd], b2 = pc[(11 + 3 * mm) * bd];
-        const double beta = fma(b0, b0, fma(b1, b1, b2 * b2));
-        if (valid >> mm & 1) tz += fabs(beta0 - beta);
-        dm[mm] = (valid >> mm & 1) ? beta + P.weno_eps : 1.0;
+        const double de = fma(b0, b0, fma(b1, b1, fma(b2, b2, P.weno_eps)));
+        if (valid >> mm & 1) tz += fabs(d0 - de);
+        dm[mm] = (valid >> mm & 1) ? de : 1.0;
       }
       tz *= iM;
-      double R[NSUB], pre = beta0 + P.weno_eps, R0 = 1.0, sum = 0.0;
+      double R[NSUB], pre = d0, R0 = 1.0, sum = 0.0;
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {               // R[mm] = d0 dm[0] ... dm[mm - 1]
         R[mm] = pre;
@@ -374,8 +376,9 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
 // Moments of the normalised Maxwellian of variance il = T = p / rho about (U, V, W),
 // in u over the half range (sgn = +1: u > 0, sgn = -1: u < 0) or the full one:
 //   M_n = <u^n>, M_{n+1} = U M_n + n T M_{n-1} (+ T del for n = 0),
-// del = sgn g(u = 0) the density at the end of the half range (0 for the full range); hd = del / 2.
-struct Mom { double m0, m1, m2, m3, m4, hd; };
+// del = sgn g(u = 0) the density at the end of the half range (0 for the full range); hd = del / 2,
+// h0 = -U del / (2T).
+struct Mom { double m0, m1, m2, m3, m4, hd, h0; };
 __device__ __forceinline__ void mom_up(const Prim &p, Mom &m) {
   m.m2 = fma(p.U, m.m1, p.il * m.m0);
   m.m3 = fma(p.U, m.m2, 2.0 * p.il * m.m1);
@@ -383,13 +386,18 @@ __device__ __forceinline__ void mom_up(const Prim &p, Mom &m) {
 }
 __device__ __forceinline__ Mom mom_full(const Prim &p) {
   Mom m;
-  m.m0 = 1.0; m.m1 = p.U; m.hd = 0.0;
+  m.m0 = 1.0; m.m1 = p.U; m.hd = 0.0; m.h0 = 0.0;
   mom_up(p, m);
   return m;
 }
-// <u^0>, T del and <u^1> = U <u^0> + T del over sgn u > 0
-__device__ __forceinline__ void half01(double U, double lam, double sgn, double &m0, double &td, double &m1) {
-  const double rs = rsqrt64(lam), y = lam * rs * U, x = sgn > 0.0 ? -y : y, e = exp64(-y * y);
+// <u^0>, <u^1> = U <u^0> + T del, del / 2 = sgn exp(-y^2) / (2 sqrt(2 pi T)) and y = U / sqrt(2T)
+// over sgn u > 0; rs = 1 / sqrt(2T)
+__device__ __forceinline__ void half01(double U, double T, double sgn, double &m0, double &m1, double &hd, double &y,
+                                       double &rs) {
+  const double T2 = 2.0 * T;
+  rs = rsqrt64(T2);
+  y = rs * U;
+  const double x = sgn > 0.0 ? -y : y, e = exp64(-y * y);
   if (((unsigned)__double2hiint(x) & 0x7fffffffu) < kErfcRange) {
     m0 = half_erfc64(x);
   } else {
@@ -397,14 +405,14 @@ __device__ __forceinline__ void half01(double U, double lam, double sgn, double 
     const double t = erfcx(fabs(x)) * e;
     m0 = 0.5 * (x >= 0.0 ? t : 2.0 - t);
   }
-  td = sgn * 0.28209479177387814347 * e * rs;          // 1 / (2 sqrt(pi))
-  m1 = fma(U, m0, td);
+  hd = sgn * 0.28209479177387814347 * e * rs;          // 1 / (2 sqrt(pi))
+  m1 = fma(U, m0, T2 * hd);
 }
 __device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
   Mom m;
-  double td;
-  half01(p.U, p.lam, sgn, m.m0, td, m.m1);
-  m.hd = p.lam * td;
+  double y, rs;
+  half01(p.U, p.il, sgn, m.m0, m.m1, m.hd, y, rs);
+  m.h0 = -2.0 * y * rs * m.hd;
   mom_up(p, m);
   return m;
 }
@@ -429,7 +437,14 @@ __device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
 //   psi_4 = psi'_4 + V psi'_2 + W psi'_3 + (V^2 + W^2)/2 psi'_0.
 struct Dir { double r, u, v, w, p; };    // drho, rho dU, rho dV, rho dW, dp along one axis of the face frame
 
-// out += L x (x in the tangential frame of p, x[4] twice the component)
+// out = L x, out += L x (x in the tangential frame of p, x[4] twice the component)
+__device__ __forceinline__ void from_frame(const Prim &p, const double *x, double *out) {
+  out[0] = x[0];
+  out[1] = x[1];
+  out[2] = fma(p.V, x[0], x[2]);
+  out[3] = fma(p.W, x[0], x[3]);
+  out[4] = fma(p.V, x[2], fma(p.W, x[3], 0.5 * fma(fma(p.V, p.V, p.W * p.W), x[0], x[4])));
+}
 __device__ __forceinline__ void acc_from_frame(const Prim &p, const double *x, double *out) {
   const double q = fma(p.V, p.V, p.W * p.W);
   out[0] += x[0];
@@ -493,7 +508,7 @@ __device__ __forceinline__ void acc_flux(const Prim &p, const Mom &m, const Dir 
 // the moments sum_d <u_d d_d psi'> without the part of conv (u d_0, v' d_1, w' d_2)
 __device__ __forceinline__ void own_moments(const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
                                             double *z) {
-  const double T = p.il, hd = m.hd, del = 2.0 * hd, h0 = -p.lam * p.U * del;
+  const double T = p.il, hd = m.hd, del = 2.0 * hd, h0 = m.h0;
   const double E1 = fma(d[0].r, m.m1, fma(d[0].u, m.m0, k.s0 * hd));
   const double E2 = fma(d[0].r, m.m2, fma(2.0 * d[0].u, m.m1, k.s0 * m.m0));
   const double E3 = fma(d[0].r, m.m3, 3.0 * fma(d[0].u, m.m2, k.s0 * m.m1));
@@ -508,7 +523,7 @@ __device__ __forceinline__ void own_moments(const Prim &p, const Mom &m, const D
 // W += c rho <psi> + e sum_d <u_d d_d psi> + f <d_t psi>, z from own_moments
 __device__ __forceinline__ void acc_state(const Prim &p, const Mom &m, const Slopes &k, const double *z, double K2, double c,
                                           double e, double f, double *W) {
-  const double T = p.il, ef = e - f, hd = m.hd, del = 2.0 * hd, h0 = -p.lam * p.U * del;
+  const double T = p.il, ef = e - f, hd = m.hd, del = 2.0 * hd, h0 = m.h0;
   const double br = fma(c, p.rho, fma(ef, k.cr, -f * k.qr)), bu = fma(ef, k.cu, -f * k.qu);
   const double bv = fma(ef, k.cv, -f * k.qv), bw = fma(ef, k.cw, -f * k.qw), bs = fma(ef, k.cs, -f * k.qs);
   const double B0 = fma(br, m.m0, fma(bu, del, bs * h0));
@@ -551,8 +566,8 @@ __device__ void image_state(const KParams &P, int tag, const double *T, const Pr
   // Maxwellian; otherwise the image has the cell's pressure and temperature
   double rg = l.rho;
   if (T_odd) {
-    double m0, td, Mg;
-    half01(l.U, 0.5 * rcp(Tg), 1.0, m0, td, Mg);
+    double m0, Mg, hd, y, rs;
+    half01(l.U, Tg, 1.0, m0, Mg, hd, y, rs);
     rg = l.rho * M1 * rcp(Mg);
   }
   Wr[0] = rg;
@@ -574,14 +589,14 @@ __device__ __forceinline__ void image_slopes(int tag, const Prim &l, const Prim 
     return;
   }
   const bool T_odd = tag == HGKS_BC_WALL_ISO || tag == HGKS_BC_WALL_LID;
-  const double rr = g.rho * l.ir, ps = T_odd ? rr * g.il * (2.0 * l.lam) : 1.0;
+  const double rr = g.rho * l.ir, ps = T_odd ? rr * g.il * rcp(l.il) : 1.0, ig = rcp(g.il);
   const double vt = tag == HGKS_BC_SLIP ? rr : -rr;
   const double tt = held ? 0.0 : (T_odd ? -rr : rr);     // rho_g dT_g from rho dT
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     const double sn = a == 0 ? -1.0 : 1.0;
     const double s = fma(-l.il, d[a].r, d[a].p), dp = sn * ps * d[a].p;
-    d[a].r = 2.0 * g.lam * fma(-sn * tt, s, dp);
+    d[a].r = ig * fma(-sn * tt, s, dp);
     d[a].u *= -sn * rr;
     d[a].v *= sn * vt;
     d[a].w *= sn * vt;
@@ -589,44 +604,52 @@ __device__ __forceinline__ void image_slopes(int tag, const Prim &l, const Prim 
   }
 }
 
-// Derivatives of side s (a Maxwellian with primitive state p) at one Gauss point, from the
-// reconstruction's derivatives `in` (15 rows of pitch F). In characteristic variables
-// R* q back-projects to conservative derivatives, whose primitive form with respect to the
-// side's own state follows directly: with (du, dv, dw) = u* - (U, V, W) and c* the sound
-// speed of the projection state, dp = (gamma - 1)(dE - u . dm + |u|^2/2 drho) takes five
-// products instead of the fourteen of R* and nine of the change of variables.
-__device__ __forceinline__ void load_dirs(const KParams &P, const Eig &e, const double *T, const Prim &p,
-                                          const double *__restrict__ in, size_t F, Dir *d) {
+// Derivatives of a Maxwellian with primitive state p from the reconstruction's derivatives q
+// along the three axes. In characteristic variables R* q back-projects to conservative
+// derivatives, whose primitive form with respect to p follows directly: with (du, dv, dw) =
+// u* - (U, V, W) and c* the sound speed of the projection state, dp = (gamma - 1)(dE - u . dm +
+// |u|^2/2 drho) takes five products instead of the fourteen of R* and nine of the change of variables.
+__device__ __forceinline__ void dirs_of(const KParams &P, const Eig &e, const double *T, const Prim &p, const double (*q)[5],
+                                        Dir *d) {
   const double g1 = P.g1;
   if (P.characteristic) {
     const double du = e.u - p.U, dv = e.v - p.V, dw = e.w - p.W;
     const double gu = g1 * du, gv = g1 * dv, gw = g1 * dw, h = 0.5 * fma(gu, du, fma(gv, dv, gw * dw)), a2 = e.a * e.a;
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-      double q[5];
-#pragma unroll
-      for (int c = 0; c < 5; c++) q[c] = in[(size_t)(5 * k + c) * F];
-      const double ad = e.a * (q[4] - q[0]), t = q[0] + q[4], r = t + q[1];
+      const double ad = e.a * (q[k][4] - q[k][0]), t = q[k][0] + q[k][4], r = t + q[k][1];
       d[k].r = r;
       d[k].u = fma(du, r, ad);
-      d[k].v = fma(dv, r, q[2]);
-      d[k].w = fma(dw, r, q[3]);
-      d[k].p = fma(a2, t, fma(h, r, fma(gu, ad, fma(gv, q[2], gw * q[3]))));
+      d[k].v = fma(dv, r, q[k][2]);
+      d[k].w = fma(dw, r, q[k][3]);
+      d[k].p = fma(a2, t, fma(h, r, fma(gu, ad, fma(gv, q[k][2], gw * q[k][3]))));
     }
   } else {
     const double h = 0.5 * fma(p.U, p.U, fma(p.V, p.V, p.W * p.W));
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-      double q[5], x[5];
-#pragma unroll
-      for (int c = 0; c < 5; c++) q[c] = in[(size_t)(5 * k + c) * F];
-      rot_in(T, q, x);
+      double x[5];
+      rot_in(T, q[k], x);
       d[k].r = x[0];
       d[k].u = fma(-p.U, x[0], x[1]);
       d[k].v = fma(-p.V, x[0], x[2]);
       d[k].w = fma(-p.W, x[0], x[3]);
       d[k].p = g1 * (x[4] - p.U * x[1] - p.V * x[2] - p.W * x[3] + h * x[0]);
     }
+  }
+}
+// d, derivatives with respect to a state of velocity p, with respect to Q0 (velocity p0): a
+// change of the reference velocity by (du, dv, dw) adds (0, du r, dv r, dw r,
+// (gamma - 1)(du . m + |du|^2 r / 2)); added to d0
+__device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim &p0, const Dir *d, double (*d0)[5]) {
+  const double du = p.U - p0.U, dv = p.V - p0.V, dw = p.W - p0.W, h = 0.5 * fma(du, du, fma(dv, dv, dw * dw));
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    d0[a][0] += d[a].r;
+    d0[a][1] += fma(du, d[a].r, d[a].u);
+    d0[a][2] += fma(dv, d[a].r, d[a].v);
+    d0[a][3] += fma(dw, d[a].r, d[a].w);
+    d0[a][4] += fma(g1, fma(du, d[a].u, fma(dv, d[a].v, fma(dw, d[a].w, h * d[a].r))), d[a].p);
   }
 }
 
@@ -638,7 +661,8 @@ __device__ __forceinline__ void load_dirs(const KParams &P, const Eig &e, const 
 // are read where they are used, so one side's fifteen are live at a time. Against slopes
 // solved for each axis and summed with moments up to u^6: 37.5 -> 24.5 ms at 14.2M Gauss
 // points (inviscid, 2,359,296 tetrahedra), 1.22 -> 0.74 ms at 295k (viscous, compact scheme);
-// with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms.
+// with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms;
+// with g_0's derivatives from the sum of the characteristic ones 19.1 and 0.61 ms.
 template <bool BATCH, class S, bool COMPACT>
 __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                   const double *__restrict__ dt, const double *__restrict__ wface,
@@ -669,7 +693,7 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
     for (int c = 0; c < 5; c++) {
       QL[c] = Q[(size_t)c * N + L];
       QR[c] = inner ? Q[(size_t)c * N + R] : QL[c];
-      Qs[c] = inner ? 0.5 * (QL[c] + QR[c]) : QL[c];
+      Qs[c] = inner ? QL[c] + QR[c] : QL[c];             // twice Q*: only ratios are taken
     }
     rot_in(T, Qs, Qsl);
     e = eig_of(Qsl, P.gamma, g1);
@@ -703,10 +727,10 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   // compatibility condition: Q0 = int_{u>0} psi g_l + int_{u<0} psi g_r
   Prim p0;
   {
-    double Q0[5] = {0, 0, 0, 0, 0};
+    double Q0[5];
     const double xl[5] = {pl.rho * ml.m0, pl.rho * ml.m1, 0.0, 0.0, pl.rho * fma(K2 * pl.il, ml.m0, ml.m2)};
     const double xr[5] = {pr.rho * mr.m0, pr.rho * mr.m1, 0.0, 0.0, pr.rho * fma(K2 * pr.il, mr.m0, mr.m2)};
-    acc_from_frame(pl, xl, Q0);
+    from_frame(pl, xl, Q0);
     acc_from_frame(pr, xr, Q0);
     p0 = to_prim(Q0, rho_p(Q0, g1));
   }
@@ -724,12 +748,15 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   const bool prandtl = P.fix_prandtl;
   const double ts = P.tstar_end ? dtf : 0.0, es = P.tstar_end ? eta : 1.0;   // exp(-t* / tau)
   double Fl[5] = {0, 0, 0, 0, 0}, Wb[5] = {0, 0, 0, 0, 0}, Pt[5] = {0, 0, 0, 0, 0};
-  // derivatives of g_0: the mean of both sides' conservative derivatives, taken with
-  // respect to Q0 (a change of the reference velocity by (du, dv, dw) adds
-  // (0, du r, dv r, dw r, (gamma - 1)(du . m + |du|^2 r / 2)))
-  Dir d[3], d0[3];
+  // The derivatives of g_0 are the mean of both sides' conservative derivatives. They enter
+  // linearly, so their sum is taken and the time coefficients halved. An interior face sums the
+  // characteristic derivatives (which share R*) and converts the sum to Q0's primitive form;
+  // other faces sum each side's primitive ones shifted to Q0's velocity.
+  const bool sums = inner && P.characteristic;
+  Dir d[3];
+  double q0[3][5];
 #pragma unroll
-  for (int a = 0; a < 3; a++) d0[a] = Dir{0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = 0.0;
   Prim pk = pl;
   Mom mk = ml;
   double C = c4, Ce = -c5, Cf = -dtf * k4;              // flux: c rho <u psi> + e sum <u u_d d_d psi> + f <u d_t psi>
@@ -739,29 +766,34 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
     if (s < 2) {
       if (s == 1 && !inner) {
         image_slopes(m.ftag[f], pl, pr, held, d);
-      } else if (bad >> s & 1) {
-#pragma unroll
-        for (int a = 0; a < 3; a++) d[a] = Dir{0.0, 0.0, 0.0, 0.0, 0.0};
       } else {
-        load_dirs(P, e, T, pk, wface + ((size_t)(s * NG + g) * kFaceState + 5) * F + f, F, d);
-      }
-      const double hu = 0.5 * (pk.U - p0.U), hv = 0.5 * (pk.V - p0.V), hw = 0.5 * (pk.W - p0.W);
-      const double hg = hu * hu + hv * hv + hw * hw;    // |du|^2 / 4
+        const double *in = wface + ((size_t)(s * NG + g) * kFaceState + 5) * F + f;
+        double q[3][5];
 #pragma unroll
-      for (int a = 0; a < 3; a++) {
-        d0[a].r = fma(0.5, d[a].r, d0[a].r);
-        d0[a].u = fma(0.5, d[a].u, fma(hu, d[a].r, d0[a].u));
-        d0[a].v = fma(0.5, d[a].v, fma(hv, d[a].r, d0[a].v));
-        d0[a].w = fma(0.5, d[a].w, fma(hw, d[a].r, d0[a].w));
-        d0[a].p = fma(0.5, d[a].p, fma(g1, fma(hu, d[a].u, fma(hv, d[a].v, fma(hw, d[a].w, hg * d[a].r))), d0[a].p));
+        for (int a = 0; a < 15; a++) q[a / 5][a % 5] = bad >> s & 1 ? 0.0 : in[(size_t)a * F];
+        dirs_of(P, e, T, pk, q, d);
+        if (sums) {
+          if (s == 0) {
+#pragma unroll
+            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = q[a / 5][a % 5];
+          } else {
+#pragma unroll
+            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] += q[a / 5][a % 5];
+          }
+        }
       }
+      if (!sums) add_shifted(g1, pk, p0, d, q0);
     } else {
-#pragma unroll
-      for (int a = 0; a < 3; a++) d[a] = d0[a];
       pk = p0;
       mk = mom_full(p0);
-      C = c1; Ce = c2; Cf = c3;
-      A = 1.0 - es; Ae = fma(ts + tau, es, -tau); Af = ts - tau + tau * es;
+      if (sums) {
+        dirs_of(P, e, T, pk, q0, d);
+      } else {
+#pragma unroll
+        for (int a = 0; a < 3; a++) d[a] = Dir{q0[a][0], q0[a][1], q0[a][2], q0[a][3], q0[a][4]};
+      }
+      C = c1; Ce = 0.5 * c2; Cf = 0.5 * c3;
+      A = 1.0 - es; Ae = 0.5 * fma(ts + tau, es, -tau); Af = 0.5 * (ts - tau + tau * es);
     }
     const Slopes k = slopes_of(pk, g1, d);
     acc_flux(pk, mk, d, k, K2, K4, C, Ce, Cf, Fl);
