@@ -14,6 +14,7 @@
 #include <cmath>
 #include <type_traits>
 #include "hgks_internal.h"
+#include "fp64.cuh"
 #include "givens.cuh"
 #include "offdiag.cuh"
 
@@ -64,16 +65,33 @@ __device__ __forceinline__ void mesh_sum(T v, const BatchDev &b, T *part, double
   }
 }
 
+// 1 / h (0 for h == 0) for all threads of a block: one FP64 division instead of one per warp
+template <typename T>
+__device__ __forceinline__ T mesh_inverse(double h) {
+  __shared__ T ih;
+  if (threadIdx.x == 0) ih = h != 0.0 ? (T)(1.0 / h) : T(0);
+  __syncthreads();
+  return ih;
+}
+
 enum { kSpmv = 0, kJacobi = 1, kNeumann = 2, kE = 3, kNegE = 4 };   // as k_apply of the single-mesh path
 // SpMV / Jacobi sweep over the merged cells with an optional per-mesh (y, dotv)
-template <typename TM, typename TV, typename TO, int Mode, bool First, int NF>
+// Scaled: x is w and v = w / h(mesh) (0 for h == 0) is formed on the way, as k_apply
+template <typename TM, typename TV, typename TO, int Mode, bool First, bool Scaled, int NF>
 __global__ void __launch_bounds__(kB) k_bapply(DevMesh m, BatchDev bd, const TM *__restrict__ off,
                                                const TM *__restrict__ dval, const TM *__restrict__ dinv,
                                                const TV *__restrict__ b, const TV *__restrict__ x, TO *__restrict__ y,
-                                               const TO *__restrict__ dotv, TO *part, double *dot_out, int stride) {
+                                               const TO *__restrict__ dotv, TO *part, double *dot_out, int stride,
+                                               const double *__restrict__ h, TO *__restrict__ v) {
   const int N = m.N;
   const int i = blockIdx.x * kB + threadIdx.x;
   if (!bd.active[bd.bmesh[blockIdx.x]]) return;
+  TV ih = TV(1);
+  if constexpr (Scaled) {
+    ih = mesh_inverse<TV>(h[(size_t)bd.bmesh[blockIdx.x] * stride]);
+#pragma unroll
+    for (int r = 0; r < 5; r++) v[(size_t)r * N + i] = x[(size_t)r * N + i] * ih;
+  }
   TV acc[5];
   const TV di = Mode == kSpmv ? (TV)dval[i] : TV(0);
 #pragma unroll
@@ -85,7 +103,7 @@ __global__ void __launch_bounds__(kB) k_bapply(DevMesh m, BatchDev bd, const TM 
     TV xj[5];
     const TV sj = First ? (TV)dinv[j] : TV(1);
 #pragma unroll
-    for (int c = 0; c < 5; c++) xj[c] = First ? sj * b[(size_t)c * N + j] : x[(size_t)c * N + j];
+    for (int c = 0; c < 5; c++) xj[c] = First ? sj * b[(size_t)c * N + j] : Scaled ? x[(size_t)c * N + j] * ih : x[(size_t)c * N + j];
     if constexpr (std::is_same<TM, float>::value) {
       offdiag_product<TV>(reinterpret_cast<const float *>(off), N, i, p, j, xj, acc);
     } else {
@@ -116,15 +134,24 @@ __global__ void __launch_bounds__(kB) k_bapply(DevMesh m, BatchDev bd, const TM 
 }
 
 // k_bapply for the batch's cell kind (4 or 6 off-diagonal blocks per row)
-template <typename TM, typename TV, typename TO, int Mode, bool First>
+template <typename TM, typename TV, typename TO, int Mode, bool First, bool Scaled = false>
 void bapply(unsigned g, cudaStream_t st, const DevMesh &m, const BatchDev &bd, const TM *off, const TM *dval,
-            const TM *dinv, const TV *b, const TV *x, TO *y, const TO *dotv, TO *part, double *dot_out, int stride) {
+            const TM *dinv, const TV *b, const TV *x, TO *y, const TO *dotv, TO *part, double *dot_out, int stride,
+            const double *h = nullptr, TO *v = nullptr) {
   if (m.hex)
-    k_bapply<TM, TV, TO, Mode, First, HexShape::NF><<<g, kB, 0, st>>>(m, bd, off, dval, dinv, b, x, y, dotv, part,
-                                                                      dot_out, stride);
+    k_bapply<TM, TV, TO, Mode, First, Scaled, HexShape::NF><<<g, kB, 0, st>>>(m, bd, off, dval, dinv, b, x, y, dotv, part,
+                                                                              dot_out, stride, h, v);
   else
-    k_bapply<TM, TV, TO, Mode, First, TetShape::NF><<<g, kB, 0, st>>>(m, bd, off, dval, dinv, b, x, y, dotv, part,
-                                                                      dot_out, stride);
+    k_bapply<TM, TV, TO, Mode, First, Scaled, TetShape::NF><<<g, kB, 0, st>>>(m, bd, off, dval, dinv, b, x, y, dotv, part,
+                                                                              dot_out, stride, h, v);
+}
+
+// y = x rounded, for every mesh that iterates
+__global__ void __launch_bounds__(kB) k_bround(int N, BatchDev bd, const double *__restrict__ x, float *__restrict__ y) {
+  const int i = blockIdx.x * kB + threadIdx.x;
+  if (!bd.active[bd.bmesh[blockIdx.x]]) return;
+#pragma unroll
+  for (int c = 0; c < 5; c++) y[(size_t)c * N + i] = (float)x[(size_t)c * N + i];
 }
 
 // w -= h(mesh) v (if v); out(mesh) = (w, x) or ||w|| (self; x is not read then,
@@ -222,20 +249,13 @@ __global__ void __launch_bounds__(kB) k_bmdot(int N, BatchDev bd, const T *__res
   if (threadIdx.x == 0) bd.counters[mesh] = 0u;
 }
 
-// one thread per mesh: row j of the Gram matrix from g, then h_ij by forward substitution
+// one warp per mesh: column j of the Gram matrix from g, then h_ij by forward substitution
 __global__ void k_bmgs_coef(BatchDev bd, int j, int mk, double *__restrict__ hs, int hz, int aoff, int goff,
                             int gram_off) {
-  const int mesh = blockIdx.x * blockDim.x + threadIdx.x;
+  const int mesh = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (mesh >= bd.nmesh || !bd.active[mesh]) return;
-  double *rec = hs + (size_t)mesh * hz, *G = rec + gram_off;
-  const double *a = rec + aoff, *g = rec + goff;
-  const int ld = mk + 1;
-  for (int k = 0; k < j; k++) G[k * ld + j] = g[k];
-  for (int i = 0; i <= j; i++) {
-    double h = a[i];
-    for (int k = 0; k < i; k++) h -= rec[k * mk + j] * G[k * ld + i];
-    rec[i * mk + j] = h;
-  }
+  double *rec = hs + (size_t)mesh * hz;
+  mgs_coef_warp(threadIdx.x % 32, j, mk, mk + 1, rec + aoff, rec + goff, rec + gram_off, rec);
 }
 
 // w -= sum_{k <= j} h_kj(mesh) v_k in the order of k, then h_{j+1,j}(mesh) = ||w||
@@ -266,8 +286,7 @@ __global__ void __launch_bounds__(kB) k_bscale(int N, BatchDev bd, const T *__re
                                                int hstride, T *__restrict__ v) {
   const int i = blockIdx.x * kB + threadIdx.x;
   if (!bd.active[bd.bmesh[blockIdx.x]]) return;
-  const double hv = h[(size_t)bd.bmesh[blockIdx.x] * hstride];
-  const T ih = hv != 0.0 ? (T)(1.0 / hv) : T(0);
+  const T ih = mesh_inverse<T>(h[(size_t)bd.bmesh[blockIdx.x] * hstride]);
 #pragma unroll
   for (int c = 0; c < 5; c++) v[(size_t)c * N + i] = w[(size_t)c * N + i] * ih;
 }
@@ -408,15 +427,28 @@ void bprecondition(const DevMesh &m, BatchState &bs, const BBuf<T> &k, int sweep
 // w = P^{-1} A v for a Krylov vector v of every mesh: w = v + E (-E)^k v with
 // E = D^{-1} O (the sign in the first product), as neumann_t of the single-mesh
 // path; (w, dotv) per mesh from the last launch
+// (with h and sweeps > 0, v = w / h per mesh is formed on the way)
 template <typename T>
-void bneumann(const DevMesh &m, BatchState &bs, const BBuf<T> &k, int sweeps, const T *v, T *w, const T *dotv,
+void bneumann(const DevMesh &m, BatchState &bs, const BBuf<T> &k, int sweeps, const double *h, T *v, T *w, const T *dotv,
               double *dot_out, cudaStream_t st) {
   const unsigned g = std::max(1, bs.b.nblocks);
   const int hz = bs.hsz;
-  const T *z = v;
+  const T *z = h ? w : v;
   for (int q = 0; q < sweeps; q++) {
     T *dst = (q % 2 == 0) ? k.t : k.t2;
     HGKS_PROF_BEGIN(K_JACOBI, st);
+    if constexpr (std::is_same<T, float>::value)
+      if (q == 0 && h) {
+        if (sweeps % 2 == 1)
+          bapply<T, T, T, kNegE, false, true>(g, st, m, bs.b, k.off, k.dval, k.dinv, nullptr, z, dst, nullptr, k.part,
+                                              nullptr, hz, h, v);
+        else
+          bapply<T, T, T, kE, false, true>(g, st, m, bs.b, k.off, k.dval, k.dinv, nullptr, z, dst, nullptr, k.part,
+                                           nullptr, hz, h, v);
+        HGKS_PROF_END(K_JACOBI, st);
+        z = dst;
+        continue;
+      }
     if (q == 0 && sweeps % 2 == 1)
       bapply<T, T, T, kNegE, false>(g, st, m, bs.b, k.off, k.dval, k.dinv, nullptr, z, dst, nullptr, k.part,
                                                          nullptr, hz);
@@ -445,8 +477,14 @@ void bgmres_t(const DevMesh &m, Scratch &s, BatchState &bs, const BBuf<T> &k, co
   for (int it = 0; it < p.restarts; it++) {
     cudaMemset2DAsync(H, sizeof(double) * hz, 0, sizeof(double) * (mk + 1) * mk, nm, st);
     HGKS_PROF_BEGIN(K_SPMV, st);
-    bapply<T, double, T, kSpmv, false>(g, st, m, bs.b, k.off, k.dval, k.dinv, rhs, dx, k.t, nullptr, nullptr,
-                                                            nullptr, hz);
+    bool product = true;
+    if constexpr (std::is_same<T, float>::value)
+      if (it == 0) {                       // dx = 0: the right-hand side itself
+        k_bround<<<g, kB, 0, st>>>(N, bs.b, rhs, k.t);
+        product = false;
+      }
+    if (product)
+      bapply<T, double, T, kSpmv, false>(g, st, m, bs.b, k.off, k.dval, k.dinv, rhs, dx, k.t, nullptr, nullptr, nullptr, hz);
     HGKS_PROF_END(K_SPMV, st);
     bprecondition<T>(m, bs, k, p.jacobi_sweeps, k.t, k.w, nullptr, nullptr, st);
     HGKS_PROF_BEGIN(K_DOT, st);
@@ -454,14 +492,21 @@ void bgmres_t(const DevMesh &m, Scratch &s, BatchState &bs, const BBuf<T> &k, co
     HGKS_PROF_END(K_DOT, st);
     if (it == 0) cudaMemcpy2DAsync(lres, sizeof(double) * hz, beta, sizeof(double) * hz, sizeof(double), nm,
                                    cudaMemcpyDeviceToDevice, st);
-    HGKS_PROF_BEGIN(K_SCALE, st);
-    k_bscale<T><<<g, kB, 0, st>>>(N, bs.b, k.w, beta, hz, k.V);
-    HGKS_PROF_END(K_SCALE, st);
+    // v_j = w / h: FP32 on the way of the first product, if there is one before w is written again
+    const bool on_the_way = std::is_same<T, float>::value && p.jacobi_sweeps > 0;
+    auto scale = [&](const double *h, T *v) {
+      if (on_the_way) return;
+      HGKS_PROF_BEGIN(K_SCALE, st);
+      k_bscale<T><<<g, kB, 0, st>>>(N, bs.b, k.w, h, hz, v);
+      HGKS_PROF_END(K_SCALE, st);
+    };
+    scale(beta, k.V);
     // FP32 vectors: MGS from one pass over the basis (HBM bound, about half the
     // bytes); FP64 vectors: one basis vector per pass (bound by the FP64 rate either way)
     constexpr bool one_pass = std::is_same<T, float>::value;
     for (int j = 0; j < mk; j++) {
-      bneumann<T>(m, bs, k, p.jacobi_sweeps, k.V + (size_t)j * vs, k.w, one_pass ? nullptr : k.V,
+      bneumann<T>(m, bs, k, p.jacobi_sweeps, on_the_way ? (j == 0 ? beta : H + j * mk + j - 1) : nullptr,
+                  k.V + (size_t)j * vs, k.w, one_pass ? nullptr : k.V,
                   one_pass ? nullptr : H + j, st);
       if constexpr (one_pass) {
         for (int k0 = 0; k0 <= j; k0 += kBatchMdot) {
@@ -471,7 +516,7 @@ void bgmres_t(const DevMesh &m, Scratch &s, BatchState &bs, const BBuf<T> &k, co
           HGKS_PROF_END(K_DOT, st);
         }
         HGKS_PROF_BEGIN(K_DOT, st);
-        k_bmgs_coef<<<(nm + 63) / 64, 64, 0, st>>>(bs.b, j, mk, bs.hs, hz, bs.a_off, bs.g_off, bs.gram_off);
+        k_bmgs_coef<<<(nm + 3) / 4, 128, 0, st>>>(bs.b, j, mk, bs.hs, hz, bs.a_off, bs.g_off, bs.gram_off);
         HGKS_PROF_END(K_DOT, st);
         HGKS_PROF_BEGIN(K_DOT, st);
         k_bmupdate<T><<<g, kB, 0, st>>>(N, bs.b, k.w, k.V, vs, j, mk, bs.hs, hz, k.part);
@@ -485,9 +530,7 @@ void bgmres_t(const DevMesh &m, Scratch &s, BatchState &bs, const BBuf<T> &k, co
                                          H + (i + 1) * mk + j, hz);
         HGKS_PROF_END(K_DOT, st);
       }
-      HGKS_PROF_BEGIN(K_SCALE, st);
-      k_bscale<T><<<g, kB, 0, st>>>(N, bs.b, k.w, H + (j + 1) * mk + j, hz, k.V + (size_t)(j + 1) * vs);
-      HGKS_PROF_END(K_SCALE, st);
+      if (j + 1 < mk) scale(H + (j + 1) * mk + j, k.V + (size_t)(j + 1) * vs);   // v_mk is not used
     }
     HGKS_PROF_BEGIN(K_GIVENS, st);
     k_bgivens<<<(nm + 63) / 64, 64, 0, st>>>(bs.b, mk, bs.hs, hz);

@@ -195,23 +195,38 @@ __device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, 
   }
 }
 
+// 1 / h in single precision (0 for h == 0) for all threads of a block: one FP64 division instead of one per warp
+__device__ __forceinline__ float block_inverse(const double *h) {
+  __shared__ float ih;
+  if (threadIdx.x == 0) ih = *h != 0.0 ? (float)(1.0 / *h) : 0.0f;
+  __syncthreads();
+  return ih;
+}
+
 // One product with the off-diagonal part of A from FP32 operands (mixed precision; FP64
 // vectors: gmres64.cu). Modes:
 //   kSpmv   : y = b - (d x + sum_p A_ip x_p)
 //   kJacobi : y = D^{-1} (b - sum_p A_ip x_p); FirstSweep: x_p = D^{-1} b at the neighbours
 //   kNeumann: y = b + D^{-1} sum_p A_ip x_p
 //   kE, kNegE: y = +- D^{-1} sum_p A_ip x_p
-// TV: type of b and x (and of the accumulation).
+// TV: type of b and x (and of the accumulation). Scaled: x is w, and v = w / h (0 for h == 0) is
+// formed on the way: stored for the cell itself, used for its neighbours (the same rounding), so a
+// new basis vector takes no launch of its own.
 enum { kSpmv = 0, kJacobi = 1, kNeumann = 2, kE = 3, kNegE = 4 };
 
-template <typename TV, int Mode, bool FirstSweep, int NF>
+template <typename TV, int Mode, bool FirstSweep, bool Scaled, int NF>
 __global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const float *__restrict__ jv,
                                                       const float *__restrict__ dval, const float *__restrict__ dinv,
                                                       const TV *__restrict__ b, const TV *__restrict__ x,
-                                                      float *__restrict__ y) {
+                                                      float *__restrict__ y, const double *__restrict__ h,
+                                                      float *__restrict__ v) {
   const int N = m.N;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const float ih = Scaled ? block_inverse(h) : 1.0f;
   if (i >= N) return;
+  if (Scaled)
+#pragma unroll
+    for (int r = 0; r < 5; r++) v[(size_t)r * N + i] = x[(size_t)r * N + i] * ih;
   TV acc[5];
   const TV di = Mode == kSpmv ? (TV)dval[i] : TV(0);
 #pragma unroll
@@ -223,7 +238,7 @@ __global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const float *__
     TV xj[5];
     const TV sj = FirstSweep ? (TV)dinv[j] : TV(1);
 #pragma unroll
-    for (int c = 0; c < 5; c++) xj[c] = FirstSweep ? sj * b[(size_t)c * N + j] : x[(size_t)c * N + j];
+    for (int c = 0; c < 5; c++) xj[c] = FirstSweep ? sj * b[(size_t)c * N + j] : Scaled ? x[(size_t)c * N + j] * ih : x[(size_t)c * N + j];
     offdiag_product<TV>(jv, N, i, p, j, xj, acc);
   }
 #pragma unroll
@@ -239,13 +254,16 @@ __global__ void __launch_bounds__(kCellBlock) k_apply(DevMesh m, const float *__
 }
 
 // k_apply for the mesh's cell kind (4 or 6 off-diagonal blocks per row)
-template <typename TV, int Mode, bool FirstSweep>
-void apply_launch(cudaStream_t st, const DevMesh &m, const Scratch &s, const TV *b, const TV *x, float *y) {
+template <typename TV, int Mode, bool FirstSweep, bool Scaled = false>
+void apply_launch(cudaStream_t st, const DevMesh &m, const Scratch &s, const TV *b, const TV *x, float *y,
+                  const double *h = nullptr, float *v = nullptr) {
   const unsigned grid = grid_for(m.N, kCellBlock);
   if (m.hex)
-    k_apply<TV, Mode, FirstSweep, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x, y);
+    k_apply<TV, Mode, FirstSweep, Scaled, HexShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x,
+                                                                                     y, h, v);
   else
-    k_apply<TV, Mode, FirstSweep, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x, y);
+    k_apply<TV, Mode, FirstSweep, Scaled, TetShape::NF><<<grid, kCellBlock, 0, st>>>(m, s.jv32, s.dval32, s.dinv32, b, x,
+                                                                                     y, h, v);
 }
 
 // y = x rounded to float
@@ -325,6 +343,28 @@ __global__ void __launch_bounds__(kBlock) k_axpy_dot(int64_t n, T *__restrict__ 
 // (used with FP32 vectors, see gmres_t).
 constexpr int kMdot = 8;              // basis vectors per k_mdot launch (register accumulators)
 
+// block_sum of each v[q] into tot[q] with two barriers for all of them: the warps' sums, then
+// eight lanes per value (the same order of additions)
+template <typename T>
+__device__ __forceinline__ void block_sum_all(T *v, T (*sh)[kBlock / 32], T *tot) {
+  constexpr int W = kBlock / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 2 * kMdot; q++) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if (lane == 0) sh[q][warp] = v[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * kMdot * W) {
+    T s = sh[threadIdx.x / W][threadIdx.x % W];
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, W);
+    if (threadIdx.x % W == 0) tot[threadIdx.x / W] = s;
+  }
+  __syncthreads();
+}
+
 // a[k] = (w, v_k) for k in [k0, k0 + nk), and g[k] = (v_j, v_k) for those k < j
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_mdot(int64_t n, const T *__restrict__ w, const T *__restrict__ V, int64_t vs,
@@ -367,11 +407,16 @@ __global__ void __launch_bounds__(kBlock) k_mdot(int64_t n, const T *__restrict_
   }
   // per block: 2 kMdot partials; the last block adds every slot's partials in block order
   __shared__ bool last;
+  __shared__ T sh[2 * kMdot][kBlock / 32], tot[2 * kMdot];
+  T v[2 * kMdot];
 #pragma unroll
-  for (int q = 0; q < 2 * kMdot; q++) {
-    const T bs = block_sum(q < kMdot ? sa[q] : sg[q - kMdot]);
-    if (threadIdx.x == 0) partials[(size_t)q * gridDim.x + blockIdx.x] = bs;
+  for (int q = 0; q < kMdot; q++) { v[q] = sa[q]; v[kMdot + q] = sg[q]; }
+  block_sum_all(v, sh, tot);
+  if (threadIdx.x < 2 * kMdot) {
+    partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = tot[threadIdx.x];
+    __threadfence();
   }
+  __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     last = (atomicAdd(count, 1u) == gridDim.x - 1);
@@ -379,30 +424,24 @@ __global__ void __launch_bounds__(kBlock) k_mdot(int64_t n, const T *__restrict_
   __syncthreads();
   if (!last) return;
   __threadfence();
+#pragma unroll
   for (int q = 0; q < 2 * kMdot; q++) {
-    const int kk = k0 + (q % kMdot);
-    const bool want = (q % kMdot) < nk && (q < kMdot || kk < j);   // uniform over the block
-    if (!want) continue;
-    T sum = T(0);
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) sum += ((volatile T *)partials)[(size_t)q * gridDim.x + b];
-    sum = block_sum(sum);
-    if (threadIdx.x == 0) (q < kMdot ? a : g)[kk] = (double)sum;
+    v[q] = T(0);
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) v[q] += ((volatile T *)partials)[(size_t)q * gridDim.x + b];
   }
+  block_sum_all(v, sh, tot);
+  const int q = threadIdx.x, kk = k0 + q % kMdot;
+  if (q < 2 * kMdot && q % kMdot < nk && (q < kMdot || kk < j)) (q < kMdot ? a : g)[kk] = (double)tot[q];
   if (threadIdx.x == 0) *count = 0u;
 }
 
 // the MGS coefficients of step j by forward substitution; column j of H and row
 // j of the basis Gram matrix G (leading dimension kGramLd, G[k][i] = (v_k, v_i), k < i)
 constexpr int kGramLd = 65;
+// (a lane per coefficient, two beyond 32: each h_i subtracts its terms in the order of k)
 __global__ void k_mgs_coef(int j, int mk, const double *__restrict__ a, const double *__restrict__ g,
                            double *__restrict__ G, double *__restrict__ H) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int k = 0; k < j; k++) G[k * kGramLd + j] = g[k];
-  for (int i = 0; i <= j; i++) {
-    double h = a[i];
-    for (int k = 0; k < i; k++) h -= H[k * mk + j] * G[k * kGramLd + i];
-    H[i * mk + j] = h;
-  }
+  mgs_coef_warp(threadIdx.x, j, mk, kGramLd, a, g, G, H);
 }
 
 // w -= sum_{k <= j} h_kj v_k in the order of k (MGS order), then h_{j+1,j} = ||w||
@@ -447,7 +486,7 @@ __global__ void k_scale(int64_t n, const T *__restrict__ w, const double *__rest
   typedef typename Vec16<T>::type TV;
   constexpr int L = Vec16<T>::n;
   const double hv = *h;
-  const T ih = hv != 0.0 ? (T)(1.0 / hv) : T(0);
+  const T ih = hv != 0.0 ? (T)rcp(hv) : T(0);
   const int64_t nv = n / L, stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nv; k += stride) {
     TV x = reinterpret_cast<const TV *>(w)[k];
@@ -610,13 +649,16 @@ void precondition_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, int sweeps, 
 // products with O instead of the product with A followed by k sweeps: the same
 // vector up to rounding, without the diagonal terms of A and the scaling of the
 // neighbours' values by D^{-1}. (FP32 vectors; FP64: launch_neumann_z.)
-void neumann32(const DevMesh &m, Scratch &s, const KBuf<float> &k, int sweeps, const float *v, float *w,
+// With h (and sweeps > 0) v = w / h is formed on the way, otherwise it is given.
+void neumann32(const DevMesh &m, Scratch &s, const KBuf<float> &k, int sweeps, const double *h, float *v, float *w,
                cudaStream_t st) {
-  const float *z = v, *none = nullptr;
+  const float *z = h ? w : v, *none = nullptr;
   for (int q = 0; q < sweeps; q++) {
     float *dst = (q % 2 == 0) ? k.t : k.t2;
     HGKS_PROF_BEGIN(K_JACOBI, st);
-    if (q == 0 && sweeps % 2 == 1) apply_launch<float, kNegE, false>(st, m, s, none, z, dst);
+    if (q == 0 && h && sweeps % 2 == 1) apply_launch<float, kNegE, false, true>(st, m, s, none, z, dst, h, v);
+    else if (q == 0 && h) apply_launch<float, kE, false, true>(st, m, s, none, z, dst, h, v);
+    else if (q == 0 && sweeps % 2 == 1) apply_launch<float, kNegE, false>(st, m, s, none, z, dst);
     else apply_launch<float, kE, false>(st, m, s, none, z, dst);
     HGKS_PROF_END(K_JACOBI, st);
     z = dst;
@@ -667,10 +709,13 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
     k_axpy_dot<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, nullptr, nullptr, k.w, 1, k.red, s.red_count, beta);
     HGKS_PROF_END(K_DOT, st);
     if (it == 0) cudaMemcpyAsync(lres, beta, sizeof(double), cudaMemcpyDeviceToDevice, st);
-    // v = w / h; FP64 with the assembled A: with the form that the products read
+    // v_j = w / h: FP64 with the assembled A, with the form that the products read; FP32 on the
+    // way of the first product, if there is one before w is written again
+    const bool on_the_way = one_pass && !fd && p.jacobi_sweeps > 0;
     auto scale = [&](const double *h, T *v) {
       if constexpr (!one_pass)
         if (!fd) return launch_scale_z(m, s, k.w, h, v, s.z[0], st);
+      if (on_the_way) return;
       HGKS_PROF_BEGIN(K_SCALE, st);
       k_scale<T><<<vg, kBlock, 0, st>>>(n, k.w, h, v);
       HGKS_PROF_END(K_SCALE, st);
@@ -678,12 +723,12 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
     scale(beta, k.V);
     for (int j = 0; j < mk; j++) {
       // w = P^{-1} A v_j (FP64: with the first block's coefficients from the last product)
-      const T *vj = k.V + (size_t)j * vs;
+      T *vj = k.V + (size_t)j * vs;
       if (fd) {
         fd_apply<T, T>(m, s, p, Q, G, vj, nullptr, k.t, st);
         precondition_t<T>(m, s, k, p.jacobi_sweeps, k.t, k.w, st);
       } else if constexpr (one_pass) {
-        neumann32(m, s, k, p.jacobi_sweeps, vj, k.w, st);
+        neumann32(m, s, k, p.jacobi_sweeps, on_the_way ? (j == 0 ? beta : H + j * mk + j - 1) : nullptr, vj, k.w, st);
       } else {
         launch_neumann_z(m, s, p.jacobi_sweeps, vj, k.w, j, mk, H + j, st);
       }
@@ -705,7 +750,7 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
       } else {
         launch_mgs_blocks(s, n, k.w, j, mk, H + j, !fd, st);
       }
-      scale(H + (j + 1) * mk + j, k.V + (size_t)(j + 1) * vs);
+      if (j + 1 < mk) scale(H + (j + 1) * mk + j, k.V + (size_t)(j + 1) * vs);   // v_mk is not used
     }
     HGKS_PROF_BEGIN(K_GIVENS, st);
     k_givens<<<1, 32, 0, st>>>(mk, H, beta, y, lres + 1);
