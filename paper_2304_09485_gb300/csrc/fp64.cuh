@@ -14,6 +14,22 @@
 
 namespace hgks {
 
+// An FMA of three registers takes 64 clocks; an addition, a multiplication and an FMA with a
+// constant operand take 76 (measured, 4 to 32 warps a SM). So the hot kernels multiply and add by
+// FMAs with -0.0 and 1.0 held in registers (the same results): loaded, or the compiler would turn
+// them back.
+static __device__ double kUnits[2] = {-0.0, 1.0};
+struct Units {
+  double nz, one;
+  __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, nz); }
+  __device__ __forceinline__ double add(double a, double b) const { return fma(a, one, b); }
+  __device__ __forceinline__ double sub(double a, double b) const { return fma(a, one, -b); }
+};
+__device__ __forceinline__ Units units() {
+  const volatile double *p = kUnits;
+  return {p[0], p[1]};
+}
+
 __device__ __forceinline__ float frcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -38,7 +54,7 @@ __device__ __forceinline__ void mantissa(int hi, int lo, float &m1, float &m2) {
 
 // 1 / x: a seed good to 2^-45 from two floats, one Newton step (its square is below
 // rounding, so the result is the rounded reciprocal but for rare ties)
-__device__ __forceinline__ double rcp(double x) {
+__device__ __forceinline__ double rcp(double x, double one = 1.0) {
   const int hi = __double2hiint(x), lo = __double2loint(x), e = (hi >> 20) & 0x7ff;
   if ((unsigned)(e - 2) >= 2040u) return 1.0 / x;
   float m1, m2;
@@ -46,7 +62,7 @@ __device__ __forceinline__ double rcp(double x) {
   const float r = fminf(fmaxf(frcp_approx(m1), 0.5f), 1.0f), t = fmaf(-m2, r, fmaf(-m1, r, 1.0f));
   const double y0 = join(r, r * t);
   const double y = __hiloint2double((__double2hiint(y0) + (1023 - e) * 0x100000) | (hi & 0x80000000), __double2loint(y0));
-  return fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, one), y);
 }
 
 // seed of 1/sqrt(x), good to 2^-45, for a positive normal x

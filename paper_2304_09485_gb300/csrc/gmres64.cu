@@ -70,14 +70,15 @@ __global__ void __launch_bounds__(kCell) k_scale_z(int N, const double *__restri
                                                    double *__restrict__ zv) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
+  const Units un = units();
   const double hv = *h, ih = hv != 0.0 ? rcp(hv) : 0.0;
   double y[5], z[6];
 #pragma unroll
   for (int c = 0; c < 5; c++) {
-    y[c] = w[(size_t)c * N + i] * ih;
+    y[c] = un.mul(w[(size_t)c * N + i], ih);
     v[(size_t)c * N + i] = y[c];
   }
-  z_of(cell_prim(jv, N, i), y, z);
+  z_of(un, cell_prim(jv, N, i), y, z);
   z_store(zv, N, i, z);
 }
 
@@ -86,15 +87,16 @@ __global__ void __launch_bounds__(kCell) k_z(int N, const double *__restrict__ j
                                              const double *__restrict__ x, double *__restrict__ zv) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
+  const Units un = units();
   double y[5], z[6];
 #pragma unroll
   for (int c = 0; c < 5; c++) y[c] = x[(size_t)c * N + i];
   if (dinv) {
     const double d = dinv[i];
 #pragma unroll
-    for (int c = 0; c < 5; c++) y[c] *= d;
+    for (int c = 0; c < 5; c++) y[c] = un.mul(y[c], d);
   }
-  z_of(cell_prim(jv, N, i), y, z);
+  z_of(un, cell_prim(jv, N, i), y, z);
   z_store(zv, N, i, z);
 }
 
@@ -110,24 +112,25 @@ __global__ void __launch_bounds__(kCell) k_zprod(int N, const int *__restrict__ 
                                                  double *__restrict__ y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
+  const Units un = units();
   double acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll
   for (int p = 0; p < NF; p++) {
     const int j = cnb[(size_t)p * N + i];
-    if (j >= 0) z_product(jv, N, i, p, j, x, acc);
+    if (j >= 0) z_product(un, jv, N, i, p, j, x, acc);
   }
   const double d = Mode == kE ? sign * dd[i] : dd[i];    // D^{-1}, or D for kSpmv
 #pragma unroll
   for (int c = 0; c < 5; c++) {
     const size_t k = (size_t)c * N + i;
-    if (Mode == kE) acc[c] *= d;
-    else if (Mode != kSpmv) acc[c] = d * (b[k] - acc[c]);
+    if (Mode == kE) acc[c] = un.mul(acc[c], d);
+    else if (Mode != kSpmv) acc[c] = un.mul(d, un.sub(b[k], acc[c]));
     else acc[c] = b ? b[k] - fma(d, x5[k], acc[c]) : fma(d, x5[k], acc[c]);
     if (Mode == kLast || Mode == kSpmv) y[k] = acc[c];
   }
   if (Mode == kE || Mode == kSweep) {
     double z[6];
-    z_of(cell_prim(jv, N, i), acc, z);
+    z_of(un, cell_prim(jv, N, i), acc, z);
     z_store(y, N, i, z);
   }
 }
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(kCell) k_zlast(int N, const int *__restrict__ 
                                                  unsigned *count) {
   constexpr int K = ND == 3 ? 4 : ND;
   __shared__ double sh[kCell / 32][K];
+  const Units un = units();
   double s[K];
 #pragma unroll
   for (int q = 0; q < K; q++) s[q] = 0.0;
@@ -157,7 +161,7 @@ __global__ void __launch_bounds__(kCell) k_zlast(int N, const int *__restrict__ 
 #pragma unroll
     for (int p = 0; p < NF; p++) {
       const int j = cnb[(size_t)p * N + i];
-      if (j >= 0) z_product(jv, N, i, p, j, x, acc);
+      if (j >= 0) z_product(un, jv, N, i, p, j, x, acc);
     }
     const double d = dinv[i];
 #pragma unroll
@@ -436,6 +440,7 @@ __global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
   GridShared &S = *reinterpret_cast<GridShared *>(smem);
   double *ws = reinterpret_cast<double *>(smem + sizeof(GridShared));   // !ONE: [5][C]
   const int tid = threadIdx.x, mk = a.mk, l = tid % LPC;
+  const Units un = units();
   const size_t N = a.N;
   const int c0 = blockIdx.x * a.C, nc = min(a.C, a.N - c0);             // this block's cells (nc <= 0: none)
   const int nwarps = min(kPT / 32, (a.C * LPC + 31) / 32);
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
     for (int q = 0; q < LF; q++) nb[q] = ONE ? own_nb[q] : a.cnb[q * N + i];
 #pragma unroll
     for (int q = 0; q < LF; q++)
-      if (nb[q] >= 0) z_product(a.jv, N, i, q * LPC + l, nb[q], z, t);
+      if (nb[q] >= 0) z_product(un, a.jv, N, i, q * LPC + l, nb[q], z, t);
     lane_components<LPC>(t, acc);
   };
   // z form of a cell's vector from its lanes' components
@@ -494,7 +499,7 @@ __global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
     for (int c = 0; c < 5; c++)
       y[c] = LPC == 1 ? x[c] : __shfl_sync(0xffffffffu, x[c / LPC], (tid & 31 & ~(LPC - 1)) | (c % LPC));
     if (ONE && i < 0) return;
-    z_of(ONE ? own_prim : cell_prim(a.jv, N, i), y, t);
+    z_of(un, ONE ? own_prim : cell_prim(a.jv, N, i), y, t);
 #pragma unroll
     for (int k = 0; k < 6; k++)
       if (LPC == 1 || k % LPC == l) z[k * N + i] = t[k];
@@ -564,7 +569,7 @@ __global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
 #pragma unroll
         for (int k = 0; k < CP; k++)
           if (mine(i, k)) {
-            w[k] *= ih;
+            w[k] = un.mul(w[k], ih);
             a.V[(size_t)j * a.vs + at(i, k)] = w[k];
           }
       });
@@ -576,7 +581,7 @@ __global__ void __launch_bounds__(kPT + 32, 1) k_gmres_grid(GridSolve a) {
           off(i, zs, acc);
           const double d = q == 0 ? sc * dinv(i) : dinv(i);
 #pragma unroll
-          for (int k = 0; k < CP; k++) acc[k] *= d;
+          for (int k = 0; k < CP; k++) acc[k] = un.mul(acc[k], d);
           put_z(zd, i, acc);
         });
         if (!grid_barrier(a, S, gen)) return;

@@ -1,6 +1,7 @@
 // Product form of the off-diagonal Jacobian blocks.
 #pragma once
 #include <cuda_runtime.h>
+#include "fp64.cuh"
 
 namespace hgks {
 
@@ -34,12 +35,12 @@ struct CellPrim { double u, v, w, H, phi, g1; };
 __device__ __forceinline__ CellPrim cell_prim(const double *__restrict__ jv, size_t N, int i) {
   return {jv[i], jv[N + i], jv[2 * N + i], jv[3 * N + i], jv[4 * N + i], jv[5 * N + i]};
 }
-__device__ __forceinline__ void z_of(const CellPrim &q, const double *y, double *z) {
+__device__ __forceinline__ void z_of(const Units &un, const CellPrim &q, const double *y, double *z) {
   z[0] = y[0];
   z[1] = fma(-q.u, y[0], y[1]);
   z[2] = fma(-q.v, y[0], y[2]);
   z[3] = fma(-q.w, y[0], y[3]);
-  z[4] = fma(q.g1, fma(-q.u, z[1], fma(-q.v, z[2], fma(-q.w, z[3], y[4]))), -q.phi * y[0]);
+  z[4] = fma(q.g1, fma(-q.u, z[1], fma(-q.v, z[2], fma(-q.w, z[3], y[4]))), un.mul(-q.phi, y[0]));
   z[5] = y[4];
 }
 __device__ __forceinline__ void z_store(double *zv, size_t N, int i, const double *z) {
@@ -47,13 +48,13 @@ __device__ __forceinline__ void z_store(double *zv, size_t N, int i, const doubl
   for (int k = 0; k < 6; k++) zv[k * N + i] = z[k];
 }
 // zv is not const __restrict__: other blocks of the same launch may write it before a grid barrier
-__device__ __forceinline__ void z_product(const double *__restrict__ jv, size_t N, int i, int p, int j, const double *zv,
+__device__ __forceinline__ void z_product(const Units &un, const double *__restrict__ jv, size_t N, int i, int p, int j, const double *zv,
                                           double *acc) {
   const double *f = jv + (6 + 5 * (size_t)p) * N + i;
   const double nx = f[0], ny = f[N], nz = f[2 * N], s = f[3 * N], t = f[4 * N];
   const double x0 = zv[j], a0 = zv[N + j], a1 = zv[2 * N + j], a2 = zv[3 * N + j], dp = zv[4 * N + j], x4 = zv[5 * N + j];
-  const double r = fma(nx, a0, fma(ny, a1, nz * a2)), r0 = fma(s, x0, r);
-  acc[0] += r0;
+  const double r = fma(nx, a0, fma(ny, a1, un.mul(nz, a2))), r0 = fma(s, x0, r);
+  acc[0] = un.add(r0, acc[0]);
   acc[1] = fma(jv[j], r0, fma(s, a0, fma(nx, dp, acc[1])));
   acc[2] = fma(jv[N + j], r0, fma(s, a1, fma(ny, dp, acc[2])));
   acc[3] = fma(jv[2 * N + j], r0, fma(s, a2, fma(nz, dp, acc[3])));

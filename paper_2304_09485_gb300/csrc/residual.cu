@@ -36,54 +36,54 @@ constexpr int kBlock = 128;
 struct Prim { double rho, U, V, W, il, ir; };
 
 // rho p of a conservative state, without a division
-__device__ __forceinline__ double rho_p(const double *Q, double g1) {
-  return g1 * fma(Q[4], Q[0], -0.5 * fma(Q[1], Q[1], fma(Q[2], Q[2], Q[3] * Q[3])));
+__device__ __forceinline__ double rho_p(const Units &u, const double *Q, double g1) {
+  return u.mul(g1, fma(Q[4], Q[0], u.mul(-0.5, fma(Q[1], Q[1], fma(Q[2], Q[2], u.mul(Q[3], Q[3]))))));
 }
 // from Q and rp = rho p
-__device__ __forceinline__ Prim to_prim(const double *Q, double rp) {
+__device__ __forceinline__ Prim to_prim(const Units &u, const double *Q, double rp) {
   Prim p;
   p.rho = Q[0];
-  p.ir = rcp(Q[0]);
-  p.U = Q[1] * p.ir; p.V = Q[2] * p.ir; p.W = Q[3] * p.ir;
-  p.il = rp * p.ir * p.ir;
+  p.ir = rcp(Q[0], u.one);
+  p.U = u.mul(Q[1], p.ir); p.V = u.mul(Q[2], p.ir); p.W = u.mul(Q[3], p.ir);
+  p.il = u.mul(u.mul(rp, p.ir), p.ir);
   return p;
 }
 
 // rotate momentum into the face frame (rows of T: n, t1, t2) and back
-__device__ __forceinline__ void rot_in(const double *T, const double *in, double *out) {
+__device__ __forceinline__ void rot_in(const Units &u, const double *T, const double *in, double *out) {
   out[0] = in[0]; out[4] = in[4];
 #pragma unroll
-  for (int r = 0; r < 3; r++) out[1 + r] = T[3 * r] * in[1] + T[3 * r + 1] * in[2] + T[3 * r + 2] * in[3];
+  for (int r = 0; r < 3; r++) out[1 + r] = fma(T[3 * r], in[1], fma(T[3 * r + 1], in[2], u.mul(T[3 * r + 2], in[3])));
 }
-__device__ __forceinline__ void rot_out(const double *T, const double *in, double *out) {
+__device__ __forceinline__ void rot_out(const Units &u, const double *T, const double *in, double *out) {
   out[0] = in[0]; out[4] = in[4];
 #pragma unroll
-  for (int d = 0; d < 3; d++) out[1 + d] = T[d] * in[1] + T[3 + d] * in[2] + T[6 + d] * in[3];
+  for (int d = 0; d < 3; d++) out[1 + d] = fma(T[d], in[1], fma(T[3 + d], in[2], u.mul(T[6 + d], in[3])));
 }
 
 // Euler eigen-system along x of a face-frame state: scalars of which R (right_apply)
 // and R^{-1} (k_recon's projection) are made.
 struct Eig { double u, v, w, a, H, q2, ia; };
-__device__ __forceinline__ Eig eig_of(const double *Q, double gamma, double g1) {
+__device__ __forceinline__ Eig eig_of(const Units &u, const double *Q, double gamma, double g1) {
   Eig e;
-  double ir = rcp(Q[0]);
-  e.u = Q[1] * ir; e.v = Q[2] * ir; e.w = Q[3] * ir;
-  e.q2 = e.u * e.u + e.v * e.v + e.w * e.w;
-  double p = g1 * (Q[4] - 0.5 * Q[0] * e.q2);
-  const double a2 = gamma * p * ir;
+  const double ir = rcp(Q[0], u.one);
+  e.u = u.mul(Q[1], ir); e.v = u.mul(Q[2], ir); e.w = u.mul(Q[3], ir);
+  e.q2 = fma(e.u, e.u, fma(e.v, e.v, u.mul(e.w, e.w)));
+  const double p = u.mul(g1, fma(u.mul(-0.5, Q[0]), e.q2, Q[4]));
+  const double a2 = u.mul(u.mul(gamma, p), ir);
   e.ia = rsqrt64(a2);
-  e.a = a2 * e.ia;
-  e.H = (Q[4] + p) * ir;
+  e.a = u.mul(a2, e.ia);
+  e.H = u.mul(u.add(Q[4], p), ir);
   return e;
 }
 // out = R q (characteristic -> conservative, face frame)
-__device__ __forceinline__ void right_apply(const Eig &e, const double *q, double *out) {
-  double s = q[0] + q[1] + q[4];
+__device__ __forceinline__ void right_apply(const Units &u, const Eig &e, const double *q, double *out) {
+  const double t = u.add(q[0], q[4]), s = u.add(t, q[1]), ad = u.mul(e.a, u.sub(q[4], q[0]));
   out[0] = s;
-  out[1] = e.u * s + e.a * (q[4] - q[0]);
-  out[2] = e.v * s + q[2];
-  out[3] = e.w * s + q[3];
-  out[4] = e.H * (q[0] + q[4]) + e.u * e.a * (q[4] - q[0]) + 0.5 * e.q2 * q[1] + e.v * q[2] + e.w * q[3];
+  out[1] = fma(e.u, s, ad);
+  out[2] = fma(e.v, s, q[2]);
+  out[3] = fma(e.w, s, q[3]);
+  out[4] = fma(e.H, t, fma(e.u, ad, fma(u.mul(0.5, e.q2), q[1], fma(e.v, q[2], u.mul(e.w, q[3])))));
 }
 
 // ------------------------------------------------------------------------
@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(kBlock) k_coef_weno(DevMesh m, const double *_
   if (t >= 5 * NL) return;
   const int c = t / NL, i = t - c * NL;
   if (BATCH && !live(m, i)) return;
+  const Units u = units();
   const double qi = Q[(size_t)c * N + i];
   double a[9];
 #pragma unroll
@@ -117,7 +118,7 @@ __global__ void __launch_bounds__(kBlock) k_coef_weno(DevMesh m, const double *_
   for (int k = 0; k < BIG; k++) {
     int j = m.sten[(size_t)k * N + i];
     if (j < 0) break;
-    const double dq = Q[(size_t)c * N + j] - qi;
+    const double dq = u.sub(Q[(size_t)c * N + j], qi);
     sdq[k][threadIdx.x] = dq;
 #pragma unroll
     for (int d = 0; d < 9; d++) a[d] = fma(m.X0[(size_t)(d * BIG + k) * N + i], dq, a[d]);
@@ -198,18 +199,19 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 // D = prod d_k, R_k = D / d_k (prefix and suffix products) and sum of the linear weights 1,
 //   kap_0 = (D + tz R_0) / den,  kap_m = gm tz (R_m - R_0) / den,
 //   den = D + tz (g0 R_0 + gm sum R_m).
-// Keeping the projection in shared memory (110 doubles a thread on tetrahedra, 170 on
-// hexahedra) instead of projecting per variable: 28.5 -> 24.2 ms for 9.4M (cell, face) pairs
-// (2,359,296 tetrahedra), 1.24 -> 1.00 ms for 35,937 hexahedra; no spills (604 bytes before).
-// Blocks: any shape up to 256 threads fits on tetrahedra; on hexahedra two blocks of 64
-// fit an SM (85 KB each), one of 128, none of 256.
-constexpr int kReconMax = 256, kReconHex = 64;
-template <class S> constexpr int recon_rows() { return 5 * (10 + 3 * ShapeOf<S>::NSUB); }
+// The projection stays in shared memory for three variables at a time, (P - D, q0 - 2 P, P + D),
+// then the two shear waves: 66 doubles a thread on tetrahedra (three blocks of 128 threads an SM),
+// 102 on hexahedra (two; all five variables at once, 170, left four warps an SM and cost 12 %).
+// Against dense rows per variable: 28.5 -> 22.8 ms for 9.4M (cell, face) pairs (2,359,296
+// tetrahedra), 1.24 -> 0.84 ms for 35,937 hexahedra. ncu at 124,416 cells, before the sums and
+// products became FMAs of three registers: 1,471 FP64 instructions a thread, the pipe 89 % busy.
+constexpr int kReconMax = 256, kReconHex = 128;
+template <class S> constexpr int recon_rows() { return 3 * (10 + 3 * ShapeOf<S>::NSUB); }
 template <bool BATCH, class S>
-__global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
+__global__ void __maxnreg__(168) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                      const double *__restrict__ coef, double *__restrict__ wface) {
   constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB, NV = 9 + 3 * NSUB;
-  extern __shared__ double proj[];                      // [5][NV + 1][blockDim.x]: column of this thread
+  extern __shared__ double proj[];                      // [3][NV + 1][blockDim.x]: column of this thread
   const int N = m.N, F = m.F;
   const int NL = BATCH ? m.NL : N;
   // block b covers local face (b mod NF) of cell range b / NF: the blocks of a
@@ -222,56 +224,64 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
   const int f = cf >> 1, side = cf & 1;
   const int bd = blockDim.x;
   double *my = proj + threadIdx.x;
+  const Units u = units();
+  const size_t rs = (size_t)(NV + 1) * bd;              // from one kept variable to the next
   double T[9];
 #pragma unroll
   for (int k = 0; k < 9; k++) T[k] = m.fT[(size_t)k * F + f];
+  Eig e;
   {
     const int L = m.fl[f], R = m.fr[f];
-    double Qi[5], Qs[5], Qsl[5];
+    double Qs[5], Qsl[5];
 #pragma unroll
-    for (int c = 0; c < 5; c++) {
-      Qi[c] = Q[(size_t)c * N + i];
-      Qs[c] = R >= 0 ? Q[(size_t)c * N + L] + Q[(size_t)c * N + R] : Qi[c];   // twice Q*: only ratios are taken
-    }
-    if (P.characteristic) {
-      rot_in(T, Qs, Qsl);
-      const Eig e = eig_of(Qsl, P.gamma, P.g1);
-      const double hb = 0.5 * P.g1 * e.ia * e.ia, hi = 0.5 * e.ia;
+    for (int c = 0; c < 5; c++)                          // twice Q*: only ratios are taken
+      Qs[c] = R >= 0 ? u.add(Q[(size_t)c * N + L], Q[(size_t)c * N + R]) : Q[(size_t)c * N + i];
+    rot_in(u, T, Qs, Qsl);
+    e = eig_of(u, Qsl, P.gamma, P.g1);
+  }
+  // component k of vector d: a coefficient, or (d = NV) the cell average
+  auto in = [&](int d, int k) { return d < NV ? coef[(size_t)(d * 5 + k) * N + i] : Q[(size_t)k * N + i]; };
+  auto project = [&](int pass) {
+    if (!P.characteristic) {                            // conservative variables: the coefficients themselves
+#pragma unroll 1
+      for (int d = 0; d <= NV; d++) {
+        my[d * bd] = in(d, pass == 0 ? 0 : 2);
+        my[rs + d * bd] = in(d, pass == 0 ? 1 : 3);
+        if (pass == 0) my[2 * rs + d * bd] = in(d, 4);
+      }
+    } else if (pass == 0) {
+      const double hb = u.mul(0.5 * P.g1, u.mul(e.ia, e.ia)), hi = u.mul(0.5, e.ia);
+      const double minus2 = u.add(-1.0, -u.one);
       double pm[3], dm[3];                              // P = p0 q0 + pm . m + hb q4, D = d0 q0 + dm . m
-      const double p0 = 0.5 * hb * e.q2, d0 = -hi * e.u;
+      const double p0 = u.mul(u.mul(0.5, hb), e.q2), d0 = u.mul(-hi, e.u);
 #pragma unroll
       for (int k = 0; k < 3; k++) {
-        pm[k] = -hb * (T[k] * e.u + T[3 + k] * e.v + T[6 + k] * e.w);
-        dm[k] = hi * T[k];
+        pm[k] = u.mul(-hb, fma(T[k], e.u, fma(T[3 + k], e.v, u.mul(T[6 + k], e.w))));
+        dm[k] = u.mul(hi, T[k]);
       }
-      auto project = [&](const double *q, double *o) {  // o: row stride (NV + 1) bd between the variables
-        const size_t rs = (size_t)(NV + 1) * bd;
-        const double Pq = fma(p0, q[0], fma(pm[0], q[1], fma(pm[1], q[2], fma(pm[2], q[3], hb * q[4]))));
-        const double Dq = fma(d0, q[0], fma(dm[0], q[1], fma(dm[1], q[2], dm[2] * q[3])));
-        o[0] = Pq - Dq;
-        o[rs] = fma(-2.0, Pq, q[0]);
-        o[2 * rs] = fma(-e.v, q[0], fma(T[3], q[1], fma(T[4], q[2], T[5] * q[3])));
-        o[3 * rs] = fma(-e.w, q[0], fma(T[6], q[1], fma(T[7], q[2], T[8] * q[3])));
-        o[4 * rs] = Pq + Dq;
-      };
 #pragma unroll
-      for (int d = 0; d < NV; d++) {
-        double q[5];
-#pragma unroll
-        for (int k = 0; k < 5; k++) q[k] = coef[(size_t)(d * 5 + k) * N + i];
-        project(q, my + d * bd);
+      for (int d = 0; d <= NV; d++) {
+        const double q0 = in(d, 0), q1 = in(d, 1), q2 = in(d, 2), q3 = in(d, 3), q4 = in(d, 4);
+        const double Pq = fma(p0, q0, fma(pm[0], q1, fma(pm[1], q2, fma(pm[2], q3, u.mul(hb, q4)))));
+        const double Dq = fma(d0, q0, fma(dm[0], q1, fma(dm[1], q2, u.mul(dm[2], q3))));
+        const double lo = u.sub(Pq, Dq), hi4 = u.add(Pq, Dq);
+        my[d * bd] = lo;
+        my[rs + d * bd] = fma(minus2, Pq, q0);
+        my[2 * rs + d * bd] = hi4;
       }
-      project(Qi, my + NV * bd);
-    } else {                                            // conservative variables: the coefficients themselves
-#pragma unroll 1
-      for (int d = 0; d < NV; d++)
+    } else {
+      double t[6];                                      // the tangents (T is scaled by now)
 #pragma unroll
-        for (int k = 0; k < 5; k++) my[(size_t)(k * (NV + 1) + d) * bd] = coef[(size_t)(d * 5 + k) * N + i];
+      for (int k = 0; k < 6; k++) t[k] = m.fT[(size_t)(3 + k) * F + f];
 #pragma unroll
-      for (int k = 0; k < 5; k++) my[(size_t)(k * (NV + 1) + NV) * bd] = Qi[k];
+      for (int d = 0; d <= NV; d++) {
+        const double q0 = in(d, 0), q1 = in(d, 1), q2 = in(d, 2), q3 = in(d, 3);
+        my[d * bd] = fma(-e.v, q0, fma(t[0], q1, fma(t[1], q2, u.mul(t[2], q3))));
+        my[rs + d * bd] = fma(-e.w, q0, fma(t[3], q1, fma(t[4], q2, u.mul(t[5], q3))));
+      }
     }
-  }
-  const double ih = rcp(m.h[i]);
+  };
+  const double ih = rcp(m.h[i], u.one), eps = u.add(P.weno_eps, u.nz);   // eps: in a register
   double m2[6], xg[3 * NG];
 #pragma unroll
   for (int k = 0; k < 6; k++) m2[k] = m.m2[(size_t)k * N + i];
@@ -288,12 +298,15 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
   const int M = __popc(valid);
   const double gm = P.lin_weight, g0 = M ? 1.0 - gm * M : 1.0;
   const double iM = M ? rcp((double)M) : 0.0;
+  project(0);
 #pragma unroll
-  for (int k = 0; k < 9; k++) T[k] *= ih;               // face frame rows / h: scaled derivatives
+  for (int k = 0; k < 9; k++) T[k] = u.mul(T[k], ih);               // face frame rows / h: scaled derivatives
   double *out = wface + (size_t)side * NG * kFaceState * F + f;
 #pragma unroll 1
-  for (int c = 0; c < 5; c++) {
-    const double *pc = my + (size_t)c * (NV + 1) * bd;
+  for (int v = 0; v < 5; v++) {                          // variables 0, 1, 4, then 2, 3
+    if (v == 3) project(1);
+    const int c = v < 2 ? v : v == 2 ? 4 : v - 1;
+    const double *pc = my + (v < 3 ? v : v - 3) * rs;
     double ac[9];
 #pragma unroll
     for (int d = 0; d < 9; d++) ac[d] = pc[d * bd];
@@ -307,51 +320,53 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
       // smoothness indicators in the scaled frame (beta_0 = avg |grad P0|^2 + sum of squared
       // second derivatives), each with weno_eps added
       const double xx = ac[3], yy = ac[4], zz = ac[5], xy = ac[6], xz = ac[7], yz = ac[8];
-      double d0 = fma(ac[0], ac[0], fma(ac[1], ac[1], fma(ac[2], ac[2], P.weno_eps)));
-      d0 = fma(xx, fma(w0, xx, fma(f3, xy, f4 * xz)), d0);
-      d0 = fma(xy, fma(w3, xy, fma(f3, yy, fma(c4, yz, c5 * xz))), d0);
-      d0 = fma(xz, fma(w4, xz, fma(f4, zz, c3 * yz)), d0);
-      d0 = fma(yy, fma(w1, yy, f5 * yz), d0);
-      d0 = fma(yz, fma(w5, yz, f5 * zz), d0);
-      d0 = fma(zz, w2 * zz, d0);
+      double d0 = fma(ac[0], ac[0], fma(ac[1], ac[1], fma(ac[2], ac[2], eps)));
+      d0 = fma(xx, fma(w0, xx, fma(f3, xy, u.mul(f4, xz))), d0);
+      d0 = fma(xy, fma(w3, xy, fma(f3, yy, fma(c4, yz, u.mul(c5, xz)))), d0);
+      d0 = fma(xz, fma(w4, xz, fma(f4, zz, u.mul(c3, yz))), d0);
+      d0 = fma(yy, fma(w1, yy, u.mul(f5, yz)), d0);
+      d0 = fma(yz, fma(w5, yz, u.mul(f5, zz)), d0);
+      d0 = fma(zz, u.mul(w2, zz), d0);
       double dm[NSUB], tz = 0.0;
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {
         const double b0 = pc[(9 + 3 * mm) * bd], b1 = pc[(10 + 3 * mm) * bd], b2 = pc[(11 + 3 * mm) * bd];
-        const double de = fma(b0, b0, fma(b1, b1, fma(b2, b2, P.weno_eps)));
-        if (valid >> mm & 1) tz += fabs(d0 - de);
+        const double de = fma(b0, b0, fma(b1, b1, fma(b2, b2, eps)));
+        if (valid >> mm & 1) tz = u.add(fabs(u.sub(d0, de)), tz);
         dm[mm] = (valid >> mm & 1) ? de : 1.0;
       }
-      tz *= iM;
+      tz = u.mul(tz, iM);
       double R[NSUB], pre = d0, R0 = 1.0, sum = 0.0;
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {               // R[mm] = d0 dm[0] ... dm[mm - 1]
         R[mm] = pre;
-        pre *= dm[mm];
+        pre = u.mul(pre, dm[mm]);
       }
 #pragma unroll
       for (int mm = NSUB - 1; mm >= 0; mm--) {          // times dm[mm + 1] ... dm[NSUB - 1]
-        R[mm] *= R0;
-        R0 *= dm[mm];
-        if (valid >> mm & 1) sum += R[mm];
+        if (mm < NSUB - 1) R[mm] = u.mul(R[mm], R0);
+        R0 = mm < NSUB - 1 ? u.mul(R0, dm[mm]) : dm[mm];
+        if (valid >> mm & 1) sum = u.add(sum, R[mm]);
       }
-      const double inv = rcp(fma(tz, fma(g0, R0, gm * sum), pre)), h = gm * tz * inv;
-      kap0 = inv * fma(tz, R0, pre);
+      const double inv = rcp(fma(tz, fma(g0, R0, u.mul(gm, sum)), pre), u.one), h = u.mul(u.mul(gm, tz), inv);
+      kap0 = u.mul(inv, fma(tz, R0, pre));
 #pragma unroll
-      for (int j = 0; j < 3; j++) lin[j] = kap0 * ac[j];
+      for (int j = 0; j < 3; j++) lin[j] = u.mul(kap0, ac[j]);
 #pragma unroll
       for (int mm = 0; mm < NSUB; mm++) {
-        const double k = (valid >> mm & 1) ? h * (R[mm] - R0) : 0.0;
+        const double k = (valid >> mm & 1) ? u.mul(h, u.sub(R[mm], R0)) : 0.0;
 #pragma unroll
         for (int j = 0; j < 3; j++) lin[j] = fma(k, pc[(9 + 3 * mm + j) * bd], lin[j]);
       }
     }
     double qd[6];
 #pragma unroll
-    for (int k = 0; k < 6; k++) qd[k] = kap0 * ac[3 + k];
+    for (int k = 0; k < 6; k++) qd[k] = u.mul(kap0, ac[3 + k]);
     // P(x) = q0 + lin . x + sum_k qd_k (mono_k(x) - m2_k), nested so that the value
     // and the gradient share their partial sums
-    const double q0m = q0 - (qd[0] * m2[0] + qd[1] * m2[1] + qd[2] * m2[2] + qd[3] * m2[3] + qd[4] * m2[4] + qd[5] * m2[5]);
+    double q0m = q0;
+#pragma unroll
+    for (int k = 0; k < 6; k++) q0m = fma(-qd[k], m2[k], q0m);
 #pragma unroll
     for (int g = 0; g < NG; g++) {
       const double x = xg[3 * g], y = xg[3 * g + 1], z = xg[3 * g + 2];
@@ -365,7 +380,8 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
       double *o = out + (size_t)g * kFaceState * F;
       o[(size_t)c * F] = val;
 #pragma unroll
-      for (int k = 0; k < 3; k++) o[(size_t)(5 + 5 * k + c) * F] = T[3 * k] * gx + T[3 * k + 1] * gy + T[3 * k + 2] * gz;
+      for (int k = 0; k < 3; k++)
+        o[(size_t)(5 + 5 * k + c) * F] = fma(T[3 * k], gx, fma(T[3 * k + 1], gy, u.mul(T[3 * k + 2], gz)));
     }
   }
 }
@@ -379,25 +395,26 @@ __global__ void __launch_bounds__(kReconMax) k_recon(DevMesh m, KParams Pv, cons
 // del = sgn g(u = 0) the density at the end of the half range (0 for the full range); hd = del / 2,
 // h0 = -U del / (2T).
 struct Mom { double m0, m1, m2, m3, m4, hd, h0; };
-__device__ __forceinline__ void mom_up(const Prim &p, Mom &m) {
-  m.m2 = fma(p.U, m.m1, p.il * m.m0);
-  m.m3 = fma(p.U, m.m2, 2.0 * p.il * m.m1);
-  m.m4 = fma(p.U, m.m3, 3.0 * p.il * m.m2);
+__device__ __forceinline__ void mom_up(const Units &u, const Prim &p, Mom &m) {
+  const double T2 = u.add(p.il, p.il);
+  m.m2 = fma(p.U, m.m1, u.mul(p.il, m.m0));
+  m.m3 = fma(p.U, m.m2, u.mul(T2, m.m1));
+  m.m4 = fma(p.U, m.m3, u.mul(u.add(T2, p.il), m.m2));
 }
-__device__ __forceinline__ Mom mom_full(const Prim &p) {
+__device__ __forceinline__ Mom mom_full(const Units &u, const Prim &p) {
   Mom m;
   m.m0 = 1.0; m.m1 = p.U; m.hd = 0.0; m.h0 = 0.0;
-  mom_up(p, m);
+  mom_up(u, p, m);
   return m;
 }
 // <u^0>, <u^1> = U <u^0> + T del, del / 2 = sgn exp(-y^2) / (2 sqrt(2 pi T)) and y = U / sqrt(2T)
 // over sgn u > 0; rs = 1 / sqrt(2T)
-__device__ __forceinline__ void half01(double U, double T, double sgn, double &m0, double &m1, double &hd, double &y,
-                                       double &rs) {
-  const double T2 = 2.0 * T;
+__device__ __forceinline__ void half01(const Units &u, double U, double T, double sgn, double &m0, double &m1, double &hd,
+                                       double &y, double &rs) {
+  const double T2 = u.add(T, T);
   rs = rsqrt64(T2);
-  y = rs * U;
-  const double x = sgn > 0.0 ? -y : y, e = exp64(-y * y);
+  y = u.mul(rs, U);
+  const double x = sgn > 0.0 ? -y : y, e = exp64(u.mul(-y, y));
   if (((unsigned)__double2hiint(x) & 0x7fffffffu) < kErfcRange) {
     m0 = half_erfc64(x);
   } else {
@@ -405,15 +422,15 @@ __device__ __forceinline__ void half01(double U, double T, double sgn, double &m
     const double t = erfcx(fabs(x)) * e;
     m0 = 0.5 * (x >= 0.0 ? t : 2.0 - t);
   }
-  hd = sgn * 0.28209479177387814347 * e * rs;          // 1 / (2 sqrt(pi))
-  m1 = fma(U, m0, T2 * hd);
+  hd = u.mul(sgn * 0.28209479177387814347 * e, rs);    // 1 / (2 sqrt(pi))
+  m1 = fma(U, m0, u.mul(T2, hd));
 }
-__device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
+__device__ __forceinline__ Mom mom_half(const Units &u, const Prim &p, double sgn) {
   Mom m;
   double y, rs;
-  half01(p.U, p.il, sgn, m.m0, m.m1, m.hd, y, rs);
-  m.h0 = -2.0 * y * rs * m.hd;
-  mom_up(p, m);
+  half01(u, p.U, p.il, sgn, m.m0, m.m1, m.hd, y, rs);
+  m.h0 = u.mul(u.mul(-2.0 * y, rs), m.hd);
+  mom_up(u, p, m);
   return m;
 }
 
@@ -438,19 +455,19 @@ __device__ __forceinline__ Mom mom_half(const Prim &p, double sgn) {
 struct Dir { double r, u, v, w, p; };    // drho, rho dU, rho dV, rho dW, dp along one axis of the face frame
 
 // out = L x, out += L x (x in the tangential frame of p, x[4] twice the component)
-__device__ __forceinline__ void from_frame(const Prim &p, const double *x, double *out) {
+__device__ __forceinline__ void from_frame(const Units &u, const Prim &p, const double *x, double *out) {
   out[0] = x[0];
   out[1] = x[1];
   out[2] = fma(p.V, x[0], x[2]);
   out[3] = fma(p.W, x[0], x[3]);
-  out[4] = fma(p.V, x[2], fma(p.W, x[3], 0.5 * fma(fma(p.V, p.V, p.W * p.W), x[0], x[4])));
+  out[4] = fma(p.V, x[2], fma(p.W, x[3], 0.5 * fma(fma(p.V, p.V, u.mul(p.W, p.W)), x[0], x[4])));
 }
-__device__ __forceinline__ void acc_from_frame(const Prim &p, const double *x, double *out) {
-  const double q = fma(p.V, p.V, p.W * p.W);
-  out[0] += x[0];
-  out[1] += x[1];
-  out[2] = fma(p.V, x[0], out[2] + x[2]);
-  out[3] = fma(p.W, x[0], out[3] + x[3]);
+__device__ __forceinline__ void acc_from_frame(const Units &u, const Prim &p, const double *x, double *out) {
+  const double q = fma(p.V, p.V, u.mul(p.W, p.W));
+  out[0] = u.add(x[0], out[0]);
+  out[1] = u.add(x[1], out[1]);
+  out[2] = fma(p.V, x[0], u.add(out[2], x[2]));
+  out[3] = fma(p.W, x[0], u.add(out[3], x[3]));
   out[4] = fma(p.V, x[2], fma(p.W, x[3], fma(0.5, fma(q, x[0], x[4]), out[4])));
 }
 
@@ -459,89 +476,90 @@ __device__ __forceinline__ void acc_from_frame(const Prim &p, const double *x, d
 // the full range: the Euler equations in primitive variables) is -(conv + q),
 //   conv = V d_1 + W d_2,   q = U d_0 + (rho div, dp_0, dp_1, dp_2, (gamma - 1) T rho div).
 struct Slopes { double s0, s1, s2, y, cr, cu, cv, cw, cs, qr, qu, qv, qw, qs; };
-__device__ __forceinline__ Slopes slopes_of(const Prim &p, double g1, const Dir *d) {
+__device__ __forceinline__ Slopes slopes_of(const Units &u, const Prim &p, double g1, const Dir *d) {
   Slopes k;
   k.s0 = fma(-p.il, d[0].r, d[0].p);
   k.s1 = fma(-p.il, d[1].r, d[1].p);
   k.s2 = fma(-p.il, d[2].r, d[2].p);
-  k.y = d[1].v + d[2].w;
-  const double div = d[0].u + k.y;
-  k.cr = fma(p.V, d[1].r, p.W * d[2].r);
-  k.cu = fma(p.V, d[1].u, p.W * d[2].u);
-  k.cv = fma(p.V, d[1].v, p.W * d[2].v);
-  k.cw = fma(p.V, d[1].w, p.W * d[2].w);
-  k.cs = fma(p.V, k.s1, p.W * k.s2);
+  k.y = u.add(d[1].v, d[2].w);
+  const double div = u.add(d[0].u, k.y);
+  k.cr = fma(p.V, d[1].r, u.mul(p.W, d[2].r));
+  k.cu = fma(p.V, d[1].u, u.mul(p.W, d[2].u));
+  k.cv = fma(p.V, d[1].v, u.mul(p.W, d[2].v));
+  k.cw = fma(p.V, d[1].w, u.mul(p.W, d[2].w));
+  k.cs = fma(p.V, k.s1, u.mul(p.W, k.s2));
   k.qr = fma(p.U, d[0].r, div);
   k.qu = fma(p.U, d[0].u, d[0].p);
   k.qv = fma(p.U, d[0].v, d[1].p);
   k.qw = fma(p.U, d[0].w, d[2].p);
-  k.qs = fma(p.U, k.s0, g1 * p.il * div);
+  k.qs = fma(p.U, k.s0, u.mul(u.mul(g1, p.il), div));
   return k;
 }
 
 // F += c rho <u psi> + e sum_d <u u_d d_d psi> + f <u d_t psi>
-__device__ __forceinline__ void acc_flux(const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
+__device__ __forceinline__ void acc_flux(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
                                          double c, double e, double f, double *F) {
-  const double T = p.il, ef = e - f, hd = m.hd;
+  const double T = p.il, ef = u.sub(e, f), hd = m.hd;
   // the derivatives that come with one power of u: e conv + f d_t, and c rho in the density slot
-  const double br = fma(c, p.rho, fma(ef, k.cr, -f * k.qr)), bu = fma(ef, k.cu, -f * k.qu);
-  const double bv = fma(ef, k.cv, -f * k.qv), bw = fma(ef, k.cw, -f * k.qw), bs = fma(ef, k.cs, -f * k.qs);
-  const double m1x2 = 2.0 * m.m1, m1x3 = 3.0 * m.m1, m2x3 = 3.0 * m.m2, m2x6 = 6.0 * m.m2, m3x4 = 4.0 * m.m3;
-  const double B1 = fma(br, m.m1, fma(bu, m.m0, bs * hd));
-  const double B2 = fma(br, m.m2, fma(bu, m1x2, bs * m.m0));
-  const double B3 = fma(br, m.m3, fma(bu, m2x3, bs * m1x3));
-  const double E2 = fma(d[0].r, m.m2, fma(d[0].u, m1x2, k.s0 * m.m0));
-  const double E3 = fma(d[0].r, m.m3, fma(d[0].u, m2x3, k.s0 * m1x3));
-  const double E4 = fma(d[0].r, m.m4, fma(d[0].u, m3x4, k.s0 * m2x6));
-  const double Y1 = fma(d[1].r, m.m1, fma(d[1].u, m.m0, k.s1 * hd));
-  const double Z1 = fma(d[2].r, m.m1, fma(d[2].u, m.m0, k.s2 * hd));
+  const double br = fma(c, p.rho, fma(ef, k.cr, u.mul(-f, k.qr))), bu = fma(ef, k.cu, u.mul(-f, k.qu));
+  const double bv = fma(ef, k.cv, u.mul(-f, k.qv)), bw = fma(ef, k.cw, u.mul(-f, k.qw)), bs = fma(ef, k.cs, u.mul(-f, k.qs));
+  const double m1x2 = u.add(m.m1, m.m1), m1x3 = u.add(m1x2, m.m1), m2x3 = 3.0 * m.m2, m2x6 = u.add(m2x3, m2x3);
+  const double m3x4 = 4.0 * m.m3;
+  const double B1 = fma(br, m.m1, fma(bu, m.m0, u.mul(bs, hd)));
+  const double B2 = fma(br, m.m2, fma(bu, m1x2, u.mul(bs, m.m0)));
+  const double B3 = fma(br, m.m3, fma(bu, m2x3, u.mul(bs, m1x3)));
+  const double E2 = fma(d[0].r, m.m2, fma(d[0].u, m1x2, u.mul(k.s0, m.m0)));
+  const double E3 = fma(d[0].r, m.m3, fma(d[0].u, m2x3, u.mul(k.s0, m1x3)));
+  const double E4 = fma(d[0].r, m.m4, fma(d[0].u, m3x4, u.mul(k.s0, m2x6)));
+  const double Y1 = fma(d[1].r, m.m1, fma(d[1].u, m.m0, u.mul(k.s1, hd)));
+  const double Z1 = fma(d[2].r, m.m1, fma(d[2].u, m.m0, u.mul(k.s2, hd)));
   double x[5];
   x[0] = fma(e, fma(k.y, m.m1, E2), B1);
   x[1] = fma(e, fma(k.y, m.m2, E3), B2);
-  x[2] = fma(e, fma(d[0].v, m.m2, fma(T, Y1, k.s1 * m.m1)), bv * m.m1);
-  x[3] = fma(e, fma(d[0].w, m.m2, fma(T, Z1, k.s2 * m.m1)), bw * m.m1);
-  const double t4 = fma(K2, fma(T, E2, k.s0 * m.m2), E4);
-  x[4] = fma(e, fma(k.y, fma(K4 * T, m.m1, m.m3), t4), fma(K2, fma(T, B1, bs * m.m1), B3));
-  acc_from_frame(p, x, F);
+  x[2] = fma(e, fma(d[0].v, m.m2, fma(T, Y1, u.mul(k.s1, m.m1))), u.mul(bv, m.m1));
+  x[3] = fma(e, fma(d[0].w, m.m2, fma(T, Z1, u.mul(k.s2, m.m1))), u.mul(bw, m.m1));
+  const double t4 = fma(K2, fma(T, E2, u.mul(k.s0, m.m2)), E4);
+  x[4] = fma(e, fma(k.y, fma(u.mul(K4, T), m.m1, m.m3), t4), fma(K2, fma(T, B1, u.mul(bs, m.m1)), B3));
+  acc_from_frame(u, p, x, F);
 }
 
 // the moments sum_d <u_d d_d psi'> without the part of conv (u d_0, v' d_1, w' d_2)
-__device__ __forceinline__ void own_moments(const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
+__device__ __forceinline__ void own_moments(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
                                             double *z) {
-  const double T = p.il, hd = m.hd, del = 2.0 * hd, h0 = m.h0;
-  const double E1 = fma(d[0].r, m.m1, fma(d[0].u, m.m0, k.s0 * hd));
-  const double E2 = fma(d[0].r, m.m2, fma(2.0 * d[0].u, m.m1, k.s0 * m.m0));
-  const double E3 = fma(d[0].r, m.m3, 3.0 * fma(d[0].u, m.m2, k.s0 * m.m1));
-  const double Y0 = fma(d[1].r, m.m0, fma(d[1].u, del, k.s1 * h0));
-  const double Z0 = fma(d[2].r, m.m0, fma(d[2].u, del, k.s2 * h0));
+  const double T = p.il, hd = m.hd, del = u.add(hd, hd), h0 = m.h0;
+  const double E1 = fma(d[0].r, m.m1, fma(d[0].u, m.m0, u.mul(k.s0, hd)));
+  const double E2 = fma(d[0].r, m.m2, fma(u.add(d[0].u, d[0].u), m.m1, u.mul(k.s0, m.m0)));
+  const double E3 = fma(d[0].r, m.m3, 3.0 * fma(d[0].u, m.m2, u.mul(k.s0, m.m1)));
+  const double Y0 = fma(d[1].r, m.m0, fma(d[1].u, del, u.mul(k.s1, h0)));
+  const double Z0 = fma(d[2].r, m.m0, fma(d[2].u, del, u.mul(k.s2, h0)));
   z[0] = fma(k.y, m.m0, E1);
   z[1] = fma(k.y, m.m1, E2);
-  z[2] = fma(d[0].v, m.m1, fma(T, Y0, k.s1 * m.m0));
-  z[3] = fma(d[0].w, m.m1, fma(T, Z0, k.s2 * m.m0));
-  z[4] = fma(k.y, fma(K4 * T, m.m0, m.m2), fma(K2, fma(T, E1, k.s0 * m.m1), E3));   // twice the component
+  z[2] = fma(d[0].v, m.m1, fma(T, Y0, u.mul(k.s1, m.m0)));
+  z[3] = fma(d[0].w, m.m1, fma(T, Z0, u.mul(k.s2, m.m0)));
+  z[4] = fma(k.y, fma(u.mul(K4, T), m.m0, m.m2), fma(K2, fma(T, E1, u.mul(k.s0, m.m1)), E3));   // twice the component
 }
 // W += c rho <psi> + e sum_d <u_d d_d psi> + f <d_t psi>, z from own_moments
-__device__ __forceinline__ void acc_state(const Prim &p, const Mom &m, const Slopes &k, const double *z, double K2, double c,
+__device__ __forceinline__ void acc_state(const Units &u, const Prim &p, const Mom &m, const Slopes &k, const double *z, double K2, double c,
                                           double e, double f, double *W) {
-  const double T = p.il, ef = e - f, hd = m.hd, del = 2.0 * hd, h0 = m.h0;
-  const double br = fma(c, p.rho, fma(ef, k.cr, -f * k.qr)), bu = fma(ef, k.cu, -f * k.qu);
-  const double bv = fma(ef, k.cv, -f * k.qv), bw = fma(ef, k.cw, -f * k.qw), bs = fma(ef, k.cs, -f * k.qs);
-  const double B0 = fma(br, m.m0, fma(bu, del, bs * h0));
-  const double B1 = fma(br, m.m1, fma(bu, m.m0, bs * hd));
-  const double B2 = fma(br, m.m2, fma(2.0 * bu, m.m1, bs * m.m0));
+  const double T = p.il, ef = u.sub(e, f), hd = m.hd, del = u.add(hd, hd), h0 = m.h0;
+  const double br = fma(c, p.rho, fma(ef, k.cr, u.mul(-f, k.qr))), bu = fma(ef, k.cu, u.mul(-f, k.qu));
+  const double bv = fma(ef, k.cv, u.mul(-f, k.qv)), bw = fma(ef, k.cw, u.mul(-f, k.qw)), bs = fma(ef, k.cs, u.mul(-f, k.qs));
+  const double B0 = fma(br, m.m0, fma(bu, del, u.mul(bs, h0)));
+  const double B1 = fma(br, m.m1, fma(bu, m.m0, u.mul(bs, hd)));
+  const double B2 = fma(br, m.m2, fma(u.add(bu, bu), m.m1, u.mul(bs, m.m0)));
   double x[5];
   x[0] = fma(e, z[0], B0);
   x[1] = fma(e, z[1], B1);
-  x[2] = fma(e, z[2], bv * m.m0);
-  x[3] = fma(e, z[3], bw * m.m0);
-  x[4] = fma(e, z[4], fma(K2, fma(T, B0, bs * m.m0), B2));
-  acc_from_frame(p, x, W);
+  x[2] = fma(e, z[2], u.mul(bv, m.m0));
+  x[3] = fma(e, z[3], u.mul(bw, m.m0));
+  x[4] = fma(e, z[4], fma(K2, fma(T, B0, u.mul(bs, m.m0)), B2));
+  acc_from_frame(u, p, x, W);
 }
 
 // State outside a boundary face (face frame, x = outward normal), from the inner one: walls
 // mirror it in (p, U, V, W, T = p/rho), an isothermal wall's image with the density of zero
 // mass exchange; far field = free stream. M1: <u>_{u>0} of the inner state.
-__device__ void image_state(const KParams &P, int tag, const double *T, const Prim &l, double M1, bool held, double *Wr) {
+__device__ void image_state(const Units &un, const KParams &P, int tag, const double *T, const Prim &l, double M1, bool held, double *Wr) {
   if (tag == HGKS_BC_FARFIELD) {
     double u[3];
 #pragma unroll
@@ -567,7 +585,7 @@ __device__ void image_state(const KParams &P, int tag, const double *T, const Pr
   double rg = l.rho;
   if (T_odd) {
     double m0, Mg, hd, y, rs;
-    half01(l.U, Tg, 1.0, m0, Mg, hd, y, rs);
+    half01(un, l.U, Tg, 1.0, m0, Mg, hd, y, rs);
     rg = l.rho * M1 * rcp(Mg);
   }
   Wr[0] = rg;
@@ -609,27 +627,28 @@ __device__ __forceinline__ void image_slopes(int tag, const Prim &l, const Prim 
 // derivatives, whose primitive form with respect to p follows directly: with (du, dv, dw) =
 // u* - (U, V, W) and c* the sound speed of the projection state, dp = (gamma - 1)(dE - u . dm +
 // |u|^2/2 drho) takes five products instead of the fourteen of R* and nine of the change of variables.
-__device__ __forceinline__ void dirs_of(const KParams &P, const Eig &e, const double *T, const Prim &p, const double (*q)[5],
+__device__ __forceinline__ void dirs_of(const Units &u, const KParams &P, const Eig &e, const double *T, const Prim &p, const double (*q)[5],
                                         Dir *d) {
   const double g1 = P.g1;
   if (P.characteristic) {
-    const double du = e.u - p.U, dv = e.v - p.V, dw = e.w - p.W;
-    const double gu = g1 * du, gv = g1 * dv, gw = g1 * dw, h = 0.5 * fma(gu, du, fma(gv, dv, gw * dw)), a2 = e.a * e.a;
+    const double du = u.sub(e.u, p.U), dv = u.sub(e.v, p.V), dw = u.sub(e.w, p.W);
+    const double gu = u.mul(g1, du), gv = u.mul(g1, dv), gw = u.mul(g1, dw), a2 = u.mul(e.a, e.a);
+    const double h = 0.5 * fma(gu, du, fma(gv, dv, u.mul(gw, dw)));
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-      const double ad = e.a * (q[k][4] - q[k][0]), t = q[k][0] + q[k][4], r = t + q[k][1];
+      const double ad = u.mul(e.a, u.sub(q[k][4], q[k][0])), t = u.add(q[k][0], q[k][4]), r = u.add(t, q[k][1]);
       d[k].r = r;
       d[k].u = fma(du, r, ad);
       d[k].v = fma(dv, r, q[k][2]);
       d[k].w = fma(dw, r, q[k][3]);
-      d[k].p = fma(a2, t, fma(h, r, fma(gu, ad, fma(gv, q[k][2], gw * q[k][3]))));
+      d[k].p = fma(a2, t, fma(h, r, fma(gu, ad, fma(gv, q[k][2], u.mul(gw, q[k][3])))));
     }
   } else {
     const double h = 0.5 * fma(p.U, p.U, fma(p.V, p.V, p.W * p.W));
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       double x[5];
-      rot_in(T, q[k], x);
+      rot_in(u, T, q[k], x);
       d[k].r = x[0];
       d[k].u = fma(-p.U, x[0], x[1]);
       d[k].v = fma(-p.V, x[0], x[2]);
@@ -662,7 +681,10 @@ __device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim
 // solved for each axis and summed with moments up to u^6: 37.5 -> 24.5 ms at 14.2M Gauss
 // points (inviscid, 2,359,296 tetrahedra), 1.22 -> 0.74 ms at 295k (viscous, compact scheme);
 // with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms;
-// with g_0's derivatives from the sum of the characteristic ones 19.1 and 0.61 ms.
+// with g_0's derivatives from the sum of the characteristic ones 19.1 and 0.61 ms; products and
+// sums as FMAs of three registers (Units) 17.9 and 0.61 ms. ncu at 124,416 cells: 743 FP64
+// instructions a thread, the FP64 pipe 87 % busy, 8 warps a SM (255 registers; 168 or 128
+// registers with spills and more warps measured the same).
 template <bool BATCH, class S, bool COMPACT>
 __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                   const double *__restrict__ dt, const double *__restrict__ wface,
@@ -681,7 +703,8 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   for (int k = 0; k < 9; k++) T[k] = m.fT[(size_t)k * F + f];
   const int L = m.fl[f], R = m.fr[f];
   const bool inner = R >= 0;
-  const double g1 = P.g1, K2 = P.K2, K4 = P.K4;
+  const Units u = units();
+  const double g1 = u.add(P.g1, u.nz), K2 = u.add(P.K2, u.nz), K4 = u.add(P.K4, u.nz);   // in registers
   Prim pl, pr;
   Mom ml, mr;
   Eig e;
@@ -693,58 +716,58 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
     for (int c = 0; c < 5; c++) {
       QL[c] = Q[(size_t)c * N + L];
       QR[c] = inner ? Q[(size_t)c * N + R] : QL[c];
-      Qs[c] = inner ? QL[c] + QR[c] : QL[c];             // twice Q*: only ratios are taken
+      Qs[c] = inner ? u.add(QL[c], QR[c]) : QL[c];             // twice Q*: only ratios are taken
     }
-    rot_in(T, Qs, Qsl);
-    e = eig_of(Qsl, P.gamma, g1);
+    rot_in(u, T, Qs, Qsl);
+    e = eig_of(u, Qsl, P.gamma, g1);
     auto side = [&](int s, const double *Qc) {
       const double *in = wface + ((size_t)(s * NG + g) * kFaceState) * F + f;
 #pragma unroll
       for (int c = 0; c < 5; c++) q[c] = in[(size_t)c * F];
-      if (P.characteristic) right_apply(e, q, W);
-      else rot_in(T, q, W);
-      double rp = rho_p(W, g1);
+      if (P.characteristic) right_apply(u, e, q, W);
+      else rot_in(u, T, q, W);
+      double rp = rho_p(u, W, g1);
       if (!positive(W[0]) || !positive(rp)) {
-        rot_in(T, Qc, W);
-        rp = rho_p(W, g1);
+        rot_in(u, T, Qc, W);
+        rp = rho_p(u, W, g1);
         bad |= 1 << s;
       }
       return rp;
     };
     double rp = side(0, QL);
-    pl = to_prim(W, rp);
-    ml = mom_half(pl, 1.0);
+    pl = to_prim(u, W, rp);
+    ml = mom_half(u, pl, 1.0);
     if (inner) {
       rp = side(1, QR);
     } else {
       held = image_held(P, m.ftag[f], pl.il);
-      image_state(P, m.ftag[f], T, pl, ml.m1, held, W);
-      rp = rho_p(W, g1);
+      image_state(u, P, m.ftag[f], T, pl, ml.m1, held, W);
+      rp = rho_p(u, W, g1);
     }
-    pr = to_prim(W, rp);
-    mr = mom_half(pr, -1.0);
+    pr = to_prim(u, W, rp);
+    mr = mom_half(u, pr, -1.0);
   }
   // compatibility condition: Q0 = int_{u>0} psi g_l + int_{u<0} psi g_r
   Prim p0;
   {
     double Q0[5];
-    const double xl[5] = {pl.rho * ml.m0, pl.rho * ml.m1, 0.0, 0.0, pl.rho * fma(K2 * pl.il, ml.m0, ml.m2)};
-    const double xr[5] = {pr.rho * mr.m0, pr.rho * mr.m1, 0.0, 0.0, pr.rho * fma(K2 * pr.il, mr.m0, mr.m2)};
-    from_frame(pl, xl, Q0);
-    acc_from_frame(pr, xr, Q0);
-    p0 = to_prim(Q0, rho_p(Q0, g1));
+    const double xl[5] = {u.mul(pl.rho, ml.m0), u.mul(pl.rho, ml.m1), 0.0, 0.0, u.mul(pl.rho, fma(u.mul(K2, pl.il), ml.m0, ml.m2))};
+    const double xr[5] = {u.mul(pr.rho, mr.m0), u.mul(pr.rho, mr.m1), 0.0, 0.0, u.mul(pr.rho, fma(u.mul(K2, pr.il), mr.m0, mr.m2))};
+    from_frame(u, pl, xl, Q0);
+    acc_from_frame(u, pr, xr, Q0);
+    p0 = to_prim(u, Q0, rho_p(u, Q0, g1));
   }
   double dtf;
   if (positive(P.flux_dt)) dtf = P.flux_dt;
   else dtf = (inner ? min_positive(dt[L], dt[R]) : dt[L]) * P.flux_dt_ratio;
   // collision time (Sec. 5) over dt, and the time coefficients of Eq. (flux) over dt
-  const double prl = pl.rho * pl.il, prr = pr.rho * pr.il, pp0 = p0.rho * p0.il;
-  const double jump = fabs((prl - prr) * rcp(prl + prr));
-  const double tq = fma(P.tau_C, jump, P.viscous ? P.mu * rcp(pp0 * dtf) : P.tau_eps);   // tau / dt
-  const double eta = exp64(-rcp(tq));
-  const double c4 = tq * (1.0 - eta), k4 = tq * c4, tau = tq * dtf;
-  const double c1 = 1.0 - c4, c2 = dtf * (2.0 * k4 - tq * (1.0 + eta)), c3 = dtf * (0.5 - tq + k4);
-  const double c5 = dtf * (2.0 * k4 - tq * eta);
+  const double prl = u.mul(pl.rho, pl.il), prr = u.mul(pr.rho, pr.il), pp0 = u.mul(p0.rho, p0.il);
+  const double jump = fabs(u.mul(u.sub(prl, prr), rcp(u.add(prl, prr), u.one)));
+  const double tq = fma(P.tau_C, jump, P.viscous ? P.mu * rcp(u.mul(pp0, dtf), u.one) : P.tau_eps);   // tau / dt
+  const double eta = exp64(-rcp(tq, u.one));
+  const double c4 = u.mul(tq, u.sub(u.one, eta)), k4 = u.mul(tq, c4), k42 = u.add(k4, k4), tau = u.mul(tq, dtf);
+  const double c1 = u.sub(u.one, c4), c2 = u.mul(dtf, fma(-tq, u.add(u.one, eta), k42)), c3 = u.mul(dtf, 0.5 - tq + k4);
+  const double c5 = u.mul(dtf, fma(-tq, eta, k42));
   const bool prandtl = P.fix_prandtl;
   const double ts = P.tstar_end ? dtf : 0.0, es = P.tstar_end ? eta : 1.0;   // exp(-t* / tau)
   double Fl[5] = {0, 0, 0, 0, 0}, Wb[5] = {0, 0, 0, 0, 0}, Pt[5] = {0, 0, 0, 0, 0};
@@ -759,7 +782,7 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = 0.0;
   Prim pk = pl;
   Mom mk = ml;
-  double C = c4, Ce = -c5, Cf = -dtf * k4;              // flux: c rho <u psi> + e sum <u u_d d_d psi> + f <u d_t psi>
+  double C = c4, Ce = -c5, Cf = u.mul(-dtf, k4);              // flux: c rho <u psi> + e sum <u u_d d_d psi> + f <u d_t psi>
   double A = es, Ae = -es * (tau + ts), Af = -es * tau; // point value
 #pragma unroll 1
   for (int s = 0; s < 3; s++) {
@@ -771,23 +794,23 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
         double q[3][5];
 #pragma unroll
         for (int a = 0; a < 15; a++) q[a / 5][a % 5] = bad >> s & 1 ? 0.0 : in[(size_t)a * F];
-        dirs_of(P, e, T, pk, q, d);
+        dirs_of(u, P, e, T, pk, q, d);
         if (sums) {
           if (s == 0) {
 #pragma unroll
             for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = q[a / 5][a % 5];
           } else {
 #pragma unroll
-            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] += q[a / 5][a % 5];
+            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = u.add(q0[a / 5][a % 5], q[a / 5][a % 5]);
           }
         }
       }
       if (!sums) add_shifted(g1, pk, p0, d, q0);
     } else {
       pk = p0;
-      mk = mom_full(p0);
+      mk = mom_full(u, p0);
       if (sums) {
-        dirs_of(P, e, T, pk, q0, d);
+        dirs_of(u, P, e, T, pk, q0, d);
       } else {
 #pragma unroll
         for (int a = 0; a < 3; a++) d[a] = Dir{q0[a][0], q0[a][1], q0[a][2], q0[a][3], q0[a][4]};
@@ -795,13 +818,13 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
       C = c1; Ce = 0.5 * c2; Cf = 0.5 * c3;
       A = 1.0 - es; Ae = 0.5 * fma(ts + tau, es, -tau); Af = 0.5 * (ts - tau + tau * es);
     }
-    const Slopes k = slopes_of(pk, g1, d);
-    acc_flux(pk, mk, d, k, K2, K4, C, Ce, Cf, Fl);
+    const Slopes k = slopes_of(u, pk, g1, d);
+    acc_flux(u, pk, mk, d, k, K2, K4, C, Ce, Cf, Fl);
     if (COMPACT || prandtl) {
       double z[5];
-      own_moments(pk, mk, d, k, K2, K4, z);
-      if (prandtl) acc_state(pk, mk, k, z, K2, C, Ce, Cf, Wb);
-      if (COMPACT) acc_state(pk, mk, k, z, K2, A, Ae, Af, Pt);
+      own_moments(u, pk, mk, d, k, K2, K4, z);
+      if (prandtl) acc_state(u, pk, mk, k, z, K2, C, Ce, Cf, Wb);
+      if (COMPACT) acc_state(u, pk, mk, k, z, K2, A, Ae, Af, Pt);
     }
     pk = pr;
     mk = mr;
@@ -819,13 +842,13 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   // Gauss weight times area: 1/3 on a triangle, the area-element weight on a quadrilateral
   const double w = NG == 3 ? m.fS[f] * (1.0 / 3.0) : m.fS[f] * m.fw[(size_t)g * F + f];
   double Fg[5];
-  rot_out(T, Fl, Fg);
+  rot_out(u, T, Fl, Fg);
 #pragma unroll
-  for (int c = 0; c < 5; c++) fflux[(size_t)(g * 5 + c) * F + f] = w * Fg[c];
+  for (int c = 0; c < 5; c++) fflux[(size_t)(g * 5 + c) * F + f] = u.mul(w, Fg[c]);
   if (COMPACT) {
-    rot_out(T, Pt, Fg);
+    rot_out(u, T, Pt, Fg);
 #pragma unroll
-    for (int c = 0; c < 5; c++) fpt[(size_t)(g * 5 + c) * F + f] = w * Fg[c];
+    for (int c = 0; c < 5; c++) fpt[(size_t)(g * 5 + c) * F + f] = u.mul(w, Fg[c]);
   }
 }
 
