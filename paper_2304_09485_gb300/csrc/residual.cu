@@ -496,63 +496,68 @@ __device__ __forceinline__ Slopes slopes_of(const Units &u, const Prim &p, doubl
   return k;
 }
 
-// F += c rho <u psi> + e sum_d <u u_d d_d psi> + f <u d_t psi>
-__device__ __forceinline__ void acc_flux(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
-                                         double c, double e, double f, double *F) {
-  const double T = p.il, ef = u.sub(e, f), hd = m.hd;
-  // the derivatives that come with one power of u: e conv + f d_t, and c rho in the density slot
-  const double br = fma(c, p.rho, fma(ef, k.cr, u.mul(-f, k.qr))), bu = fma(ef, k.cu, u.mul(-f, k.qu));
-  const double bv = fma(ef, k.cv, u.mul(-f, k.qv)), bw = fma(ef, k.cw, u.mul(-f, k.qw)), bs = fma(ef, k.cs, u.mul(-f, k.qs));
+// The derivatives that come with one power less of the velocity, e conv + f d_t, with c rho in
+// the density slot.
+struct Comb { double r, u, v, w, s; };
+__device__ __forceinline__ Comb combine(const Units &u, const Prim &p, const Slopes &k, double c, double e, double f) {
+  const double ef = u.sub(e, f);
+  return {fma(c, p.rho, fma(ef, k.cr, u.mul(-f, k.qr))), fma(ef, k.cu, u.mul(-f, k.qu)), fma(ef, k.cv, u.mul(-f, k.qv)),
+          fma(ef, k.cw, u.mul(-f, k.qw)), fma(ef, k.cs, u.mul(-f, k.qs))};
+}
+// sums that the flux and the state moments have in common
+struct Sums { double B1, B2, E2, E3, m1x2; };
+
+// F += c rho <u psi> + e sum_d <u u_d d_d psi> + f <u d_t psi>, b = combine(c, e, f)
+__device__ __forceinline__ Sums acc_flux(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2,
+                                         double K4, const Comb &b, double e, double *F) {
+  const double T = p.il, hd = m.hd;
   const double m1x2 = u.add(m.m1, m.m1), m1x3 = u.add(m1x2, m.m1), m2x3 = 3.0 * m.m2, m2x6 = u.add(m2x3, m2x3);
   const double m3x4 = 4.0 * m.m3;
-  const double B1 = fma(br, m.m1, fma(bu, m.m0, u.mul(bs, hd)));
-  const double B2 = fma(br, m.m2, fma(bu, m1x2, u.mul(bs, m.m0)));
-  const double B3 = fma(br, m.m3, fma(bu, m2x3, u.mul(bs, m1x3)));
-  const double E2 = fma(d[0].r, m.m2, fma(d[0].u, m1x2, u.mul(k.s0, m.m0)));
-  const double E3 = fma(d[0].r, m.m3, fma(d[0].u, m2x3, u.mul(k.s0, m1x3)));
+  Sums t;
+  t.m1x2 = m1x2;
+  t.B1 = fma(b.r, m.m1, fma(b.u, m.m0, u.mul(b.s, hd)));
+  t.B2 = fma(b.r, m.m2, fma(b.u, m1x2, u.mul(b.s, m.m0)));
+  const double B3 = fma(b.r, m.m3, fma(b.u, m2x3, u.mul(b.s, m1x3)));
+  t.E2 = fma(d[0].r, m.m2, fma(d[0].u, m1x2, u.mul(k.s0, m.m0)));
+  t.E3 = fma(d[0].r, m.m3, fma(d[0].u, m2x3, u.mul(k.s0, m1x3)));
   const double E4 = fma(d[0].r, m.m4, fma(d[0].u, m3x4, u.mul(k.s0, m2x6)));
   const double Y1 = fma(d[1].r, m.m1, fma(d[1].u, m.m0, u.mul(k.s1, hd)));
   const double Z1 = fma(d[2].r, m.m1, fma(d[2].u, m.m0, u.mul(k.s2, hd)));
   double x[5];
-  x[0] = fma(e, fma(k.y, m.m1, E2), B1);
-  x[1] = fma(e, fma(k.y, m.m2, E3), B2);
-  x[2] = fma(e, fma(d[0].v, m.m2, fma(T, Y1, u.mul(k.s1, m.m1))), u.mul(bv, m.m1));
-  x[3] = fma(e, fma(d[0].w, m.m2, fma(T, Z1, u.mul(k.s2, m.m1))), u.mul(bw, m.m1));
-  const double t4 = fma(K2, fma(T, E2, u.mul(k.s0, m.m2)), E4);
-  x[4] = fma(e, fma(k.y, fma(u.mul(K4, T), m.m1, m.m3), t4), fma(K2, fma(T, B1, u.mul(bs, m.m1)), B3));
+  x[0] = fma(e, fma(k.y, m.m1, t.E2), t.B1);
+  x[1] = fma(e, fma(k.y, m.m2, t.E3), t.B2);
+  x[2] = fma(e, fma(d[0].v, m.m2, fma(T, Y1, u.mul(k.s1, m.m1))), u.mul(b.v, m.m1));
+  x[3] = fma(e, fma(d[0].w, m.m2, fma(T, Z1, u.mul(k.s2, m.m1))), u.mul(b.w, m.m1));
+  const double t4 = fma(K2, fma(T, t.E2, u.mul(k.s0, m.m2)), E4);
+  x[4] = fma(e, fma(k.y, fma(u.mul(K4, T), m.m1, m.m3), t4), fma(K2, fma(T, t.B1, u.mul(b.s, m.m1)), B3));
   acc_from_frame(u, p, x, F);
+  return t;
 }
 
 // the moments sum_d <u_d d_d psi'> without the part of conv (u d_0, v' d_1, w' d_2)
-__device__ __forceinline__ void own_moments(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k, double K2, double K4,
-                                            double *z) {
+__device__ __forceinline__ void own_moments(const Units &u, const Prim &p, const Mom &m, const Dir *d, const Slopes &k,
+                                            const Sums &t, double K2, double K4, double *z) {
   const double T = p.il, hd = m.hd, del = u.add(hd, hd), h0 = m.h0;
   const double E1 = fma(d[0].r, m.m1, fma(d[0].u, m.m0, u.mul(k.s0, hd)));
-  const double E2 = fma(d[0].r, m.m2, fma(u.add(d[0].u, d[0].u), m.m1, u.mul(k.s0, m.m0)));
-  const double E3 = fma(d[0].r, m.m3, 3.0 * fma(d[0].u, m.m2, u.mul(k.s0, m.m1)));
   const double Y0 = fma(d[1].r, m.m0, fma(d[1].u, del, u.mul(k.s1, h0)));
   const double Z0 = fma(d[2].r, m.m0, fma(d[2].u, del, u.mul(k.s2, h0)));
   z[0] = fma(k.y, m.m0, E1);
-  z[1] = fma(k.y, m.m1, E2);
+  z[1] = fma(k.y, m.m1, t.E2);
   z[2] = fma(d[0].v, m.m1, fma(T, Y0, u.mul(k.s1, m.m0)));
   z[3] = fma(d[0].w, m.m1, fma(T, Z0, u.mul(k.s2, m.m0)));
-  z[4] = fma(k.y, fma(u.mul(K4, T), m.m0, m.m2), fma(K2, fma(T, E1, u.mul(k.s0, m.m1)), E3));   // twice the component
+  z[4] = fma(k.y, fma(u.mul(K4, T), m.m0, m.m2), fma(K2, fma(T, E1, u.mul(k.s0, m.m1)), t.E3));   // twice the component
 }
-// W += c rho <psi> + e sum_d <u_d d_d psi> + f <d_t psi>, z from own_moments
-__device__ __forceinline__ void acc_state(const Units &u, const Prim &p, const Mom &m, const Slopes &k, const double *z, double K2, double c,
-                                          double e, double f, double *W) {
-  const double T = p.il, ef = u.sub(e, f), hd = m.hd, del = u.add(hd, hd), h0 = m.h0;
-  const double br = fma(c, p.rho, fma(ef, k.cr, u.mul(-f, k.qr))), bu = fma(ef, k.cu, u.mul(-f, k.qu));
-  const double bv = fma(ef, k.cv, u.mul(-f, k.qv)), bw = fma(ef, k.cw, u.mul(-f, k.qw)), bs = fma(ef, k.cs, u.mul(-f, k.qs));
-  const double B0 = fma(br, m.m0, fma(bu, del, u.mul(bs, h0)));
-  const double B1 = fma(br, m.m1, fma(bu, m.m0, u.mul(bs, hd)));
-  const double B2 = fma(br, m.m2, fma(u.add(bu, bu), m.m1, u.mul(bs, m.m0)));
+// W += c rho <psi> + e sum_d <u_d d_d psi> + f <d_t psi>: z from own_moments, b = combine(c, e, f),
+// B1 and B2 the sums of b in <u d psi>
+__device__ __forceinline__ void acc_state(const Units &u, const Prim &p, const Mom &m, const double *z, double K2, const Comb &b,
+                                          double B1, double B2, double e, double *W) {
+  const double B0 = fma(b.r, m.m0, fma(b.u, u.add(m.hd, m.hd), u.mul(b.s, m.h0)));
   double x[5];
   x[0] = fma(e, z[0], B0);
   x[1] = fma(e, z[1], B1);
-  x[2] = fma(e, z[2], u.mul(bv, m.m0));
-  x[3] = fma(e, z[3], u.mul(bw, m.m0));
-  x[4] = fma(e, z[4], fma(K2, fma(T, B0, u.mul(bs, m.m0)), B2));
+  x[2] = fma(e, z[2], u.mul(b.v, m.m0));
+  x[3] = fma(e, z[3], u.mul(b.w, m.m0));
+  x[4] = fma(e, z[4], fma(K2, fma(p.il, B0, u.mul(b.s, m.m0)), B2));
   acc_from_frame(u, p, x, W);
 }
 
@@ -682,9 +687,10 @@ __device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim
 // points (inviscid, 2,359,296 tetrahedra), 1.22 -> 0.74 ms at 295k (viscous, compact scheme);
 // with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms;
 // with g_0's derivatives from the sum of the characteristic ones 19.1 and 0.61 ms; products and
-// sums as FMAs of three registers (Units) 17.9 and 0.61 ms. ncu at 124,416 cells: 743 FP64
-// instructions a thread, the FP64 pipe 87 % busy, 8 warps a SM (255 registers; 168 or 128
-// registers with spills and more warps measured the same).
+// sums as FMAs of three registers (Units) 17.9 and 0.61 ms; sums shared by flux, heat flux and
+// point values 17.9 and 0.57 ms. ncu at 124,416 cells: 743 FP64 instructions a thread (inviscid),
+// the FP64 pipe 87 % busy with 8 warps an SM; 168 or 128 registers, with spills and more warps,
+// take 9 and 6 % longer.
 template <bool BATCH, class S, bool COMPACT>
 __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                   const double *__restrict__ dt, const double *__restrict__ wface,
@@ -819,22 +825,28 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
       A = 1.0 - es; Ae = 0.5 * fma(ts + tau, es, -tau); Af = 0.5 * (ts - tau + tau * es);
     }
     const Slopes k = slopes_of(u, pk, g1, d);
-    acc_flux(u, pk, mk, d, k, K2, K4, C, Ce, Cf, Fl);
+    const Comb b = combine(u, pk, k, C, Ce, Cf);
+    const Sums t = acc_flux(u, pk, mk, d, k, K2, K4, b, Ce, Fl);
     if (COMPACT || prandtl) {
       double z[5];
-      own_moments(u, pk, mk, d, k, K2, K4, z);
-      if (prandtl) acc_state(u, pk, mk, k, z, K2, C, Ce, Cf, Wb);
-      if (COMPACT) acc_state(u, pk, mk, k, z, K2, A, Ae, Af, Pt);
+      own_moments(u, pk, mk, d, k, t, K2, K4, z);
+      if (prandtl) acc_state(u, pk, mk, z, K2, b, t.B1, t.B2, Ce, Wb);
+      if (COMPACT) {
+        const Comb a = combine(u, pk, k, A, Ae, Af);
+        const double A1 = fma(a.r, mk.m1, fma(a.u, mk.m0, u.mul(a.s, mk.hd)));
+        const double A2 = fma(a.r, mk.m2, fma(a.u, t.m1x2, u.mul(a.s, mk.m0)));
+        acc_state(u, pk, mk, z, K2, a, A1, A2, Ae, Pt);
+      }
     }
     pk = pr;
     mk = mr;
   }
   if (prandtl) {
     // heat flux of the averaged distribution about the velocity of Q0 times 1/Pr - 1
-    const double U = p0.U, V = p0.V, W = p0.W, q2 = U * U + V * V + W * W;
-    const double q = Fl[4] - (U * Fl[1] + V * Fl[2] + W * Fl[3]) + 0.5 * q2 * Fl[0] - U * Wb[4] +
-                     U * (U * Wb[1] + V * Wb[2] + W * Wb[3]) - 0.5 * U * q2 * Wb[0];
-    Fl[4] += P.prandtl * q;
+    const double U = p0.U, V = p0.V, W = p0.W, h2 = 0.5 * fma(U, U, fma(V, V, u.mul(W, W)));
+    const double qf = fma(-U, Fl[1], fma(-V, Fl[2], fma(-W, Fl[3], fma(h2, Fl[0], Fl[4]))));
+    const double qw = fma(-U, Wb[1], fma(-V, Wb[2], fma(-W, Wb[3], fma(h2, Wb[0], Wb[4]))));
+    Fl[4] = fma(P.prandtl, fma(-U, qw, qf), Fl[4]);
   }
   // walls are impermeable: their faces carry momentum and energy, no mass
   if (!inner && m.ftag[f] >= HGKS_BC_WALL_ISO && m.ftag[f] <= HGKS_BC_NOSLIP_ADIA) Fl[0] = 0.0;
