@@ -179,6 +179,7 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     for (double *&z : s.z)
       if (!arena && (st = dalloc(m, &z, 6 * N))) return st;
     HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
+    HGKS_CUDA(cudaMemset(s.hs + kHsStuck, 0, sizeof(double)));
   }
   if (implicit && mixed && !s.jv32) {
     if ((st = dalloc(m, &s.jv32, (6 + 4 * NF) * N))) return st;
@@ -500,7 +501,7 @@ static hgks_status enqueue_step(Mesh &m, const hgks_params *p, double *Q, double
                                 bool have_residual, cudaStream_t st_) {
   const DevMesh &d = m.d;
   Scratch &s = m.s;
-  double *res_dev = s.hs + 65 * 64 + 200;
+  double *res_dev = s.hs + kHsRes;
   if (!have_residual) {
     launch_residual(d, s, *p, Q, G, s.R, p->scheme == HGKS_HWENO ? s.Gnew : nullptr, st_);
     launch_density_l1(d, s, s.R, res_dev, st_);
@@ -553,29 +554,34 @@ static hgks_status run_step(Mesh &m, const hgks_params *p, double *Q, double *G,
   return HGKS_OK;
 }
 
+static hgks_status barrier_failed(Scratch &s, cudaStream_t st) {
+  HGKS_CUDA(cudaMemsetAsync(s.hs + kHsStuck, 0, sizeof(double), st));
+  return fail(HGKS_ERR_CUDA, "a grid barrier of the GMRES solve timed out");
+}
+
 static hgks_status gmres_step_impl(Mesh &m, const hgks_params *p, double *Q, double *G, double *dQ_out,
-                                   hgks_step_info *info, cudaStream_t st_, bool have_residual = false) {
+                                   hgks_step_info *info, cudaStream_t st_) {
   Scratch &s = m.s;
-  double *res_dev = s.hs + 65 * 64 + 200;
-  hgks_status st = run_step(m, p, Q, G, dQ_out, have_residual, st_);
+  double *res_dev = s.hs + kHsRes;
+  hgks_status st = run_step(m, p, Q, G, dQ_out, false, st_);
   if (st) return st;
   if (info) info->krylov_iters = p->restarts * p->krylov_dim;
-  double host[3];
+  struct { double res; int64_t stuck; double lin[2]; } host;
   const int mk = p->krylov_dim;
-  HGKS_CUDA(cudaMemcpyAsync(host, res_dev, sizeof(double), cudaMemcpyDeviceToHost, st_));
-  HGKS_CUDA(cudaMemcpyAsync(host + 1, s.hs + (mk + 1) * mk + 1 + mk, 2 * sizeof(double), cudaMemcpyDeviceToHost, st_));
-  int flags[2] = {0, 0};               // non-physical states, a grid barrier that gave up
-  HGKS_CUDA(cudaMemcpyAsync(flags, s.flags, sizeof(flags), cudaMemcpyDeviceToHost, st_));
-  HGKS_CUDA(cudaMemsetAsync(s.flags, 0, sizeof(flags), st_));
+  int nonphys = 0;
+  HGKS_CUDA(cudaMemcpyAsync(&host, res_dev, 16, cudaMemcpyDeviceToHost, st_));
+  HGKS_CUDA(cudaMemcpyAsync(host.lin, s.hs + (mk + 1) * mk + 1 + mk, 2 * sizeof(double), cudaMemcpyDeviceToHost, st_));
+  HGKS_CUDA(cudaMemcpyAsync(&nonphys, s.flags, sizeof(int), cudaMemcpyDeviceToHost, st_));
+  HGKS_CUDA(cudaMemsetAsync(s.flags, 0, sizeof(int), st_));
   HGKS_CUDA(cudaStreamSynchronize(st_));
-  const double res = host[0] / (double)m.N;
+  const double res = host.res / (double)m.N;
   if (info) {
     info->res_l1 = res;
-    info->lin_res[0] = host[1];
-    info->lin_res[1] = host[2];
-    info->nonphysical = flags[0];
+    info->lin_res[0] = host.lin[0];
+    info->lin_res[1] = host.lin[1];
+    info->nonphysical = nonphys;
   }
-  if (flags[1]) return fail(HGKS_ERR_CUDA, "a grid barrier of the GMRES solve timed out");
+  if (host.stuck) return barrier_failed(s, st_);
   if (!std::isfinite(res)) return fail(HGKS_ERR_NONPHYSICAL, "non-finite residual");
   return HGKS_OK;
 }
@@ -620,19 +626,21 @@ static hgks_status solve_impl(hgks_mesh mesh, const hgks_params *p, double *Q, d
   for (;; k++) {
     // the residual of the current state decides; the step then updates it
     launch_residual(m.d, m.s, *p, Q, G, m.s.R, p->scheme == HGKS_HWENO ? m.s.Gnew : nullptr, s_);
-    double *res_dev = m.s.hs + 65 * 64 + 200;
+    double *res_dev = m.s.hs + kHsRes;
     launch_density_l1(m.d, m.s, m.s.R, res_dev, s_);
-    double h = 0.0;
-    HGKS_CUDA(cudaMemcpyAsync(&h, res_dev, sizeof(double), cudaMemcpyDeviceToHost, s_));
+    struct { double res; int64_t stuck; } h;
+    HGKS_CUDA(cudaMemcpyAsync(&h, res_dev, sizeof(h), cudaMemcpyDeviceToHost, s_));
     HGKS_CUDA(cudaStreamSynchronize(s_));
-    res = h / (double)m.N;
+    if (h.stuck) { st = barrier_failed(m.s, s_); break; }
+    res = h.res / (double)m.N;
     if (!std::isfinite(res)) { st = fail(HGKS_ERR_NONPHYSICAL, "non-finite residual"); break; }
     if (hist_host) hist_host[k] = res;
     if (res > ref) ref = res;
     if (ref > 0.0 && res <= drop_tol * ref) { conv = true; break; }   // a zero reference certifies no drop
     if (k >= max_steps) break;
-    hgks_step_info si;
-    if ((st = gmres_step_impl(m, p, Q, G, nullptr, &si, s_, true))) break;
+    // the next residual follows the step on the stream: one wait of the host per step
+    if ((st = run_step(m, p, Q, G, nullptr, true, s_))) break;
+    HGKS_CUDA(cudaMemsetAsync(m.s.flags, 0, sizeof(int), s_));   // the step's non-physical count
   }
   if (info) { info->steps = k; info->converged = conv; info->res_ref = ref; info->res_final = res; }
   if (st) return st;

@@ -796,7 +796,7 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
   }
   cudaMemsetAsync(s.red_count + 2, 0, sizeof(unsigned), st);
   GridSolve a{m.N, C, m.cnb, s.jv64, s.dval, s.dinv, rhs, dx, s.t, s.V, s.z[0], s.z[1], s.red,
-              s.hs + (p.krylov_dim + 1) * p.krylov_dim + 1 + p.krylov_dim, s.vstride, s.red_count + 2, s.flags + 1,
+              s.hs + (p.krylov_dim + 1) * p.krylov_dim + 1 + p.krylov_dim, s.vstride, s.red_count + 2, reinterpret_cast<int *>(s.hs + kHsStuck),
               p.krylov_dim, p.restarts, p.jacobi_sweeps};
   void *args[] = {&a};
   HGKS_PROF_BEGIN(K_JACOBI, st);

@@ -155,7 +155,7 @@ struct Scratch {
   unsigned int *red_count = nullptr;
   double *hs = nullptr;          // small device scalars: H, beta, y, norms
   double *gram = nullptr;        // [65*65 + 2*65] inner products of the Krylov basis and the MGS pass sums
-  int *flags = nullptr;          // [8] device flags (nonphysical count, a grid barrier that gave up)
+  int *flags = nullptr;          // [8] device flags (nonphysical count)
   double *hostbuf = nullptr;     // [40][N] device state of the *_host entry points
   double *Qp = nullptr, *Rp = nullptr;   // [5][N] perturbed state and its residual (matrix-free products)
   int kdim = 0;
@@ -235,6 +235,8 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
 void launch_norm(const DevMesh &m, Scratch &s, const double *x, double *out_dev, cudaStream_t st);
 // force[3] on the boundary faces tagged `tag`, from the face fluxes of the last residual
 void launch_wall_force(const DevMesh &m, const Scratch &s, int tag, double *force_dev, cudaStream_t st);
+// hs slots: density L1 and, behind it, whether a grid barrier gave up (int64, read together)
+constexpr int kHsRes = 65 * 64 + 200, kHsStuck = kHsRes + 1;
 constexpr int kHsNormQ = 65 * 64 + 210;   // hs slots of the matrix-free products: ||Q||, ||x||, sigma, 0
 void launch_density_l1(const DevMesh &m, Scratch &s, const double *R, double *out_dev, cudaStream_t st);
 // G = G + relax (Gnew - G) (relax 0 or 1: G = Gnew)
