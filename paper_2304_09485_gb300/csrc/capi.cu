@@ -196,6 +196,8 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     m.bytes -= bytes;
   };
   if (implicit && kdim > s.kdim) {
+    // a captured step holds the addresses of the basis that goes
+    if (m.graph && m.graph->exec) { cudaGraphExecDestroy(m.graph->exec); m.graph->exec = nullptr; }
     if (s.V) { release(s.V, sizeof(double) * (size_t)(s.kdim + 1) * s.vstride); s.V = nullptr; }
     if (s.V32) { release(s.V32, sizeof(float) * (size_t)(s.kdim + 1) * s.vstride); s.V32 = nullptr; }
     s.kdim = kdim;

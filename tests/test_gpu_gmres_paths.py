@@ -69,3 +69,19 @@ def test_matrix_free_blocks(cuda, k):
     H.hgks_gmres_step(hm, H.hgks_default_params(**kw), Qd, None, dQ)
     Qo, _, _, _ = O.OracleMesh(m).gmres_step(O.make_params(**kw), Q)
     assert np.linalg.norm(hm.to_caller(dQ) - (Qo - Q)) / np.linalg.norm(Qo - Q) < 1e-4
+
+
+def test_step_after_a_larger_krylov_size(cuda):
+    """The basis moves when a later call needs more vectors; a step with the earlier
+    parameters and buffers must not replay with the old addresses."""
+    m, cond = I.sphere_mesh(4, 6, stretch=1.3), I.sphere_conditions(0.3)
+    Q, _ = I.smooth_state(m, amp=0.03, base=(1.0, 0.35, 0.03, -0.02, cond["p_inf"]))
+    hm = H.hgks_mesh_create(m, scheme_mask=1)
+    Q0 = hm.to_internal(Q)
+    Qd = Q0.clone()
+    out = []
+    for k in (4, 12, 4):
+        Qd.copy_(Q0)
+        H.hgks_gmres_step(hm, H.hgks_default_params(krylov_dim=k, **cond), Qd)
+        out.append(Qd.clone())
+    assert bool((out[0] == out[2]).all())
