@@ -665,17 +665,33 @@ __device__ __forceinline__ void dirs_of(const Units &u, const KParams &P, const 
 // d, derivatives with respect to a state of velocity p, with respect to Q0 (velocity p0): a
 // change of the reference velocity by (du, dv, dw) adds (0, du r, dv r, dw r,
 // (gamma - 1)(du . m + |du|^2 r / 2)); added to d0
-__device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim &p0, const Dir *d, double (*d0)[5]) {
+__device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim &p0, const Dir *d, double *d0, int bd) {
   const double du = p.U - p0.U, dv = p.V - p0.V, dw = p.W - p0.W, h = 0.5 * fma(du, du, fma(dv, dv, dw * dw));
 #pragma unroll
   for (int a = 0; a < 3; a++) {
-    d0[a][0] += d[a].r;
-    d0[a][1] += fma(du, d[a].r, d[a].u);
-    d0[a][2] += fma(dv, d[a].r, d[a].v);
-    d0[a][3] += fma(dw, d[a].r, d[a].w);
-    d0[a][4] += fma(g1, fma(du, d[a].u, fma(dv, d[a].v, fma(dw, d[a].w, h * d[a].r))), d[a].p);
+    double *o = d0 + 5 * a * bd;
+    o[0] += d[a].r;
+    o[bd] += fma(du, d[a].r, d[a].u);
+    o[2 * bd] += fma(dv, d[a].r, d[a].v);
+    o[3 * bd] += fma(dw, d[a].r, d[a].w);
+    o[4 * bd] += fma(g1, fma(du, d[a].u, fma(dv, d[a].v, fma(dw, d[a].w, h * d[a].r))), d[a].p);
   }
 }
+
+// a state or moments in a thread's column of shared memory (rows of bd)
+__device__ __forceinline__ void keep(double *c, int bd, const Prim &p) {
+  c[0] = p.rho; c[bd] = p.U; c[2 * bd] = p.V; c[3 * bd] = p.W; c[4 * bd] = p.il; c[5 * bd] = p.ir;
+}
+__device__ __forceinline__ void keep(double *c, int bd, const Mom &m) {
+  c[0] = m.m0; c[bd] = m.m1; c[2 * bd] = m.m2; c[3 * bd] = m.m3; c[4 * bd] = m.m4; c[5 * bd] = m.hd; c[6 * bd] = m.h0;
+}
+__device__ __forceinline__ Prim kept_prim(const double *c, int bd) {
+  return {c[0], c[bd], c[2 * bd], c[3 * bd], c[4 * bd], c[5 * bd]};
+}
+__device__ __forceinline__ Mom kept_mom(const double *c, int bd) {
+  return {c[0], c[bd], c[2 * bd], c[3 * bd], c[4 * bd], c[5 * bd], c[6 * bd]};
+}
+constexpr int kFluxRows = 34;          // doubles that a thread of k_flux keeps in shared memory
 
 // Flux of Eq. (flux), averaged over [0, dt], at one Gauss point and, for the compact scheme,
 // the point value of Eq. (point) at t*. Bound by the FP64 pipe (2 DFMA per SM and clock), so
@@ -688,13 +704,16 @@ __device__ __forceinline__ void add_shifted(double g1, const Prim &p, const Prim
 // with the functions of fp64.cuh and the parameters' divisions on the host 19.8 and 0.63 ms;
 // with g_0's derivatives from the sum of the characteristic ones 19.1 and 0.61 ms; products and
 // sums as FMAs of three registers (Units) 17.9 and 0.61 ms; sums shared by flux, heat flux and
-// point values 17.9 and 0.57 ms. ncu at 124,416 cells: 743 FP64 instructions a thread (inviscid),
-// the FP64 pipe 87 % busy with 8 warps an SM; 168 or 128 registers, with spills and more warps,
-// take 9 and 6 % longer.
+// point values 17.9 and 0.57 ms. ncu at 124,416 cells then: 743 FP64 instructions a thread
+// (inviscid), the FP64 pipe 87 % busy with 8 warps an SM. What lives through the whole loop and
+// is used once or twice (g_0's state and derivatives, g_r's state and moments) waits in shared
+// memory instead of in spills: 7.60 -> 7.46 ms at 6.0M Gauss points (inviscid, 995,328
+// tetrahedra), 0.567 -> 0.541 ms viscous and compact. The inviscid kernel then fits 168 registers, 12
+// warps an SM (128 registers, 16 warps: 7.81 ms); the compact one takes 240 (168: 0.572 ms).
 template <bool BATCH, class S, bool COMPACT>
-__global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
-                                                  const double *__restrict__ dt, const double *__restrict__ wface,
-                                                  double *__restrict__ fflux, double *__restrict__ fpt, int *__restrict__ flags) {
+__global__ void __launch_bounds__(COMPACT ? 256 : 384) k_flux(DevMesh m, KParams Pv, const double *__restrict__ Q,
+                                                                      const double *__restrict__ dt, const double *__restrict__ wface,
+                                                                      double *__restrict__ fflux, double *__restrict__ fpt, int *__restrict__ flags) {
   constexpr int NG = S::NG;
   const int N = m.N, F = m.F;
   const int FL = BATCH ? m.FL : F;
@@ -709,13 +728,19 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   for (int k = 0; k < 9; k++) T[k] = m.fT[(size_t)k * F + f];
   const int L = m.fl[f], R = m.fr[f];
   const bool inner = R >= 0;
+  // long-lived values of the thread wait in shared memory (rows of blockDim.x): the sum of the
+  // derivatives, g_r's state and moments, g_0's state
+  extern __shared__ double kept[];
+  const int bd = blockDim.x;
+  double *const kq = kept + threadIdx.x, *const kr = kq + 15 * bd, *const k0 = kq + 28 * bd;
   const Units u = units();
   const double g1 = u.add(P.g1, u.nz), K2 = u.add(P.K2, u.nz), K4 = u.add(P.K4, u.nz);   // in registers
-  Prim pl, pr;
-  Mom ml, mr;
+  Prim pk;               // state and moments of the Maxwellian at hand: g_l first
+  Mom mk;
   Eig e;
   int bad = 0;            // bit s: side s fell back to its cell average with zero slopes
   bool held = false;
+  double jump, pp0;       // |p_l - p_r| / (p_l + p_r), p of g_0
   {
     double QL[5], QR[5], Qs[5], Qsl[5], W[5], q[5];
 #pragma unroll
@@ -741,34 +766,35 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
       return rp;
     };
     double rp = side(0, QL);
-    pl = to_prim(u, W, rp);
-    ml = mom_half(u, pl, 1.0);
+    pk = to_prim(u, W, rp);
+    mk = mom_half(u, pk, 1.0);
     if (inner) {
       rp = side(1, QR);
     } else {
-      held = image_held(P, m.ftag[f], pl.il);
-      image_state(u, P, m.ftag[f], T, pl, ml.m1, held, W);
+      held = image_held(P, m.ftag[f], pk.il);
+      image_state(u, P, m.ftag[f], T, pk, mk.m1, held, W);
       rp = rho_p(u, W, g1);
     }
-    pr = to_prim(u, W, rp);
-    mr = mom_half(u, pr, -1.0);
-  }
-  // compatibility condition: Q0 = int_{u>0} psi g_l + int_{u<0} psi g_r
-  Prim p0;
-  {
+    const Prim pr = to_prim(u, W, rp);
+    const Mom mr = mom_half(u, pr, -1.0);
+    // compatibility condition: Q0 = int_{u>0} psi g_l + int_{u<0} psi g_r
     double Q0[5];
-    const double xl[5] = {u.mul(pl.rho, ml.m0), u.mul(pl.rho, ml.m1), 0.0, 0.0, u.mul(pl.rho, fma(u.mul(K2, pl.il), ml.m0, ml.m2))};
+    const double xl[5] = {u.mul(pk.rho, mk.m0), u.mul(pk.rho, mk.m1), 0.0, 0.0, u.mul(pk.rho, fma(u.mul(K2, pk.il), mk.m0, mk.m2))};
     const double xr[5] = {u.mul(pr.rho, mr.m0), u.mul(pr.rho, mr.m1), 0.0, 0.0, u.mul(pr.rho, fma(u.mul(K2, pr.il), mr.m0, mr.m2))};
-    from_frame(u, pl, xl, Q0);
+    from_frame(u, pk, xl, Q0);
     acc_from_frame(u, pr, xr, Q0);
-    p0 = to_prim(u, Q0, rho_p(u, Q0, g1));
+    const Prim p0 = to_prim(u, Q0, rho_p(u, Q0, g1));
+    keep(k0, bd, p0);
+    keep(kr, bd, pr);
+    keep(kr + 6 * bd, bd, mr);
+    const double prl = u.mul(pk.rho, pk.il), prr = u.mul(pr.rho, pr.il);
+    jump = fabs(u.mul(u.sub(prl, prr), rcp(u.add(prl, prr), u.one)));
+    pp0 = u.mul(p0.rho, p0.il);
   }
   double dtf;
   if (positive(P.flux_dt)) dtf = P.flux_dt;
   else dtf = (inner ? min_positive(dt[L], dt[R]) : dt[L]) * P.flux_dt_ratio;
   // collision time (Sec. 5) over dt, and the time coefficients of Eq. (flux) over dt
-  const double prl = u.mul(pl.rho, pl.il), prr = u.mul(pr.rho, pr.il), pp0 = u.mul(p0.rho, p0.il);
-  const double jump = fabs(u.mul(u.sub(prl, prr), rcp(u.add(prl, prr), u.one)));
   const double tq = fma(P.tau_C, jump, P.viscous ? P.mu * rcp(u.mul(pp0, dtf), u.one) : P.tau_eps);   // tau / dt
   const double eta = exp64(-rcp(tq, u.one));
   const double c4 = u.mul(tq, u.sub(u.one, eta)), k4 = u.mul(tq, c4), k42 = u.add(k4, k4), tau = u.mul(tq, dtf);
@@ -783,19 +809,15 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
   // other faces sum each side's primitive ones shifted to Q0's velocity.
   const bool sums = inner && P.characteristic;
   Dir d[3];
-  double q0[3][5];
+  if (!sums)
 #pragma unroll
-  for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = 0.0;
-  Prim pk = pl;
-  Mom mk = ml;
+    for (int a = 0; a < 15; a++) kq[a * bd] = 0.0;
   double C = c4, Ce = -c5, Cf = u.mul(-dtf, k4);              // flux: c rho <u psi> + e sum <u u_d d_d psi> + f <u d_t psi>
   double A = es, Ae = -es * (tau + ts), Af = -es * tau; // point value
 #pragma unroll 1
   for (int s = 0; s < 3; s++) {
     if (s < 2) {
-      if (s == 1 && !inner) {
-        image_slopes(m.ftag[f], pl, pr, held, d);
-      } else {
+      if (s == 0 || inner) {               // a boundary face's image derivatives are in d already
         const double *in = wface + ((size_t)(s * NG + g) * kFaceState + 5) * F + f;
         double q[3][5];
 #pragma unroll
@@ -804,22 +826,25 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
         if (sums) {
           if (s == 0) {
 #pragma unroll
-            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = q[a / 5][a % 5];
+            for (int a = 0; a < 15; a++) kq[a * bd] = q[a / 5][a % 5];
           } else {
 #pragma unroll
-            for (int a = 0; a < 15; a++) q0[a / 5][a % 5] = u.add(q0[a / 5][a % 5], q[a / 5][a % 5]);
+            for (int a = 0; a < 15; a++) kq[a * bd] = u.add(kq[a * bd], q[a / 5][a % 5]);
           }
         }
       }
-      if (!sums) add_shifted(g1, pk, p0, d, q0);
+      if (!sums) add_shifted(g1, pk, kept_prim(k0, bd), d, kq, bd);
     } else {
-      pk = p0;
-      mk = mom_full(u, p0);
+      pk = kept_prim(k0, bd);
+      mk = mom_full(u, pk);
+      double q[3][5];
+#pragma unroll
+      for (int a = 0; a < 15; a++) q[a / 5][a % 5] = kq[a * bd];
       if (sums) {
-        dirs_of(u, P, e, T, pk, q0, d);
+        dirs_of(u, P, e, T, pk, q, d);
       } else {
 #pragma unroll
-        for (int a = 0; a < 3; a++) d[a] = Dir{q0[a][0], q0[a][1], q0[a][2], q0[a][3], q0[a][4]};
+        for (int a = 0; a < 3; a++) d[a] = Dir{q[a][0], q[a][1], q[a][2], q[a][3], q[a][4]};
       }
       C = c1; Ce = 0.5 * c2; Cf = 0.5 * c3;
       A = 1.0 - es; Ae = 0.5 * fma(ts + tau, es, -tau); Af = 0.5 * (ts - tau + tau * es);
@@ -838,12 +863,16 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh m, KParams Pv, const doubl
         acc_state(u, pk, mk, z, K2, a, A1, A2, Ae, Pt);
       }
     }
-    pk = pr;
-    mk = mr;
+    if (s == 0) {
+      const Prim pr = kept_prim(kr, bd);
+      if (!inner) image_slopes(m.ftag[f], pk, pr, held, d);
+      pk = pr;
+      mk = kept_mom(kr + 6 * bd, bd);
+    }
   }
   if (prandtl) {
     // heat flux of the averaged distribution about the velocity of Q0 times 1/Pr - 1
-    const double U = p0.U, V = p0.V, W = p0.W, h2 = 0.5 * fma(U, U, fma(V, V, u.mul(W, W)));
+    const double U = pk.U, V = pk.V, W = pk.W, h2 = 0.5 * fma(U, U, fma(V, V, u.mul(W, W)));
     const double qf = fma(-U, Fl[1], fma(-V, Fl[2], fma(-W, Fl[3], fma(h2, Fl[0], Fl[4]))));
     const double qw = fma(-U, Wb[1], fma(-V, Wb[2], fma(-W, Wb[3], fma(h2, Wb[0], Wb[4]))));
     Fl[4] = fma(P.prandtl, fma(-U, qw, qf), Fl[4]);
@@ -1012,10 +1041,10 @@ void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const
   HGKS_PROF_END(K_RECON, st);
   HGKS_PROF_BEGIN(K_FLUX, st);
   const unsigned gf = S::NG * grid_for(FL, s.blk_flux);
-  if (p.scheme == HGKS_HWENO)
-    k_flux<BATCH, S, true><<<gf, s.blk_flux, 0, st>>>(m, p, Q, s.dt, s.wface, s.fflux, s.fpt, s.flags);
-  else
-    k_flux<BATCH, S, false><<<gf, s.blk_flux, 0, st>>>(m, p, Q, s.dt, s.wface, s.fflux, s.fpt, s.flags);
+  const size_t fshm = sizeof(double) * kFluxRows * s.blk_flux;
+  auto flux = p.scheme == HGKS_HWENO ? k_flux<BATCH, S, true> : k_flux<BATCH, S, false>;
+  cudaFuncSetAttribute(flux, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fshm);
+  flux<<<gf, s.blk_flux, fshm, st>>>(m, p, Q, s.dt, s.wface, s.fflux, s.fpt, s.flags);
   HGKS_PROF_END(K_FLUX, st);
   HGKS_PROF_BEGIN(K_GATHER, st);
   const int grad = p.scheme == HGKS_HWENO && Gnew != nullptr;   // gradients wanted
