@@ -160,12 +160,13 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     HGKS_CUDA(cudaMemset(s.wface, 0, sizeof(double) * 2 * NG * kFaceState * F));
   }
   s.vstride = (int64_t)((5 * N + 63) / 64 * 64);
-  // the off-diagonal part of A: operands of its products, or an arena's stored blocks
+  // the off-diagonal part of A: operands of its products, with two vectors in their z form
+  // behind them, or an arena's stored blocks
   const bool arena = m.d.ptab != nullptr;
   const size_t rows = arena ? 25 * NF : 6 + 5 * NF;
   double *&blocks = arena ? s.off : s.jv64;
   if (implicit && !blocks) {
-    if ((st = dalloc(m, &blocks, rows * N))) return st;
+    if ((st = dalloc(m, &blocks, (rows + (arena ? 0 : 12)) * N))) return st;
     if ((st = dalloc(m, &s.dval, N))) return st;
     if ((st = dalloc(m, &s.dinv, N))) return st;
     if ((st = dalloc(m, &s.R, 5 * N))) return st;
@@ -173,11 +174,10 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
     if ((st = dalloc(m, &s.dQ, 5 * N))) return st;
     if ((st = dalloc(m, &s.w, 5 * N))) return st;
     if ((st = dalloc(m, &s.t, 5 * N))) return st;
-    if ((st = dalloc(m, &s.t2, 5 * N))) return st;
+    if (arena && (st = dalloc(m, &s.t2, 5 * N))) return st;
     if ((st = dalloc(m, &s.hs, 65 * 64 + 256))) return st;
     if ((st = dalloc(m, &s.gram, 65 * 65 + 2 * 65 + 64))) return st;
-    for (double *&z : s.z)
-      if (!arena && (st = dalloc(m, &z, 6 * N))) return st;
+    for (int k = 0; k < 2 && !arena; k++) s.z[k] = blocks + (rows + 6 * k) * N;
     HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
     HGKS_CUDA(cudaMemset(s.hs + kHsStuck, 0, sizeof(double)));
   }

@@ -172,9 +172,9 @@ __device__ __forceinline__ T block_sum(T v) {
   }
   return s;   // valid in thread 0
 }
-// *out = sum of all blocks' v (mode 0) or its square root (mode 1), stored as double
-template <typename T>
-__device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, double *out, int mode) {
+// *out = sum of all blocks' v or its square root, stored as double
+template <bool ROOT, typename T>
+__device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, double *out) {
   __shared__ bool last;
   const T bs = block_sum(v);
   if (threadIdx.x == 0) {
@@ -190,7 +190,7 @@ __device__ __forceinline__ void grid_sum(T v, T *partials, unsigned int *count, 
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) s += ((volatile T *)partials)[b];
   s = block_sum(s);
   if (threadIdx.x == 0) {
-    *out = mode == 1 ? (double)sqrt(s) : (double)s;
+    *out = ROOT ? (double)sqrt(s) : (double)s;
     *count = 0u;
   }
 }
@@ -286,50 +286,25 @@ template <typename T> struct Vec16;
 template <> struct Vec16<double> { typedef double2 type; static constexpr int n = 2; };
 template <> struct Vec16<float> { typedef float4 type; static constexpr int n = 4; };
 
-// w -= h v (if v != nullptr); *out = (w, x) (mode 0) or ||w|| (x == w, mode 1).
-// In mode 1 nothing is read through x, so callers may pass w itself for it
-// without breaking the restrict qualifiers.
-// 16 bytes per vector per thread and step, four steps in flight; n need not be
-// a multiple of the vector width.
+// *out = ||w||. 16 bytes per thread and step, four steps in flight; n need not be a multiple of
+// the vector width.
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_axpy_dot(int64_t n, T *__restrict__ w, const T *__restrict__ v,
-                                                     const double *__restrict__ h, const T *__restrict__ x,
-                                                     int self, T *partials, unsigned int *count, double *out) {
+__global__ void __launch_bounds__(kBlock) k_norm(int64_t n, const T *__restrict__ w, T *partials, unsigned int *count,
+                                                 double *out) {
   typedef typename Vec16<T>::type TV;
   constexpr int L = Vec16<T>::n;
-  const T hv = v ? (T)(-*h) : T(0);
   T s = T(0);
   const int64_t nv = n / L, stride = (int64_t)gridDim.x * blockDim.x;
-  TV *wv = reinterpret_cast<TV *>(w);
-  const TV *vv = reinterpret_cast<const TV *>(v);
-  const TV *xv = reinterpret_cast<const TV *>(x);
+  const TV *wv = reinterpret_cast<const TV *>(w);
 #pragma unroll 4
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nv; k += stride) {
-    TV wk = wv[k];
-    T *wa = reinterpret_cast<T *>(&wk);
-    if (v) {
-      const TV vk = vv[k];
-      const T *va = reinterpret_cast<const T *>(&vk);
+    const TV wk = wv[k];
+    const T *wa = reinterpret_cast<const T *>(&wk);
 #pragma unroll
-      for (int l = 0; l < L; l++) wa[l] = fma(hv, va[l], wa[l]);
-      wv[k] = wk;
-    }
-    if (self) {
-#pragma unroll
-      for (int l = 0; l < L; l++) s = fma(wa[l], wa[l], s);
-    } else {
-      const TV xk = xv[k];
-      const T *xa = reinterpret_cast<const T *>(&xk);
-#pragma unroll
-      for (int l = 0; l < L; l++) s = fma(wa[l], xa[l], s);
-    }
+    for (int l = 0; l < L; l++) s = fma(wa[l], wa[l], s);
   }
-  for (int64_t k = nv * L + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += stride) {
-    T wk = w[k];
-    if (v) { wk = fma(hv, v[k], wk); w[k] = wk; }
-    s = fma(wk, self ? wk : x[k], s);
-  }
-  grid_sum(s, partials, count, out, self);
+  for (int64_t k = nv * L + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += stride) s = fma(w[k], w[k], s);
+  grid_sum<true>(s, partials, count, out);
 }
 
 // ---- modified Gram-Schmidt from one pass over the basis ----
@@ -477,7 +452,7 @@ __global__ void __launch_bounds__(kBlock) k_mupdate(int64_t n, T *__restrict__ w
     w[k] = wk;
     s = fma(wk, wk, s);
   }
-  grid_sum(s, partials, count, norm_out, 1);
+  grid_sum<true>(s, partials, count, norm_out);
 }
 
 // v = w / h (v = 0 after a breakdown h == 0), 16 bytes per thread and step
@@ -541,7 +516,7 @@ __global__ void __launch_bounds__(kBlock) k_density_l1(int N, const double *__re
                                                        double *partials, unsigned int *count, double *out) {
   double s = 0.0;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) s += fabs(R[k]) * inv_vol[k];
-  grid_sum<double>(s, partials, count, out, 0);
+  grid_sum<false, double>(s, partials, count, out);
 }
 
 __global__ void k_update(int64_t n5, int64_t ng, double *__restrict__ Q, const double *__restrict__ dQ, double *__restrict__ G,
@@ -604,8 +579,7 @@ void fd_apply(const DevMesh &m, Scratch &s, const hgks_params &p, const double *
   const int64_t n = 5 * (int64_t)m.N;
   double *nrm = s.hs + kHsNormQ;
   HGKS_PROF_BEGIN(K_DOT, st);
-  k_axpy_dot<TV><<<kRedBlocks, kBlock, 0, st>>>(n, const_cast<TV *>(x), nullptr, nullptr, x, 1, partials<TV>(s),
-                                                 s.red_count, nrm + 1);
+  k_norm<TV><<<kRedBlocks, kBlock, 0, st>>>(n, x, partials<TV>(s), s.red_count, nrm + 1);
   HGKS_PROF_END(K_DOT, st);
   HGKS_PROF_BEGIN(K_SPMV, st);
   k_fd_perturb<TV><<<vec_grid(n), kBlock, 0, st>>>(n, Q, x, nrm, s.Qp);
@@ -706,7 +680,7 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
       if (!fd && it == 0) r0 = rhs;        // dx = 0
     precondition_t<T>(m, s, k, p.jacobi_sweeps, r0, k.w, st);
     HGKS_PROF_BEGIN(K_DOT, st);
-    k_axpy_dot<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, nullptr, nullptr, k.w, 1, k.red, s.red_count, beta);
+    k_norm<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, k.red, s.red_count, beta);
     HGKS_PROF_END(K_DOT, st);
     if (it == 0) cudaMemcpyAsync(lres, beta, sizeof(double), cudaMemcpyDeviceToDevice, st);
     // v_j = w / h: FP64 with the assembled A, with the form that the products read; FP32 on the
@@ -795,8 +769,7 @@ void launch_precondition(const DevMesh &m, Scratch &s, int sweeps, const double 
 
 void launch_norm(const DevMesh &m, Scratch &s, const double *x, double *out_dev, cudaStream_t st) {
   HGKS_PROF_BEGIN(K_DOT, st);
-  k_axpy_dot<double><<<kRedBlocks, kBlock, 0, st>>>(5 * (int64_t)m.N, const_cast<double *>(x), nullptr, nullptr, x, 1,
-                                                     s.red, s.red_count, out_dev);
+  k_norm<double><<<kRedBlocks, kBlock, 0, st>>>(5 * (int64_t)m.N, x, s.red, s.red_count, out_dev);
   HGKS_PROF_END(K_DOT, st);
 }
 
