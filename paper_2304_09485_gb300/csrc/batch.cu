@@ -182,11 +182,13 @@ __global__ void __launch_bounds__(kB) k_baxpy_dot(int N, BatchDev bd, T *__restr
 // (kBatchMdot basis vectors per launch, per-mesh sums), solves for h per mesh
 // and subtracts sum h_i v_i in MGS order in one more pass with ||w||.
 
-// a(mesh)[k] = (w, v_k) for k in [k0, k0 + nk), g(mesh)[k] = (v_j, v_k) for those k < j
+// a(mesh)[k] = (w, v_k) for k in [k0, k0 + nk), g(mesh)[k] = (v_j, v_k) for those k < j; with the
+// last of them (k0 + nk > j) the mesh's last block also takes column j of the Gram matrix from g
+// and h_ij by forward substitution
 template <typename T>
 __global__ void __launch_bounds__(kB) k_bmdot(int N, BatchDev bd, const T *__restrict__ w, const T *__restrict__ V,
                                               int64_t vs, int k0, int nk, int j, T *part, double *hs, int hz, int aoff,
-                                              int goff) {
+                                              int goff, int mk, int gram_off) {
   const int i = blockIdx.x * kB + threadIdx.x;
   const int mesh = bd.bmesh[blockIdx.x];
   if (!bd.active[mesh]) return;
@@ -247,15 +249,9 @@ __global__ void __launch_bounds__(kB) k_bmdot(int N, BatchDev bd, const T *__res
     if (threadIdx.x == 0) rec[(q < kBatchMdot ? aoff : goff) + kk] = (double)sum;
   }
   if (threadIdx.x == 0) bd.counters[mesh] = 0u;
-}
-
-// one warp per mesh: column j of the Gram matrix from g, then h_ij by forward substitution
-__global__ void k_bmgs_coef(BatchDev bd, int j, int mk, double *__restrict__ hs, int hz, int aoff, int goff,
-                            int gram_off) {
-  const int mesh = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  if (mesh >= bd.nmesh || !bd.active[mesh]) return;
-  double *rec = hs + (size_t)mesh * hz;
-  mgs_coef_warp(threadIdx.x % 32, j, mk, mk + 1, rec + aoff, rec + goff, rec + gram_off, rec);
+  if (k0 + nk <= j) return;
+  __syncthreads();
+  if (threadIdx.x < 32) mgs_coef_warp(threadIdx.x, j, mk, mk + 1, rec + aoff, rec + goff, rec + gram_off, rec);
 }
 
 // w -= sum_{k <= j} h_kj(mesh) v_k in the order of k, then h_{j+1,j}(mesh) = ||w||
@@ -512,12 +508,9 @@ void bgmres_t(const DevMesh &m, Scratch &s, BatchState &bs, const BBuf<T> &k, co
         for (int k0 = 0; k0 <= j; k0 += kBatchMdot) {
           HGKS_PROF_BEGIN(K_DOT, st);
           k_bmdot<T><<<g, kB, 0, st>>>(N, bs.b, k.w, k.V, vs, k0, std::min(kBatchMdot, j + 1 - k0), j, k.part, bs.hs,
-                                       hz, bs.a_off, bs.g_off);
+                                       hz, bs.a_off, bs.g_off, mk, bs.gram_off);
           HGKS_PROF_END(K_DOT, st);
         }
-        HGKS_PROF_BEGIN(K_DOT, st);
-        k_bmgs_coef<<<(nm + 3) / 4, 128, 0, st>>>(bs.b, j, mk, bs.hs, hz, bs.a_off, bs.g_off, bs.gram_off);
-        HGKS_PROF_END(K_DOT, st);
         HGKS_PROF_BEGIN(K_DOT, st);
         k_bmupdate<T><<<g, kB, 0, st>>>(N, bs.b, k.w, k.V, vs, j, mk, bs.hs, hz, k.part);
         HGKS_PROF_END(K_DOT, st);

@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kBlock) k_norm(int64_t n, const T *__restrict_
 // h_i = (w_i, v_i), w_{i+1} = w_i - h_i v_i. Since w_i = w - sum_{k<i} h_k v_k,
 //   h_i = a_i - sum_{k<i} h_k G_ki,  a_i = (w, v_i),  G_ki = (v_k, v_i),
 // so one pass over the basis (k_mdot: all a_i, and the new row of G, v_j against
-// the older vectors) and a forward substitution (k_mgs_coef) give the same
+// the older vectors) and a forward substitution give the same
 // coefficients, and one more pass (k_mupdate) subtracts them in MGS order and
 // takes ||w||: about 2 (j + 1) vector passes instead of 4 (j + 1) for step j
 // (used with FP32 vectors, see gmres_t).
@@ -340,11 +340,16 @@ __device__ __forceinline__ void block_sum_all(T *v, T (*sh)[kBlock / 32], T *tot
   __syncthreads();
 }
 
-// a[k] = (w, v_k) for k in [k0, k0 + nk), and g[k] = (v_j, v_k) for those k < j
+constexpr int kGramLd = 65;
+// a[k] = (w, v_k) for k in [k0, k0 + nk), and g[k] = (v_j, v_k) for those k < j; with the last of
+// them (k0 + nk > j) the MGS coefficients of step j by forward substitution: column j of H, and
+// of the basis Gram matrix G (leading dimension kGramLd, G[k][i] = (v_k, v_i), k < i). The block
+// that adds the partial sums does it: a launch of its own per vector took
+// 9.86 instead of 9.83 ms for the mixed step of 294,912 tetrahedra, 9.18 instead of 9.06 for a batch of six.
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_mdot(int64_t n, const T *__restrict__ w, const T *__restrict__ V, int64_t vs,
                                                  int k0, int nk, int j, T *partials, unsigned int *count,
-                                                 double *__restrict__ a, double *__restrict__ g) {
+                                                 double *a, double *g, int mk, double *G, double *H) {
   typedef typename Vec16<T>::type TV;
   constexpr int L = Vec16<T>::n;
   T sa[kMdot], sg[kMdot];
@@ -408,15 +413,9 @@ __global__ void __launch_bounds__(kBlock) k_mdot(int64_t n, const T *__restrict_
   const int q = threadIdx.x, kk = k0 + q % kMdot;
   if (q < 2 * kMdot && q % kMdot < nk && (q < kMdot || kk < j)) (q < kMdot ? a : g)[kk] = (double)tot[q];
   if (threadIdx.x == 0) *count = 0u;
-}
-
-// the MGS coefficients of step j by forward substitution; column j of H and row
-// j of the basis Gram matrix G (leading dimension kGramLd, G[k][i] = (v_k, v_i), k < i)
-constexpr int kGramLd = 65;
-// (a lane per coefficient, two beyond 32: each h_i subtracts its terms in the order of k)
-__global__ void k_mgs_coef(int j, int mk, const double *__restrict__ a, const double *__restrict__ g,
-                           double *__restrict__ G, double *__restrict__ H) {
-  mgs_coef_warp(threadIdx.x, j, mk, kGramLd, a, g, G, H);
+  if (k0 + nk <= j) return;
+  __syncthreads();
+  if (threadIdx.x < 32) mgs_coef_warp(threadIdx.x, j, mk, kGramLd, a, g, G, H);
 }
 
 // w -= sum_{k <= j} h_kj v_k in the order of k (MGS order), then h_{j+1,j} = ||w||
@@ -712,12 +711,9 @@ void gmres_t(const DevMesh &m, Scratch &s, const KBuf<T> &k, const hgks_params &
         for (int k0 = 0; k0 <= j; k0 += kMdot) {
           HGKS_PROF_BEGIN(K_DOT, st);
           k_mdot<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, k.V, vs, k0, std::min(kMdot, j + 1 - k0), j, k.red,
-                                                    s.red_count, ga, gg);
+                                                    s.red_count, ga, gg, mk, gram, H);
           HGKS_PROF_END(K_DOT, st);
         }
-        HGKS_PROF_BEGIN(K_DOT, st);
-        k_mgs_coef<<<1, 32, 0, st>>>(j, mk, ga, gg, gram, H);
-        HGKS_PROF_END(K_DOT, st);
         HGKS_PROF_BEGIN(K_DOT, st);
         k_mupdate<T><<<kRedBlocks, kBlock, 0, st>>>(n, k.w, k.V, vs, j, mk, H, k.red, s.red_count, H + (j + 1) * mk + j);
         HGKS_PROF_END(K_DOT, st);
