@@ -38,30 +38,25 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # the rate measured in the same run (hgks_fp64_peak: DFMA chains); this nominal
 # figure is reported beside it.
 FP64_NOMINAL_GFLOPS = 1258.6
-# The work per unit of each FP64-bound kernel, held fixed (the roofline
-# numerator): FP64 flops (2 per DFMA, 1 per DADD/DMUL) per unit, counted once by
-# ncu's SASS instruction counters on the 124,416-tet sphere (non-compact scheme,
-# inviscid, Pr = 1) for the kernels of the step at 190.8 ms per 2.36M-tet step,
-# and frozen there as the method's work per unit: a later rewrite that needs
-# fewer operations for the same result shows as a higher fraction, not a lower
-# count. DRAM bytes per unit of work from the same ncu captures
-# (dram__bytes_read.sum + dram__bytes_write.sum divided by the units of the
-# 124,416-tet launch); the traffic of a full launch is this times its units.
-# Since those captures the kernels were templated on the cell shape; their
-# tetrahedral instances are the same loops with the face count as a template
-# argument, compile to the same registers, stack frame and spills (-Xptxas -v)
-# and take the same time per launch, so the counters still describe them.
-KERNEL_TRAFFIC = {"flux": 395.6, "recon": 957.6, "jacobi": 858.0, "spmv": 935.0}
+# The work per unit of each FP64-bound kernel (the roofline numerator): FP64
+# instructions per unit (DFMA + DADD + DMUL, each one slot of the FP64 pipe and
+# counted as 2 flops like the DFMAs of the measured peak: the kernels form sums
+# and products as FMAs too), counted once by ncu's instruction counters on a
+# 648,000-tet sphere (non-compact scheme, inviscid, Pr = 1). DRAM bytes per unit
+# of work from the same capture (dram__bytes_read.sum + dram__bytes_write.sum
+# divided by the units of the launch); the traffic of a full launch is this times
+# its units.
+KERNEL_TRAFFIC = {"flux": 397.3, "recon": 925.6, "jacobi": 320.0, "spmv": 455.0}
 KERNEL_FLOPS = {
-    "flux": (2242.5, lambda N, F: 3 * F),        # per face Gauss point
-    "recon": (3000.9, lambda N, F: 4 * N),       # per (cell, face)
-    # the Krylov products: "jacobi" = products D^-1 O x (120 of a C2 step's 126
-    # launches are the E products of the Neumann form, 195.7 flop; 6 are the sweeps
-    # of the restart vector, ~219), "spmv" = products with O plus a vector (60 of 63
-    # are the final v + E z products with the fused inner product, 216.9; 3 are
-    # r0 = b - A x, 195.7): launch-weighted means per cell
-    "jacobi": (196.8, lambda N, F: N),
-    "spmv": (215.9, lambda N, F: N),
+    "flux": (2 * 732.0, lambda N, F: 3 * F),     # per face Gauss point
+    "recon": (2 * 1466.0, lambda N, F: 4 * N),   # per (cell, face)
+    # the Krylov products per cell: "jacobi" = products D^-1 O x of the Neumann form
+    # (81.75 instructions, 120 of a C2 step's 126 launches) and the sweeps of the
+    # restart vector; "spmv" = the final v + E z products with the fused inner
+    # products (84.0 with two of them, five more for each of up to four; 60 of 62):
+    # launch-weighted means
+    "jacobi": (2 * 82.0, lambda N, F: N),
+    "spmv": (2 * 91.9, lambda N, F: N),
 }
 
 
@@ -1001,7 +996,7 @@ def main():
             r.update({"achieved": fl / avg_s / 1e9, "frac": fl / avg_s / 1e9 / fp64_peak, "flops_per_launch": fl})
             if name in KERNEL_TRAFFIC:
                 r["traffic"] = KERNEL_TRAFFIC[name] * units(m.n_tet, F)
-                r["traffic_note"] = "bytes per launch: ncu dram bytes per unit on the 124,416-tet sphere x units"
+                r["traffic_note"] = "bytes per launch: ncu dram bytes per unit on a 648,000-tet sphere x units"
         else:
             r.update({"achieved": None, "frac": None})
         return r
