@@ -239,14 +239,29 @@ __global__ void __launch_bounds__(kB) k_bmdot(int N, BatchDev bd, const T *__res
   __threadfence();
   double *rec = hs + (size_t)mesh * hz;
   const int b0 = bd.bstart[mesh], b1 = b0 + bd.bcount[mesh];
+  // all slots at once, each in the order of bsum: loads of all in flight, two barriers instead of two a slot
+  T v[2 * kBatchMdot];
+#pragma unroll
+  for (int q = 0; q < 2 * kBatchMdot; q++) v[q] = T(0);
+  auto want = [&](int q) { return q < kBatchMdot ? q < nk : q - kBatchMdot < nk && k0 + q - kBatchMdot < j; };
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+#pragma unroll
+    for (int q = 0; q < 2 * kBatchMdot; q++)
+      if (want(q)) v[q] += ((volatile T *)part)[(size_t)q * nb + b];
+#pragma unroll
   for (int q = 0; q < 2 * kBatchMdot; q++) {
-    const int kk = k0 + (q % kBatchMdot);
-    const bool want = (q % kBatchMdot) < nk && (q < kBatchMdot || kk < j);   // uniform over the block
-    if (!want) continue;
-    T sum = T(0);
-    for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) sum += ((volatile T *)part)[(size_t)q * nb + b];
-    sum = bsum(sum);
-    if (threadIdx.x == 0) rec[(q < kBatchMdot ? aoff : goff) + kk] = (double)sum;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if (lane == 0) wsum[q][warp] = v[q];
+  }
+  __syncthreads();
+  constexpr int W = kB / 32;
+  if (threadIdx.x < 2 * kBatchMdot * W) {               // W lanes per slot
+    const int q = threadIdx.x / W;
+    T sum = wsum[q][threadIdx.x % W];
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o, W);
+    if (threadIdx.x % W == 0 && want(q)) rec[(q < kBatchMdot ? aoff : goff) + k0 + q % kBatchMdot] = (double)sum;
   }
   if (threadIdx.x == 0) bd.counters[mesh] = 0u;
   if (k0 + nk <= j) return;
