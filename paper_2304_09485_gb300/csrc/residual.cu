@@ -202,14 +202,16 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 // The projection stays in shared memory for three variables at a time, (P - D, q0 - 2 P, P + D),
 // then the two shear waves: 66 doubles a thread on tetrahedra (three blocks of 128 threads an SM),
 // 102 on hexahedra (two; all five variables at once, 170, left four warps an SM and cost 12 %).
+// Registers to match: 168 for 12 warps an SM, 255 for 8 (hexahedra with 168 spilled 348 bytes a
+// thread: 0.843 -> 0.825 ms for 35,937, 4.07 -> 4.00 for 190,464).
 // Against dense rows per variable: 28.5 -> 22.8 ms for 9.4M (cell, face) pairs (2,359,296
-// tetrahedra), 1.24 -> 0.84 ms for 35,937 hexahedra. ncu at 124,416 cells, before the sums and
-// products became FMAs of three registers: 1,471 FP64 instructions a thread, the pipe 89 % busy.
+// tetrahedra), 1.24 -> 0.83 ms for 35,937 hexahedra. ncu at 648,000 tetrahedra: 1,466 FP64 instructions a
+// thread, the pipe 97 % busy.
 constexpr int kReconMax = 256, kReconHex = 128;
 template <class S> constexpr int recon_rows() { return 3 * (10 + 3 * ShapeOf<S>::NSUB); }
 template <bool BATCH, class S>
-__global__ void __maxnreg__(168) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
-                                                     const double *__restrict__ coef, double *__restrict__ wface) {
+__global__ void __launch_bounds__(S::NF == 4 ? 384 : 256) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
+                                                                           const double *__restrict__ coef, double *__restrict__ wface) {
   constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB, NV = 9 + 3 * NSUB;
   extern __shared__ double proj[];                      // [3][NV + 1][blockDim.x]: column of this thread
   const int N = m.N, F = m.F;
