@@ -201,18 +201,21 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 //   den = D + tz (g0 R_0 + gm sum R_m).
 // The projection stays in shared memory for three variables at a time, (P - D, q0 - 2 P, P + D),
 // then the two shear waves: 66 doubles a thread on tetrahedra (three blocks of 128 threads an SM),
-// 102 on hexahedra (two; all five variables at once, 170, left four warps an SM and cost 12 %).
+// 102 on hexahedra, 84 with the compact scheme (two; all five variables at once, 170, left four warps
+// an SM and cost 12 %).
 // Registers to match: 168 for 12 warps an SM, 255 for 8 (hexahedra with 168 spilled 348 bytes a
 // thread: 0.843 -> 0.825 ms for 35,937, 4.07 -> 4.00 for 190,464).
 // Against dense rows per variable: 28.5 -> 22.8 ms for 9.4M (cell, face) pairs (2,359,296
 // tetrahedra), 1.24 -> 0.83 ms for 35,937 hexahedra. ncu at 648,000 tetrahedra: 1,466 FP64 instructions a
 // thread, the pipe 97 % busy.
+// NSUB: the scheme's sub-polynomials, one per sub-stencil or (compact) per face: on hexahedra k_coef
+// writes six vectors of three for the compact scheme and eight for the other, and no more are read.
 constexpr int kReconMax = 256, kReconHex = 128;
-template <class S> constexpr int recon_rows() { return 3 * (10 + 3 * ShapeOf<S>::NSUB); }
-template <bool BATCH, class S>
+constexpr int recon_rows(int nsub) { return 3 * (10 + 3 * nsub); }
+template <bool BATCH, class S, int NSUB>
 __global__ void __launch_bounds__(S::NF == 4 ? 384 : 256) k_recon(DevMesh m, KParams Pv, const double *__restrict__ Q,
                                                                            const double *__restrict__ coef, double *__restrict__ wface) {
-  constexpr int NF = S::NF, NG = S::NG, NSUB = ShapeOf<S>::NSUB, NV = 9 + 3 * NSUB;
+  constexpr int NF = S::NF, NG = S::NG, NV = 9 + 3 * NSUB;
   extern __shared__ double proj[];                      // [3][NV + 1][blockDim.x]: column of this thread
   const int N = m.N, F = m.F;
   const int NL = BATCH ? m.NL : N;
@@ -1037,9 +1040,11 @@ void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const
   HGKS_PROF_END(K_COEF, st);
   HGKS_PROF_BEGIN(K_RECON, st);
   const int br = std::min(s.blk_recon, S::NF == 4 ? kReconMax : kReconHex);
-  const size_t shm = sizeof(double) * recon_rows<S>() * br;
-  cudaFuncSetAttribute(k_recon<BATCH, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-  k_recon<BATCH, S><<<S::NF * grid_for(NL, br), br, shm, st>>>(m, p, Q, s.coef, s.wface);
+  const bool weno = p.scheme == HGKS_WENO;
+  const size_t shm = sizeof(double) * recon_rows(weno ? S::NSUBW : S::NF) * br;
+  auto recon = weno ? k_recon<BATCH, S, S::NSUBW> : k_recon<BATCH, S, S::NF>;
+  cudaFuncSetAttribute(recon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  recon<<<S::NF * grid_for(NL, br), br, shm, st>>>(m, p, Q, s.coef, s.wface);
   HGKS_PROF_END(K_RECON, st);
   HGKS_PROF_BEGIN(K_FLUX, st);
   const unsigned gf = S::NG * grid_for(FL, s.blk_flux);

@@ -1,0 +1,23 @@
+// Test-only shim: reaches into mesh and batch handles of the loaded libhgks.so, to put its
+// scratch and launch shapes into states that no public call produces on demand.
+#include <cstring>
+#include "../../paper_2304_09485_gb300/csrc/batch_impl.h"
+
+using namespace hgks;
+
+// as in batch_capi.cu
+struct hgks_batch_s {
+  Batch *B;
+};
+
+// every byte of the reconstruction coefficients: 0xff makes NaNs
+extern "C" int hx_fill_coef(hgks_mesh h, int byte) {
+  Mesh &m = *mesh_of(h);
+  const size_t rows = m.d.hex ? ShapeOf<HexShape>::COEF : ShapeOf<TetShape>::COEF;
+  return cudaMemset(m.s.coef, byte, sizeof(double) * rows * m.N) != cudaSuccess;
+}
+extern "C" int hx_fill_batch_coef(hgks_batch b, int byte) {
+  Mesh &m = b->B->m;
+  const size_t rows = m.d.hex ? ShapeOf<HexShape>::COEF : ShapeOf<TetShape>::COEF;
+  return cudaMemset(m.s.coef, byte, sizeof(double) * rows * m.N) != cudaSuccess;
+}
