@@ -776,22 +776,28 @@ const void *grid_kernel(int lpc, bool one) {
 }  // namespace
 
 // All restart cycles in one cooperative launch, for meshes small enough. false: not launched
-// (mesh too large, or no cooperative launches).
+// (mesh too large, or not on this device), which depends on the mesh and the device alone; a launch
+// that fails all the same is an error like any other launch's.
 bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double *rhs, double *dx, cudaStream_t st) {
-  int dev = 0, sms = 0, coop = 0;
+  int dev = 0, sms = 0, coop = 0, shm_max = 0;
   if (m.N > kGridCells || p.restarts < 1 || p.krylov_dim > kPMax || cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&shm_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (!coop || sms < 1) return false;
   const int blocks = std::min({sms, kPG, (m.N + 7) / 8}), C = (m.N + blocks - 1) / blocks;
   const int lpc = C <= 32 ? 4 : C <= 64 ? 2 : 1;        // one warp per SM sub-partition at most
   const bool one = C <= kPT;
   const size_t shm = sizeof(GridShared) + (one ? 0 : sizeof(double) * 5 * C);
   const void *fn = m.hex ? grid_kernel<HexShape::NF>(lpc, one) : grid_kernel<TetShape::NF>(lpc, one);
+  // The limit is the kernel's, for all threads of the process: always the device's largest, not this
+  // mesh's, which another thread's smaller mesh would lower before the launch.
+  const bool clean = cudaPeekAtLastError() == cudaSuccess;
   int fit = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess ||
+  if (shm > (size_t)shm_max ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, shm_max) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, kPT + 32, shm) != cudaSuccess || fit < 1) {
-    cudaGetLastError();
+    if (clean) cudaGetLastError();                      // an error of an earlier launch stays
     return false;
   }
   cudaMemsetAsync(s.red_count + 2, 0, sizeof(unsigned), st);
@@ -800,10 +806,9 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
               p.krylov_dim, p.restarts, p.jacobi_sweeps};
   void *args[] = {&a};
   HGKS_PROF_BEGIN(K_JACOBI, st);
-  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPT + 32), args, shm, st);
+  cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPT + 32), args, shm, st);
   HGKS_PROF_END(K_JACOBI, st);
-  if (e != cudaSuccess) cudaGetLastError();
-  return e == cudaSuccess;
+  return true;
 }
 
 }  // namespace hgks

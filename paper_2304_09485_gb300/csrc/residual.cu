@@ -696,7 +696,7 @@ __device__ __forceinline__ Prim kept_prim(const double *c, int bd) {
 __device__ __forceinline__ Mom kept_mom(const double *c, int bd) {
   return {c[0], c[bd], c[2 * bd], c[3 * bd], c[4 * bd], c[5 * bd], c[6 * bd]};
 }
-constexpr int kFluxRows = 34;          // doubles that a thread of k_flux keeps in shared memory
+constexpr int kFluxRows = 34, kFluxMax = 256;   // doubles that a thread of k_flux keeps in shared memory, threads of a block
 
 // Flux of Eq. (flux), averaged over [0, dt], at one Gauss point and, for the compact scheme,
 // the point value of Eq. (point) at t*. Bound by the FP64 pipe (2 DFMA per SM and clock), so
@@ -1027,6 +1027,13 @@ void launch_local_dt(const DevMesh &m, const hgks_params &hp, const double *Q, d
 }
 
 namespace {
+// Raises a kernel's dynamic shared memory to that of its largest block. The limit is the kernel's,
+// for all threads of the process: a value of the caller's own block shape would refuse the launch
+// of another thread that has just set a larger one. A failure shows in the launch that follows.
+template <class K>
+void allow_shared(K *kernel, size_t bytes_per_thread, int max_threads) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes_per_thread * max_threads));
+}
 // the four residual kernels of one cell kind
 template <bool BATCH, class S>
 void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const double *Q, const double *G, double *R,
@@ -1039,19 +1046,19 @@ void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const
   else k_coef_hweno<BATCH, S><<<gc, kBlock, 0, st>>>(m, Q, G, s.coef);
   HGKS_PROF_END(K_COEF, st);
   HGKS_PROF_BEGIN(K_RECON, st);
-  const int br = std::min(s.blk_recon, S::NF == 4 ? kReconMax : kReconHex);
+  constexpr int rmax = S::NF == 4 ? kReconMax : kReconHex;
+  const int br = std::min(s.blk_recon, rmax);
   const bool weno = p.scheme == HGKS_WENO;
-  const size_t shm = sizeof(double) * recon_rows(weno ? S::NSUBW : S::NF) * br;
+  const size_t row = sizeof(double) * recon_rows(weno ? S::NSUBW : S::NF);
   auto recon = weno ? k_recon<BATCH, S, S::NSUBW> : k_recon<BATCH, S, S::NF>;
-  cudaFuncSetAttribute(recon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-  recon<<<S::NF * grid_for(NL, br), br, shm, st>>>(m, p, Q, s.coef, s.wface);
+  allow_shared(recon, row, rmax);
+  recon<<<S::NF * grid_for(NL, br), br, row * br, st>>>(m, p, Q, s.coef, s.wface);
   HGKS_PROF_END(K_RECON, st);
   HGKS_PROF_BEGIN(K_FLUX, st);
-  const unsigned gf = S::NG * grid_for(FL, s.blk_flux);
-  const size_t fshm = sizeof(double) * kFluxRows * s.blk_flux;
+  const int bf = std::min(s.blk_flux, kFluxMax);
   auto flux = p.scheme == HGKS_HWENO ? k_flux<BATCH, S, true> : k_flux<BATCH, S, false>;
-  cudaFuncSetAttribute(flux, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fshm);
-  flux<<<gf, s.blk_flux, fshm, st>>>(m, p, Q, s.dt, s.wface, s.fflux, s.fpt, s.flags);
+  allow_shared(flux, sizeof(double) * kFluxRows, kFluxMax);
+  flux<<<S::NG * grid_for(FL, bf), bf, sizeof(double) * kFluxRows * bf, st>>>(m, p, Q, s.dt, s.wface, s.fflux, s.fpt, s.flags);
   HGKS_PROF_END(K_FLUX, st);
   HGKS_PROF_BEGIN(K_GATHER, st);
   const int grad = p.scheme == HGKS_HWENO && Gnew != nullptr;   // gradients wanted

@@ -19,4 +19,12 @@ def load(directory):
     L = C.CDLL(out)
     for f in ("hx_fill_coef", "hx_fill_batch_coef"):
         getattr(L, f).argtypes = [C.c_void_p, C.c_int]
+    L.hx_batch_shape.argtypes = [C.c_void_p, C.c_int, C.c_int]
     return L
+
+
+def limit_recorder(directory):
+    """limit_recorder.c as a library to preload."""
+    out = os.path.join(str(directory), "liblimit_recorder.so")
+    subprocess.check_call(["gcc", "-O1", "-fPIC", "-shared", os.path.join(HERE, "limit_recorder.c"), "-o", out, "-ldl"])
+    return out

@@ -21,3 +21,9 @@ extern "C" int hx_fill_batch_coef(hgks_batch b, int byte) {
   const size_t rows = m.d.hex ? ShapeOf<HexShape>::COEF : ShapeOf<TetShape>::COEF;
   return cudaMemset(m.s.coef, byte, sizeof(double) * rows * m.N) != cudaSuccess;
 }
+
+// block shapes of k_recon and k_flux, as the autotuner sets them
+extern "C" void hx_batch_shape(hgks_batch b, int recon, int flux) {
+  b->B->m.s.blk_recon = recon;
+  b->B->m.s.blk_flux = flux;
+}
