@@ -321,8 +321,8 @@ __device__ __forceinline__ bool grid_barrier(const GridSolve &a, GridShared &S, 
     unsigned seen, spin = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
-    } while (seen < want && ++spin < kSpin);
-    if (seen < want) {
+    } while (!arrived(seen, want) && ++spin < kSpin);
+    if (!arrived(seen, want)) {
       S.dead = 1;
       atomicExch(a.err, 1);
     }

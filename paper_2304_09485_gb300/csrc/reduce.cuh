@@ -4,6 +4,11 @@
 
 namespace hgks {
 
+// Whether a counter of arrivals has reached `want`. Both are taken modulo 2^32: a solve of many
+// restarts passes 2^32 arrivals (28 million barriers of 152 blocks), and the counter is never
+// further than one barrier's blocks from what is waited for.
+__host__ __device__ inline bool arrived(unsigned seen, unsigned want) { return (int)(seen - want) >= 0; }
+
 // The sums over a warp of K values per lane (K a power of two): lane l returns the sum of
 // value l / (32 / K). Each exchange halves the values a lane holds, so the K sums take
 // K - 1 + log2(32 / K) additions instead of 5 K: a warp-wide FP64 addition holds
