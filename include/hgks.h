@@ -252,7 +252,9 @@ hgks_status hgks_precondition(hgks_mesh mesh, int32_t sweeps, const double *b, d
  * taken two vectors per pass, an FP32 basis from one pass with its Gram
  * matrix), Q += dQ, and G = G_new for the compact scheme. Q, G are device
  * arrays updated in place; dQ_out (device, may be NULL) receives the update.
- * Synchronises the stream (to return info->res_l1). */
+ * Synchronises the stream (to return info->res_l1). When the solve does not end
+ * (HGKS_ERR_CUDA, a grid barrier that timed out) Q and G stay as they were and
+ * dQ_out holds an unfinished update. */
 hgks_status hgks_gmres_step(hgks_mesh mesh, const hgks_params *p, double *Q, double *G,
                             double *dQ_out, hgks_step_info *info, void *cuda_stream);
 

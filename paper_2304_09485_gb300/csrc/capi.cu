@@ -512,7 +512,7 @@ static hgks_status enqueue_step(Mesh &m, const hgks_params *p, double *Q, double
   hgks_status st = gmres_solve(d, s, *p, s.R, s.dQ, nullptr, st_, Q, G);
   if (st) return st;
   if (dQ_out) HGKS_CUDA(cudaMemcpyAsync(dQ_out, s.dQ, sizeof(double) * 5 * m.N, cudaMemcpyDeviceToDevice, st_));
-  launch_update(d, Q, s.dQ, G, s.Gnew, p->scheme == HGKS_HWENO ? 15 : 0, p->grad_relax, st_);
+  launch_update(d, s, Q, s.dQ, G, s.Gnew, p->scheme == HGKS_HWENO ? 15 : 0, p->grad_relax, st_);
   return last_launch();
 }
 

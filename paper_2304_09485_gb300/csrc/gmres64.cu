@@ -292,7 +292,6 @@ constexpr int kPMax = 64;       // Krylov vectors at most
 // 576,000 39.0 / 39.9; beyond 700,000 w no longer fits shared memory, and with w in global memory
 // 766,656 take 53.3 / 52.3, 2,359,296 159 / 153.
 constexpr int kGridCells = 600000;
-constexpr unsigned kSpin = 1u << 22;   // polls of a barrier (a second or more) before it gives up
 
 struct GridSolve {
   int N, C;                     // cells, cells per block
@@ -302,6 +301,7 @@ struct GridSolve {
   int64_t vs;
   unsigned *bar;                // arrivals, 0 at launch
   int *err;                     // set to 1 by a barrier that gave up
+  unsigned want, polls;         // arrivals that open a barrier, polls before it gives up
   int mk, restarts, sweeps;
 };
 
@@ -314,14 +314,14 @@ struct GridShared {
 
 // The arrival of every block at step `gen` (1, 2, ...). false: given up, the block returns.
 __device__ __forceinline__ bool grid_barrier(const GridSolve &a, GridShared &S, unsigned &gen) {
-  const unsigned want = ++gen * gridDim.x;
+  const unsigned want = ++gen * a.want;
   __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
     unsigned seen, spin = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.bar) : "memory");
-    } while (!arrived(seen, want) && ++spin < kSpin);
+    } while (!arrived(seen, want) && ++spin < a.polls);
     if (!arrived(seen, want)) {
       S.dead = 1;
       atomicExch(a.err, 1);
@@ -803,7 +803,7 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
   cudaMemsetAsync(s.red_count + 2, 0, sizeof(unsigned), st);
   GridSolve a{m.N, C, m.cnb, s.jv64, s.dval, s.dinv, rhs, dx, s.t, s.V, s.z[0], s.z[1], s.red,
               s.hs + (p.krylov_dim + 1) * p.krylov_dim + 1 + p.krylov_dim, s.vstride, s.red_count + 2, reinterpret_cast<int *>(s.hs + kHsStuck),
-              p.krylov_dim, p.restarts, p.jacobi_sweeps};
+              blocks + s.grid_extra, s.grid_polls, p.krylov_dim, p.restarts, p.jacobi_sweeps};
   void *args[] = {&a};
   HGKS_PROF_BEGIN(K_JACOBI, st);
   cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPT + 32), args, shm, st);

@@ -159,6 +159,9 @@ struct Scratch {
   double *hostbuf = nullptr;     // [40][N] device state of the *_host entry points
   double *Qp = nullptr, *Rp = nullptr;   // [5][N] perturbed state and its residual (matrix-free products)
   int kdim = 0;
+  // the wait of the one-launch GMRES (gmres64.cu): polls before it gives up (a second or more), and
+  // arrivals expected beyond the launch's own blocks (none; set by the test of a wait that runs out)
+  unsigned grid_polls = 1u << 22, grid_extra = 0;
   size_t bytes = 0;
   int blk_recon = 128, blk_flux = 128;   // launch shapes of the two FP64-bound kernels (autotuned for batches)
 };
@@ -239,9 +242,9 @@ void launch_wall_force(const DevMesh &m, const Scratch &s, int tag, double *forc
 constexpr int kHsRes = 65 * 64 + 200, kHsStuck = kHsRes + 1;
 constexpr int kHsNormQ = 65 * 64 + 210;   // hs slots of the matrix-free products: ||Q||, ||x||, sigma, 0
 void launch_density_l1(const DevMesh &m, Scratch &s, const double *R, double *out_dev, cudaStream_t st);
-// G = G + relax (Gnew - G) (relax 0 or 1: G = Gnew)
-void launch_update(const DevMesh &m, double *Q, const double *dQ, double *G, const double *Gnew, int ncomp_g,
-                   double relax, cudaStream_t st);
+// Q = Q + dQ, G = G + relax (Gnew - G) (relax 0 or 1: G = Gnew); neither when hs[kHsStuck] is set
+void launch_update(const DevMesh &m, const Scratch &s, double *Q, const double *dQ, double *G, const double *Gnew,
+                   int ncomp_g, double relax, cudaStream_t st);
 // batches (batch.cu): one launch per phase for all meshes of the batch
 void launch_batch_gmres(const DevMesh &m, Scratch &s, BatchState &bs, const hgks_params &p, const double *rhs,
                         double *dx, cudaStream_t st);

@@ -20,6 +20,8 @@ def load(directory):
     for f in ("hx_fill_coef", "hx_fill_batch_coef"):
         getattr(L, f).argtypes = [C.c_void_p, C.c_int]
     L.hx_batch_shape.argtypes = [C.c_void_p, C.c_int, C.c_int]
+    L.hx_barrier.argtypes = [C.c_void_p, C.c_uint, C.c_uint]
+    L.hx_set_stuck.argtypes = [C.c_void_p]
     return L
 
 

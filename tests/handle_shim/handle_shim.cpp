@@ -27,3 +27,15 @@ extern "C" void hx_batch_shape(hgks_batch b, int recon, int flux) {
   b->B->m.s.blk_recon = recon;
   b->B->m.s.blk_flux = flux;
 }
+
+// a one-launch GMRES whose barriers expect `extra` arrivals beyond its blocks and give up after `polls`
+extern "C" void hx_barrier(hgks_mesh h, unsigned extra, unsigned polls) {
+  mesh_of(h)->s.grid_extra = extra;
+  mesh_of(h)->s.grid_polls = polls;
+}
+
+// the record of a grid barrier that gave up
+extern "C" int hx_set_stuck(hgks_mesh h) {
+  const int64_t one = 1;
+  return cudaMemcpy(mesh_of(h)->s.hs + kHsStuck, &one, sizeof(one), cudaMemcpyHostToDevice) != cudaSuccess;
+}
