@@ -785,7 +785,12 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   cudaDeviceGetAttribute(&shm_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (!coop || sms < 1) return false;
-  const int blocks = std::min({sms, kPG, (m.N + 7) / 8}), C = (m.N + blocks - 1) / blocks;
+  // Four lanes a cell and one warp per SM sub-partition are 32 cells a block; a small mesh fills its
+  // SMs that far before it takes another, since a block holds its SM for the whole solve and other
+  // streams' meshes wait for a free one. Steps of 1,296 cells, one stream / eight: 845 / 697 us with
+  // eight cells a block, 854 / 235 with 32 (separate launches 2,352 / 641); 3,072 cells 877 / 737
+  // and 882 / 647 (2,457 / 741).
+  const int blocks = std::min({sms, kPG, (m.N + 31) / 32}), C = (m.N + blocks - 1) / blocks;
   const int lpc = C <= 32 ? 4 : C <= 64 ? 2 : 1;        // one warp per SM sub-partition at most
   const bool one = C <= kPT;
   const size_t shm = sizeof(GridShared) + (one ? 0 : sizeof(double) * 5 * C);

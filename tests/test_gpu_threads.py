@@ -8,6 +8,7 @@ import os
 import subprocess
 import sys
 import threading
+import time
 
 import pytest
 
@@ -144,3 +145,29 @@ def test_meshes_of_different_sizes(cuda):
     together([lambda k=k: job(k) for k in range(2)])
     for k in range(2):
         assert torch.equal(got[k], alone[k]), (got[k] != alone[k]).nonzero().flatten().tolist()[:10]
+
+
+def test_small_meshes_on_their_own_streams_overlap(cuda):
+    """A one-launch GMRES takes 41 SMs for 1,296 cells, so three of them run side by side: eight
+    threads' steps must end in less than 0.6 of the time that they take one after the other."""
+    import torch
+    m, cond = I.cavity_mesh(6), I.cavity_conditions(0.15, 100.0)
+    p = H.hgks_default_params(scheme=0, Pr=0.72, **cond)
+    handles = [H.hgks_mesh_create(m, scheme_mask=1) for _ in range(8)]
+    Q0 = handles[0].to_internal(I.smooth_state(m, amp=0.02, base=(1.0, 0.05, 0.03, -0.02, cond["p_inf"]))[0])
+    states, streams = [Q0.clone() for _ in handles], [torch.cuda.Stream() for _ in handles]
+    torch.cuda.synchronize()
+
+    def job(k, steps):
+        with torch.cuda.stream(streams[k]):
+            for _ in range(steps):
+                H.hgks_gmres_step(handles[k], p, states[k])
+    together([lambda k=k: job(k, 3) for k in range(8)])
+    t0 = time.perf_counter()
+    for k in range(8):
+        job(k, 40)
+    t1 = time.perf_counter()
+    together([lambda k=k: job(k, 40) for k in range(8)])
+    t2 = time.perf_counter()
+    assert all(torch.equal(s, states[0]) for s in states)
+    assert t2 - t1 < 0.6 * (t1 - t0), (t1 - t0, t2 - t1)
