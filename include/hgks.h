@@ -392,8 +392,8 @@ hgks_status hgks_batch_solve_steady(hgks_batch batch, double drop_tol, int32_t m
                                     double *hist_host, hgks_solve_info *info, void *cuda_stream);
 
 /* Time the reconstruction and flux kernels of this batch's current state at
- * block sizes 64, 128 and 256 (CUDA events, 3 runs each) and keep the fastest
- * for later calls; the chosen sizes are returned (may be NULL). */
+ * block sizes 64, 128 and 256 (the reconstruction on hexahedra: 64 and 128;
+ * CUDA events, 3 runs each) and keep the fastest for later calls; the chosen sizes are returned (may be NULL). */
 hgks_status hgks_batch_autotune(hgks_batch batch, int32_t *blk_recon, int32_t *blk_flux, void *cuda_stream);
 
 /* ---------------------------------------------------------------------------

@@ -803,6 +803,7 @@ hgks_status hgks_batch_autotune(hgks_batch batch, int32_t *blk_recon, int32_t *b
     int best = *blk;
     float best_ms = 1e30f, ms = 0.f;
     for (int c : cand) {
+      if (pass == 0 && c > recon_block_max(B.m.d)) continue;
       *blk = c;
       if ((st = time_residual(ms))) break;
       if (ms < best_ms) { best_ms = ms; best = c; }

@@ -215,6 +215,7 @@ void launch_local_dt(const DevMesh &m, const hgks_params &p, const double *Q, do
 // fresh_dt = false keeps s.dt (the residual then uses the step's time step)
 void launch_residual(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *G,
                      double *R, double *Gnew, cudaStream_t st, bool batch = false, bool fresh_dt = true);
+int recon_block_max(const DevMesh &m);   // threads of k_recon's block at most (Scratch::blk_recon is cut to it)
 void launch_assemble(const DevMesh &m, Scratch &s, const hgks_params &p, const double *Q, const double *dt,
                      double *diag_out, double *off_out, cudaStream_t st, bool batch = false);
 void launch_precondition(const DevMesh &m, Scratch &s, int sweeps, const double *b, double *x, cudaStream_t st);

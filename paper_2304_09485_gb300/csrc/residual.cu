@@ -1026,6 +1026,8 @@ void launch_local_dt(const DevMesh &m, const hgks_params &hp, const double *Q, d
   HGKS_PROF_END(K_DT, st);
 }
 
+int recon_block_max(const DevMesh &m) { return m.hex ? kReconHex : kReconMax; }
+
 namespace {
 // Raises a kernel's dynamic shared memory to that of its largest block. The limit is the kernel's,
 // for all threads of the process: a value of the caller's own block shape would refuse the launch
@@ -1046,7 +1048,7 @@ void residual_kernels(const DevMesh &m, Scratch &s, const hgks_params &hp, const
   else k_coef_hweno<BATCH, S><<<gc, kBlock, 0, st>>>(m, Q, G, s.coef);
   HGKS_PROF_END(K_COEF, st);
   HGKS_PROF_BEGIN(K_RECON, st);
-  constexpr int rmax = S::NF == 4 ? kReconMax : kReconHex;
+  const int rmax = recon_block_max(m);
   const int br = std::min(s.blk_recon, rmax);
   const bool weno = p.scheme == HGKS_WENO;
   const size_t row = sizeof(double) * recon_rows(weno ? S::NSUBW : S::NF);
