@@ -228,7 +228,7 @@ std::vector<ProfRec> g_prof_recs;
 std::vector<cudaEvent_t> g_prof_pool;
 int g_prof_open = -1;
 const char *kKernelNames[K_COUNT] = {"local_dt", "coef", "recon", "flux", "gather", "assemble", "spmv", "jacobi",
-                                     "diag_scale", "axpy_dot", "scale", "givens", "combine", "update", "density_l1"};
+                                     "diag_scale", "axpy_dot", "scale", "givens", "combine", "update", "density_l1", "gmres"};
 cudaEvent_t prof_event() {
   if (!g_prof_pool.empty()) { cudaEvent_t e = g_prof_pool.back(); g_prof_pool.pop_back(); return e; }
   cudaEvent_t e;

@@ -810,9 +810,9 @@ bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double
               s.hs + (p.krylov_dim + 1) * p.krylov_dim + 1 + p.krylov_dim, s.vstride, s.red_count + 2, reinterpret_cast<int *>(s.hs + kHsStuck),
               blocks + s.grid_extra, s.grid_polls, p.krylov_dim, p.restarts, p.jacobi_sweeps};
   void *args[] = {&a};
-  HGKS_PROF_BEGIN(K_JACOBI, st);
+  HGKS_PROF_BEGIN(K_GMRES, st);
   cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kPT + 32), args, shm, st);
-  HGKS_PROF_END(K_JACOBI, st);
+  HGKS_PROF_END(K_GMRES, st);
   return true;
 }
 

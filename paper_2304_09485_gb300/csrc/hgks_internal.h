@@ -311,7 +311,7 @@ inline void count_launch() { ++g_launches; }
 // Optional per-kernel timing with CUDA events on the launching stream
 // (hgks_profile_begin / hgks_profile_end). Off by default: one branch per launch.
 enum KernelId { K_DT, K_COEF, K_RECON, K_FLUX, K_GATHER, K_ASSEMBLE, K_SPMV, K_JACOBI, K_DIAG, K_DOT, K_SCALE,
-                K_GIVENS, K_COMBINE, K_UPDATE, K_NORM, K_COUNT };
+                K_GIVENS, K_COMBINE, K_UPDATE, K_NORM, K_GMRES, K_COUNT };
 extern bool g_prof_on;
 void prof_mark(int kid, cudaStream_t st, bool begin);
 #define HGKS_PROF_BEGIN(kid, st) do { if (hgks::g_prof_on) hgks::prof_mark((kid), (st), true); } while (0)
