@@ -288,10 +288,6 @@ constexpr int kPT = 384;        // threads with cells, three warps per SM sub-pa
 constexpr int kPB = 8;          // basis vectors of a block (one grid barrier each)
 constexpr int kPG = 160;        // blocks at most (the sums read one partial per block)
 constexpr int kPMax = 64;       // Krylov vectors at most
-// Cells at most. Whole steps, one launch against separate ones: 343,332 tetrahedra 23.7 / 25.3 ms,
-// 576,000 39.0 / 39.9; beyond 700,000 w no longer fits shared memory, and with w in global memory
-// 766,656 take 53.3 / 52.3, 2,359,296 159 / 153.
-constexpr int kGridCells = 600000;
 
 struct GridSolve {
   int N, C;                     // cells, cells per block
@@ -780,7 +776,7 @@ const void *grid_kernel(int lpc, bool one) {
 // that fails all the same is an error like any other launch's.
 bool gmres_grid(const DevMesh &m, Scratch &s, const hgks_params &p, const double *rhs, double *dx, cudaStream_t st) {
   int dev = 0, sms = 0, coop = 0, shm_max = 0;
-  if (m.N > kGridCells || p.restarts < 1 || p.krylov_dim > kPMax || cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (m.N > s.grid_cells || p.restarts < 1 || p.krylov_dim > kPMax || cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   cudaDeviceGetAttribute(&shm_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

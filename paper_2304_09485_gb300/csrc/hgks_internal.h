@@ -129,6 +129,11 @@ struct BatchState {
   int a_off = 0, g_off = 0, gram_off = 0;   // offsets of a, g and the basis Gram matrix (leading dimension m + 1)
 };
 
+// Largest mesh of the one-launch FP64 GMRES (gmres64.cu). Whole steps, one launch against separate
+// ones: 343,332 tetrahedra 23.7 / 25.3 ms, 576,000 39.0 / 39.9; beyond 700,000 w no longer fits shared
+// memory, and with w in global memory 766,656 take 53.3 / 52.3, 2,359,296 159 / 153.
+constexpr int kGridCells = 600000;
+
 struct Scratch {
   double *coef = nullptr;        // [COEF][N] (105 tetrahedra, 165 hexahedra)
   double *dt = nullptr;          // [N]
@@ -159,8 +164,9 @@ struct Scratch {
   double *hostbuf = nullptr;     // [40][N] device state of the *_host entry points
   double *Qp = nullptr, *Rp = nullptr;   // [5][N] perturbed state and its residual (matrix-free products)
   int kdim = 0;
-  // the wait of the one-launch GMRES (gmres64.cu): polls before it gives up (a second or more), and
-  // arrivals expected beyond the launch's own blocks (none; set by the test of a wait that runs out)
+  // the one-launch GMRES: its largest mesh, and the wait at its barriers: polls before it gives up
+  // (a second or more), and arrivals expected beyond the launch's own blocks (none; more keep it shut)
+  int grid_cells = kGridCells;
   unsigned grid_polls = 1u << 22, grid_extra = 0;
   size_t bytes = 0;
   int blk_recon = 128, blk_flux = 128;   // launch shapes of the two FP64-bound kernels (autotuned for batches)

@@ -21,7 +21,9 @@ def load(directory):
         getattr(L, f).argtypes = [C.c_void_p, C.c_int]
     L.hx_batch_shape.argtypes = [C.c_void_p, C.c_int, C.c_int]
     L.hx_barrier.argtypes = [C.c_void_p, C.c_uint, C.c_uint]
-    L.hx_set_stuck.argtypes = [C.c_void_p]
+    L.hx_grid_cells.argtypes = [C.c_void_p, C.c_int]
+    for f in ("hx_set_stuck", "hx_captured"):
+        getattr(L, f).argtypes = [C.c_void_p]
     return L
 
 

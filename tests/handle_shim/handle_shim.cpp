@@ -39,3 +39,12 @@ extern "C" int hx_set_stuck(hgks_mesh h) {
   const int64_t one = 1;
   return cudaMemcpy(mesh_of(h)->s.hs + kHsStuck, &one, sizeof(one), cudaMemcpyHostToDevice) != cudaSuccess;
 }
+
+// the largest mesh of the one-launch FP64 GMRES: 0 for separate launches
+extern "C" void hx_grid_cells(hgks_mesh h, int cells) { mesh_of(h)->s.grid_cells = cells; }
+
+// whether the mesh keeps a captured step
+extern "C" int hx_captured(hgks_mesh h) {
+  const StepGraph *g = mesh_of(h)->graph;
+  return g && g->exec;
+}
