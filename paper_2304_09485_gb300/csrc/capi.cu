@@ -165,30 +165,33 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
   const bool arena = m.d.ptab != nullptr;
   const size_t rows = arena ? 25 * NF : 6 + 5 * NF;
   double *&blocks = arena ? s.off : s.jv64;
-  if (implicit && !blocks) {
-    if ((st = dalloc(m, &blocks, (rows + (arena ? 0 : 12)) * N))) return st;
-    if ((st = dalloc(m, &s.dval, N))) return st;
-    if ((st = dalloc(m, &s.dinv, N))) return st;
-    if ((st = dalloc(m, &s.R, 5 * N))) return st;
-    if ((st = dalloc(m, &s.Gnew, 15 * N))) return st;
-    if ((st = dalloc(m, &s.dQ, 5 * N))) return st;
-    if ((st = dalloc(m, &s.w, 5 * N))) return st;
-    if ((st = dalloc(m, &s.t, 5 * N))) return st;
-    if (arena && (st = dalloc(m, &s.t2, 5 * N))) return st;
-    if ((st = dalloc(m, &s.hs, 65 * 64 + 256))) return st;
-    if ((st = dalloc(m, &s.gram, 65 * 65 + 2 * 65 + 64))) return st;
+  // a group is complete when its last array is there; after a failed allocation the next call takes up
+  // what is missing
+  auto need = [&](auto **p, size_t n) { return *p ? HGKS_OK : dalloc(m, p, n); };
+  if (implicit && !s.gram) {
+    if ((st = need(&blocks, (rows + (arena ? 0 : 12)) * N))) return st;
+    if ((st = need(&s.dval, N))) return st;
+    if ((st = need(&s.dinv, N))) return st;
+    if ((st = need(&s.R, 5 * N))) return st;
+    if ((st = need(&s.Gnew, 15 * N))) return st;
+    if ((st = need(&s.dQ, 5 * N))) return st;
+    if ((st = need(&s.w, 5 * N))) return st;
+    if ((st = need(&s.t, 5 * N))) return st;
+    if (arena && (st = need(&s.t2, 5 * N))) return st;
+    if ((st = need(&s.hs, 65 * 64 + 256))) return st;
     for (int k = 0; k < 2 && !arena; k++) s.z[k] = blocks + (rows + 6 * k) * N;
     HGKS_CUDA(cudaMemset(blocks, 0, sizeof(double) * rows * N));
     HGKS_CUDA(cudaMemset(s.hs + kHsStuck, 0, sizeof(double)));
+    if ((st = need(&s.gram, 65 * 65 + 2 * 65 + 64))) return st;
   }
-  if (implicit && mixed && !s.jv32) {
-    if ((st = dalloc(m, &s.jv32, (6 + 4 * NF) * N))) return st;
-    if ((st = dalloc(m, &s.dval32, N))) return st;
-    if ((st = dalloc(m, &s.dinv32, N))) return st;
-    if ((st = dalloc(m, &s.w32, 5 * N))) return st;
-    if ((st = dalloc(m, &s.t32, 5 * N))) return st;
-    if ((st = dalloc(m, &s.t232, 5 * N))) return st;
-    if ((st = dalloc(m, &s.red32, std::max<size_t>(16 * 608 + 64, N / 64 + 64)))) return st;
+  if (implicit && mixed && !s.red32) {
+    if ((st = need(&s.jv32, (6 + 4 * NF) * N))) return st;
+    if ((st = need(&s.dval32, N))) return st;
+    if ((st = need(&s.dinv32, N))) return st;
+    if ((st = need(&s.w32, 5 * N))) return st;
+    if ((st = need(&s.t32, 5 * N))) return st;
+    if ((st = need(&s.t232, 5 * N))) return st;
+    if ((st = need(&s.red32, std::max<size_t>(16 * 608 + 64, N / 64 + 64)))) return st;
   }
   auto release = [&](void *p, size_t bytes) {
     cudaFree(p);
@@ -215,7 +218,8 @@ hgks_status ensure_scratch(Mesh &m, int kdim, bool implicit, bool mixed) {
 // the perturbed state and its residual of the matrix-free products (jv_mode 1)
 static hgks_status ensure_fd(Mesh &m) {
   hgks_status st;
-  if (!m.s.Qp && ((st = dalloc(m, &m.s.Qp, 5 * (size_t)m.N)) || (st = dalloc(m, &m.s.Rp, 5 * (size_t)m.N)))) return st;
+  if (!m.s.Qp && (st = dalloc(m, &m.s.Qp, 5 * (size_t)m.N))) return st;
+  if (!m.s.Rp && (st = dalloc(m, &m.s.Rp, 5 * (size_t)m.N))) return st;
   return HGKS_OK;
 }
 
@@ -440,7 +444,7 @@ hgks_status hgks_assemble(hgks_mesh mesh, const hgks_params *p, const double *Q,
 hgks_status hgks_apply_jacobian(hgks_mesh mesh, const double *x, double *y, void *cuda_stream) {
   if (!mesh || !x || !y) return fail(HGKS_ERR_ARG, "NULL argument");
   Mesh &m = mesh->m;
-  if (!m.s.jv64) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
+  if (!m.s.gram) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
   HGKS_ON_DEVICE(m.device);
   launch_apply_A(m.d, m.s, nullptr, x, y, (cudaStream_t)cuda_stream);
   return last_launch();
@@ -490,7 +494,7 @@ hgks_status hgks_precondition(hgks_mesh mesh, int32_t sweeps, const double *b, d
   if (b == x) return fail(HGKS_ERR_ARG, "b and x must not alias");
   if (sweeps < 0) return fail(HGKS_ERR_ARG, "negative sweeps");
   Mesh &m = mesh->m;
-  if (!m.s.jv64) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
+  if (!m.s.gram) return fail(HGKS_ERR_ARG, "hgks_assemble has not been called");
   HGKS_ON_DEVICE(m.device);
   launch_precondition(m.d, m.s, sweeps, b, x, (cudaStream_t)cuda_stream);
   return last_launch();
