@@ -45,7 +45,8 @@ FP64_NOMINAL_GFLOPS = 1258.6
 # 648,000-tet sphere (non-compact scheme, inviscid, Pr = 1). DRAM bytes per unit
 # of work from the same capture (dram__bytes_read.sum + dram__bytes_write.sum
 # divided by the units of the launch); the traffic of a full launch is this times
-# its units.
+# its units. Fractions made with the flops of earlier kernels (an addition as one)
+# do not compare with these.
 KERNEL_TRAFFIC = {"flux": 397.3, "recon": 925.6, "jacobi": 320.0, "spmv": 455.0}
 KERNEL_FLOPS = {
     "flux": (2 * 732.0, lambda N, F: 3 * F),     # per face Gauss point
@@ -54,7 +55,8 @@ KERNEL_FLOPS = {
     # (81.75 instructions, 120 of a C2 step's 126 launches) and the sweeps of the
     # restart vector; "spmv" = the final v + E z products with the fused inner
     # products (84.0 with two of them, five more for each of up to four; 60 of 62):
-    # launch-weighted means
+    # launch-weighted means. Meshes up to 600,000 cells solve in one launch, "gmres",
+    # which has no entry here
     "jacobi": (2 * 82.0, lambda N, F: N),
     "spmv": (2 * 91.9, lambda N, F: N),
 }

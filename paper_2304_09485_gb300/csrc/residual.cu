@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kBlock) k_coef_hweno(DevMesh m, const double *
 // Registers to match: 168 for 12 warps an SM, 255 for 8 (hexahedra with 168 spilled 348 bytes a
 // thread: 0.843 -> 0.825 ms for 35,937, 4.07 -> 4.00 for 190,464).
 // Against dense rows per variable: 28.5 -> 22.8 ms for 9.4M (cell, face) pairs (2,359,296
-// tetrahedra), 1.24 -> 0.83 ms for 35,937 hexahedra. ncu at 648,000 tetrahedra: 1,466 FP64 instructions a
+// tetrahedra), 1.24 -> 0.83 ms for 35,937 hexahedra (0.72 with the compact scheme's six). ncu at 648,000 tetrahedra: 1,466 FP64 instructions a
 // thread, the pipe 97 % busy.
 // NSUB: the scheme's sub-polynomials, one per sub-stencil or (compact) per face: on hexahedra k_coef
 // writes six vectors of three for the compact scheme and eight for the other, and no more are read.
